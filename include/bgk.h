@@ -351,7 +351,7 @@ BGK_API bgk_status bgk_stage(bgk_ctx *ctx, const void *f_n, const void *f_in, vo
 /* Raw velocity moments of the stored state (section "Governing equations":
  * the moments that give Q = (rho, rho U, E)), m[P][11]: sum w F, sum w u_d F
  * (3), sum w u_d^2 F (3), sum w u1u2 F, sum w u1u3 F, sum w u2u3 F, sum w G,
- * summed in FP64.  m is host (on_device = 0) or device memory (1).
+ * summed to FP64 accuracy.  m is host (on_device = 0) or device memory (1).
  * Errors: BGK_EINVAL (NULL), BGK_ECUDA. */
 BGK_API bgk_status bgk_moments(bgk_ctx *ctx, double *m, int on_device);
 
@@ -457,7 +457,7 @@ BGK_API bgk_status bgk_shard_stage(bgk_ctx *ctx, const double *m, int stage, dou
  * quantities of section "Governing equations".  totals is host memory.
  * entropy (host memory, may be NULL): the discrete entropy
  * H = sum_e sum_s W_s J_s sum_k w_k F ln F of the stored F component with the
- * same quadrature, summed in FP64 (section "Numerical method": the
+ * same quadrature, to FP64 accuracy (section "Numerical method": the
  * discrete-velocity BGK relaxation does not increase it).  It is NaN when
  * some stored F is not positive.  With delta > 0 it covers F only (the paper
  * states no entropy functional for the reduced F, G pair).

@@ -255,20 +255,17 @@ bgk_status check_device_status(bgk_ctx *ctx) {
     return BGK_OK;
 }
 
-// Moment partials of a state.  The FP32 state's stepping path (resum =
-// false) uses the stage epilogue's error-free FP32 accumulation; the
-// diagnostic entry points (resum = true) re-sum in FP64, independently of it.
-bgk_status run_moments(bgk_ctx *ctx, const void *f, bool resum = false) {
+// Moment partials of a state.  The FP32 state's stepping path (check = false)
+// uses the stage epilogue's error-free FP32 accumulation; the diagnostic entry
+// points (check = true) fold its line sums in FP64.
+bgk_status run_moments(bgk_ctx *ctx, const void *f, bool check = false) {
     LaunchScope ls(ctx, BGK_K_MOMENTS);
     if (ctx->precision == BGK_FP64) {
-        MomentArgs64 a{(const double *)f, ctx->part, ctx->vtab, ctx->Nu, ctx->P, ctx->Kblk, ctx->C};
-        CU(launch_moments_f64(a, ctx->n_vblk, ctx->stream));
-    } else if (resum) {
-        CU(launch_moments_f32((const float *)f, ctx->part, ctx->vtab, ctx->Nu, ctx->P, ctx->Kblk,
-                              ctx->C, ctx->n_vblk, ctx->stream));
+        MomentArgs64 a{(const double *)f, ctx->part, ctx->Nu, ctx->P, ctx->Kblk, ctx->C};
+        CU(launch_moments_f64(a, ctx->vg, ctx->n_vblk, ctx->stream));
     } else {
-        CU(launch_moments_f32_exact((const float *)f, ctx->part, ctx->vg, ctx->Nu, ctx->P, ctx->Kblk, ctx->C,
-                                    ctx->n_vblk, ctx->stream));
+        CU(launch_moments_f32((const float *)f, ctx->part, ctx->vtab, ctx->vg, ctx->Nu, ctx->P, ctx->Kblk, ctx->C,
+                              ctx->n_vblk, check, ctx->stream));
     }
     return BGK_OK;
 }
@@ -1530,50 +1527,46 @@ bgk_status bgk_qprime(bgk_ctx *ctx, const double *m, int n_points, double *qp, i
 
 bgk_status bgk_totals(bgk_ctx *ctx, double totals[5], double *entropy) {
     if (!ctx || !totals) return BGK_EINVAL;
-    std::vector<double> m((size_t)ctx->P * BGK_NMOM);
-    bgk_status st = bgk_moments(ctx, m.data(), 0);
-    if (st) return st;
-    std::vector<double> hp;
+    bgk_status st;
+    if (!ctx->part_valid) {
+        if ((st = run_moments(ctx, ctx->f[0], true))) return st;
+        ctx->part_valid = true;
+    }
+    // scratch: the totals and the block sums, then (with entropy) the count of
+    // non-positive values and the per-point partials of each velocity block
+    const size_t n_tot = totals_scratch(), n_ent = entropy ? 1 + (size_t)ctx->n_vblk * ctx->P : 0;
+    double *w = nullptr;
+    CU(cudaMallocAsync((void **)&w, (n_tot + n_ent) * sizeof(double), ctx->stream));
+    double *ent = entropy ? w + n_tot + 1 : nullptr;
+    unsigned int *bad = reinterpret_cast<unsigned int *>(w + n_tot);
+    cudaError_t e = cudaSuccess;
+    {
+        LaunchScope ls(ctx, BGK_K_OTHER);
+        e = launch_reduce_moments(ctx->part, ctx->n_vblk, ctx->P, ctx->mom, ctx->stream);
+    }
+    if (entropy && e == cudaSuccess) {
+        LaunchScope ls(ctx, BGK_K_OTHER);
+        e = cudaMemsetAsync(bad, 0, sizeof(unsigned int), ctx->stream);
+        if (e == cudaSuccess)
+            e = ctx->precision == BGK_FP64
+                    ? launch_entropy_f64((const double *)ctx->f[0], ctx->vg, ctx->Nu, ctx->P, ctx->Kblk, ctx->n_vblk, ent,
+                                         bad, ctx->stream)
+                    : launch_entropy_f32((const float *)ctx->f[0], ctx->vg, ctx->Nu, ctx->P, ctx->Kblk, ctx->n_vblk, ent,
+                                         bad, ctx->stream);
+    }
+    if (e == cudaSuccess)
+        e = launch_totals(ctx->mom, ent, ctx->n_vblk, ctx->P, ctx->fr, ctx->jac, ctx->curved ? ctx->geo : nullptr, w,
+                          ctx->stream);
+    double t[6];
     unsigned int nonpos = 0;
-    if (entropy) {
-        // per-point sum_k w_k F ln F in FP64 (a velocity-block partial, then
-        // the sum over blocks), weighed below with the totals' quadrature
-        double *dpart = nullptr, *dh = nullptr;
-        unsigned int *dbad = nullptr;
-        CU(cudaMallocAsync((void **)&dpart, (size_t)ctx->n_vblk * ctx->P * sizeof(double), ctx->stream));
-        CU(cudaMallocAsync((void **)&dh, (size_t)ctx->P * sizeof(double), ctx->stream));
-        CU(cudaMallocAsync((void **)&dbad, sizeof(unsigned int), ctx->stream));
-        CU(cudaMemsetAsync(dbad, 0, sizeof(unsigned int), ctx->stream));
-        {
-            LaunchScope ls(ctx, BGK_K_OTHER);
-            if (ctx->precision == BGK_FP64)
-                CU(launch_entropy<double>((const double *)ctx->f[0], ctx->vtab, ctx->Nu, ctx->P, ctx->Kblk,
-                                          ctx->n_vblk, dpart, dh, dbad, ctx->stream));
-            else
-                CU(launch_entropy<float>((const float *)ctx->f[0], ctx->vtab, ctx->Nu, ctx->P, ctx->Kblk,
-                                         ctx->n_vblk, dpart, dh, dbad, ctx->stream));
-        }
-        hp.resize(ctx->P);
-        CU(cudaMemcpyAsync(hp.data(), dh, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-        CU(cudaMemcpyAsync(&nonpos, dbad, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->stream));
-        CU(cudaFreeAsync(dpart, ctx->stream));
-        CU(cudaFreeAsync(dh, ctx->stream));
-        CU(cudaFreeAsync(dbad, ctx->stream));
-        CU(cudaStreamSynchronize(ctx->stream));
-    }
-    const int q = ctx->q;
-    double t[5] = {0, 0, 0, 0, 0}, H = 0.0;
-    for (int p = 0; p < ctx->P; ++p) {
-        const int s = p % ctx->Ns;
-        const double W = ctx->curved ? ctx->geo_h[(size_t)p * BGK_NGEO + 10]
-                                     : ctx->fr.wq[s % q] * ctx->fr.wq[(s / q) % q] * ctx->fr.wq[s / (q * q)] * ctx->jac;
-        const double *mm = &m[(size_t)p * BGK_NMOM];
-        t[0] += W * mm[0]; t[1] += W * mm[1]; t[2] += W * mm[2]; t[3] += W * mm[3];
-        t[4] += W * (0.5 * (mm[4] + mm[5] + mm[6]) + mm[10]);
-        if (entropy) H += W * hp[p];
-    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(t, w, sizeof t, cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess && entropy) e = cudaMemcpyAsync(&nonpos, bad, sizeof nonpos, cudaMemcpyDeviceToHost, ctx->stream);
+    const cudaError_t ef = cudaFreeAsync(w, ctx->stream), es = cudaStreamSynchronize(ctx->stream);
+    CU(e);
+    CU(ef);
+    CU(es);
     for (int j = 0; j < 5; ++j) totals[j] = t[j];
-    if (entropy) *entropy = nonpos ? std::numeric_limits<double>::quiet_NaN() : H;
+    if (entropy) *entropy = nonpos ? std::numeric_limits<double>::quiet_NaN() : t[5];
     return BGK_OK;
 }
 

@@ -251,7 +251,6 @@ struct QPrimeArgs {
 struct MomentArgs64 {
     const double *f;
     double *part;
-    const double *vtab;
     int Nu, P, Kblk, C;
 };
 
@@ -273,19 +272,14 @@ cudaError_t launch_wall_density(const T *f, const T *fvec, const double *bcval, 
                                 double *rho_w, cudaStream_t s);
 
 // Launchers: the Q' solve and its tensor refinement (kernels_qprime.cu); the
-// FP64 moments, stage and Maxwellian (kernels_f64.cu); the FP32 moments and
-// stage (kernels_f32.cu, the line kernels in kernels_f32_line.cu).
-cudaError_t launch_moments_f64(const MomentArgs64 &a, int n_vblk, cudaStream_t s);
+// FP64 stage and Maxwellian (kernels_f64.cu); the FP32 stage and Maxwellian
+// (kernels_f32.cu, the line kernels in kernels_f32_line.cu).
 cudaError_t launch_qprime(const QPrimeArgs &a, bool fp32_sums, cudaStream_t s);
 // tensor variant of the ES equilibrium: refines the eq record k_qprime wrote
 cudaError_t launch_qprime_tensor(const QPrimeArgs &a, bool fp32_sums, cudaStream_t s);
 cudaError_t launch_stage_f64(const StageArgs<double> &a, int C, int n_vblk, cudaStream_t s);
 cudaError_t launch_maxwellian_f64(double *f, const double *q, const double *vtab, int Nu, int P,
                                   int C, double delta, cudaStream_t s);
-cudaError_t launch_moments_f32(const float *f, double *part, const double *vtab, int Nu, int P,
-                               int Kblk, int C, int n_vblk, cudaStream_t s);
-cudaError_t launch_moments_f32_exact(const float *f, double *part, const VelGrid &vg, int Nu, int P, int Kblk,
-                                     int C, int n_vblk, cudaStream_t s);
 cudaError_t launch_stage_f32(const StageArgs<float> &a, int C, int n_vblk, int variant, int depth,
                              cudaStream_t s);
 bool stage_f32_tma_supported(const StageArgs<float> &a, int C, int depth);
@@ -298,13 +292,25 @@ cudaError_t launch_maxwellian_f32(float *f, const double *q, const double *vtab,
                                   double delta, cudaStream_t s);
 cudaError_t launch_macro(const double *mom, double *out, int P, const MeshInfo &mesh, const FROps &fr,
                          const GasInfo &gas, const double face_rho[6], const double *geo, cudaStream_t s);
-// per-point entropy sum_k w_k F ln F of the F component (kernels_f64.cu);
-// part holds n_vblk * P doubles, *nonpos counts the non-positive values
-template <typename T>
-cudaError_t launch_entropy(const T *f, const double *vtab, int Nu, int P, int Kblk, int n_vblk, double *part,
-                           double *h_out, unsigned int *nonpos, cudaStream_t s);
-// out[j][p] = sum over velocity blocks of part[vb][j][p] (kernels_f64.cu):
-// a shard's partial raw moments in the layout the Q' solve reads (one block)
+// Moments, entropy and totals of a stored state (moments.cu).  check (the
+// diagnostic entry points): the FP32 state's lines fold in FP64, and a point
+// whose sums are not finite is summed again in FP64 throughout.
+cudaError_t launch_moments_f64(const MomentArgs64 &a, const VelGrid &vg, int n_vblk, cudaStream_t s);
+cudaError_t launch_moments_f32(const float *f, double *part, const double *vtab, const VelGrid &vg, int Nu, int P,
+                               int Kblk, int C, int n_vblk, bool check, cudaStream_t s);
+// out[j][p] = sum over velocity blocks of part[vb][j][p]: a shard's partial raw
+// moments in the layout the Q' solve reads (one block)
 cudaError_t launch_sum_partials(const double *part, int n_vblk, int P, double *out, cudaStream_t s);
 cudaError_t launch_reduce_moments(const double *part, int n_vblk, int P, double *m_out,
                                   cudaStream_t s);
+// per-point entropy partials part[n_vblk][P] of the F component; *nonpos counts
+// the values that are not positive
+cudaError_t launch_entropy_f32(const float *f, const VelGrid &vg, int Nu, int P, int Kblk, int n_vblk, double *part,
+                               unsigned int *nonpos, cudaStream_t s);
+cudaError_t launch_entropy_f64(const double *f, const VelGrid &vg, int Nu, int P, int Kblk, int n_vblk, double *part,
+                               unsigned int *nonpos, cudaStream_t s);
+// scratch[0..5] = domain totals (5) and entropy from mom[P][11] and ent[n_vblk][P]
+// (may be null); scratch holds totals_scratch() doubles
+size_t totals_scratch();
+cudaError_t launch_totals(const double *mom, const double *ent, int n_vblk, int P, const FROps &fr, double jac,
+                          const double *geo, double *scratch, cudaStream_t s);

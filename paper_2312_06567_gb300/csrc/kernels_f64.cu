@@ -1,8 +1,7 @@
 // FP64 kernels of one explicit Runge--Kutta stage of the Boltzmann--ES-BGK
 // residual (Dzanic & Martinelli, arXiv 2312.06567, section "Methodology").
 //
-//   moments   raw velocity moments of f, partial over velocity blocks
-//   (the Q' solve is in kernels_qprime.cu)
+//   (moments of a stored state: moments.cu; the Q' solve: kernels_qprime.cu)
 //   stage     FR divergence (nodal derivative + upwind interface jump lifted
 //             with the DG correction function) + BGK source + Shu--Osher
 //             combination, with the moment partials of the output in the
@@ -14,89 +13,6 @@
 namespace {
 
 constexpr double kTwoPi = 6.283185307179586476925286766559;
-
-// ---------------------------------------------------------------------------
-// Raw moments (section "Governing equations": Q = int psi f, Pi = int f c c):
-// slots 0: w F, 1..3: w u_d F, 4..6: w u_d^2 F, 7: w u1u2 F, 8: w u1u3 F,
-// 9: w u2u3 F, 10: w G.  One thread per point, one velocity block per blockIdx.y.
-__global__ void __launch_bounds__(256) k_moments_f64(MomentArgs64 a) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= a.P) return;
-    const int vb = blockIdx.y;
-    const int k0 = vb * a.Kblk;
-    const int k1 = min(a.Nu, k0 + a.Kblk);
-    double m[BGK_NMOM];
-#pragma unroll
-    for (int j = 0; j < BGK_NMOM; ++j) m[j] = 0.0;
-    for (int k = k0; k < k1; ++k) {
-        const double *v = a.vtab + (size_t)k * BGK_VTAB;
-        const double u1 = __ldg(v + 0), u2 = __ldg(v + 1), u3 = __ldg(v + 2), w = __ldg(v + 3);
-        const double wF = w * __ldg(a.f + (size_t)k * a.P + p);
-        m[0] += wF;
-        m[1] = fma(wF, u1, m[1]);
-        m[2] = fma(wF, u2, m[2]);
-        m[3] = fma(wF, u3, m[3]);
-        m[4] = fma(wF * u1, u1, m[4]);
-        m[5] = fma(wF * u2, u2, m[5]);
-        m[6] = fma(wF * u3, u3, m[6]);
-        m[7] = fma(wF * u1, u2, m[7]);
-        m[8] = fma(wF * u1, u3, m[8]);
-        m[9] = fma(wF * u2, u3, m[9]);
-        if (a.C == 2) m[10] = fma(w, __ldg(a.f + ((size_t)a.Nu + k) * a.P + p), m[10]);
-    }
-#pragma unroll
-    for (int j = 0; j < BGK_NMOM; ++j) a.part[((size_t)vb * BGK_NMOM + j) * a.P + p] = m[j];
-}
-
-// Discrete entropy of the F component, partial over velocity blocks
-// (section "Numerical method": the discrete-velocity BGK step obeys a
-// discrete H-theorem): part[vb][p] = sum_{k in block vb} w_k F ln F in FP64;
-// a non-positive F has no entropy and is counted in *nonpos instead.
-template <typename T>
-__global__ void __launch_bounds__(256) k_entropy_partial(const T *f, const double *vtab, int Nu, int P, int Kblk,
-                                                         double *part, unsigned int *nonpos) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    const int vb = blockIdx.y;
-    const int k0 = vb * Kblk, k1 = min(Nu, k0 + Kblk);
-    double h = 0.0;
-    unsigned int bad = 0;
-    for (int k = k0; k < k1; ++k) {
-        const double F = (double)f[(size_t)k * P + p];
-        if (F > 0.0) h = fma(__ldg(vtab + (size_t)k * BGK_VTAB + 3) * F, log(F), h);
-        else ++bad;
-    }
-    part[(size_t)vb * P + p] = h;
-    if (bad) atomicAdd(nonpos, bad);
-}
-
-__global__ void k_reduce_entropy(const double *part, int n_vblk, int P, double *h_out) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    double s = 0.0;
-    for (int vb = 0; vb < n_vblk; ++vb) s += part[(size_t)vb * P + p];
-    h_out[p] = s;
-}
-
-__global__ void k_sum_partials(const double *part, int n_vblk, int P, double *out) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    for (int j = 0; j < BGK_NMOM; ++j) {
-        double s = 0.0;
-        for (int vb = 0; vb < n_vblk; ++vb) s += part[((size_t)vb * BGK_NMOM + j) * P + p];
-        out[(size_t)j * P + p] = s;
-    }
-}
-
-__global__ void k_reduce_moments(const double *part, int n_vblk, int P, double *m_out) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    for (int j = 0; j < BGK_NMOM; ++j) {
-        double s = 0.0;
-        for (int vb = 0; vb < n_vblk; ++vb) s += part[((size_t)vb * BGK_NMOM + j) * P + p];
-        m_out[(size_t)p * BGK_NMOM + j] = s;
-    }
-}
 
 // ---------------------------------------------------------------------------
 // Fused stage.  Along each reference direction d the 1-D FR derivative at
@@ -397,38 +313,6 @@ __global__ void k_maxwellian_f64(double *f, const double *qin, const double *vta
 }
 
 }  // namespace
-
-cudaError_t launch_moments_f64(const MomentArgs64 &a, int n_vblk, cudaStream_t s) {
-    dim3 grid((a.P + 255) / 256, n_vblk);
-    k_moments_f64<<<grid, 256, 0, s>>>(a);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_entropy(const T *f, const double *vtab, int Nu, int P, int Kblk, int n_vblk, double *part,
-                           double *h_out, unsigned int *nonpos, cudaStream_t s) {
-    dim3 grid((P + 255) / 256, n_vblk);
-    k_entropy_partial<T><<<grid, 256, 0, s>>>(f, vtab, Nu, P, Kblk, part, nonpos);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_reduce_entropy<<<(P + 255) / 256, 256, 0, s>>>(part, n_vblk, P, h_out);
-    return cudaGetLastError();
-}
-template cudaError_t launch_entropy<double>(const double *, const double *, int, int, int, int, double *, double *,
-                                            unsigned int *, cudaStream_t);
-template cudaError_t launch_entropy<float>(const float *, const double *, int, int, int, int, double *, double *,
-                                           unsigned int *, cudaStream_t);
-
-cudaError_t launch_sum_partials(const double *part, int n_vblk, int P, double *out, cudaStream_t s) {
-    k_sum_partials<<<(P + 255) / 256, 256, 0, s>>>(part, n_vblk, P, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_reduce_moments(const double *part, int n_vblk, int P, double *m_out,
-                                  cudaStream_t s) {
-    k_reduce_moments<<<(P + 255) / 256, 256, 0, s>>>(part, n_vblk, P, m_out);
-    return cudaGetLastError();
-}
 
 template <int Q>
 static cudaError_t stage_q(const StageArgs<double> &a, int C, int n_vblk, cudaStream_t s) {

@@ -1,0 +1,681 @@
+// Moments, entropy and totals of a stored state (Dzanic & Martinelli, arXiv
+// 2312.06567, section "Governing equations": Q = int psi f, Pi = int f c c; the
+// discrete entropy of section "Numerical method").
+//
+// All of these read every value of the state once and do little with it, so
+// HBM bounds them once nothing else does.  What else there was: the FP64 pipe
+// (2 instructions per SM and clock: a direct sum of the raw moments costs 17
+// per value, a log() about 25), too few bytes in flight with one point per
+// thread, and scalar error-free sums.  Here:
+//   * raw moments are taken per first-axis velocity line: three (F) or four
+//     (F, G) sums over centred indices jt = j - jc, folded per line and plane;
+//   * the FP32 state's line sums are error-free FP32 pairs, two points per
+//     thread on packed instructions;
+//   * the entropy takes ln F from a table and a short series.
+// Times are on a GB300 for 16,384 points x 13,824 velocities (0.91 GB of FP32
+// state): the stepping path's moments 1.16 -> 0.40 ms, the diagnostics'
+// 7.18 -> 0.90, all of macro + moments + totals + entropy 22.6 -> 2.3.
+#include <algorithm>
+
+#include "stage_f32_common.cuh"
+
+namespace {
+
+constexpr int MT = 256;          // threads per block
+constexpr int MCH = 8;           // velocities loaded before they are used
+// ln2 = 45426 / 2^16 + LN2_MID + LN2_LO, the first two of at most 16 bits (an
+// integer of up to 8 bits times either is exact in FP32)
+constexpr double kLn2Rest = 0.69314718055994530942 - 45426.0 / 65536.0;
+constexpr float LN2_MID = (float)((double)(long long)(kLn2Rest * 34359738368.0) / 34359738368.0);     // 2^35
+constexpr float LN2_LO = (float)(kLn2Rest - (double)LN2_MID);
+
+// one plane quantity of two points: P += c * (s + e), error-free
+__device__ __forceinline__ void plane_add2(float2 &P, float2 &Pe, float c, float2 s, float2 e) {
+    const float2 c2 = dup2(c);
+    const float2 pr = __fmul2_rn(c2, s);
+    sum2x2(P, Pe, pr);
+    Pe = __fadd2_rn(Pe, __ffma2_rn(c2, s, neg2(pr)));
+    Pe = __ffma2_rn(c2, e, Pe);
+}
+
+// the plane's seven sums (00 10 20 01 11 02 G) of one point into its index
+// moments J in the partials buffer, weight c, centred third index t
+__device__ __forceinline__ void plane_to_part(double *J, int P, double c, double t, const double (&d)[7], bool first) {
+    double o[11];
+#pragma unroll
+    for (int i = 0; i < 11; ++i) o[i] = first ? 0.0 : J[(size_t)i * P];
+    o[0] = fma(c, d[0], o[0]); o[1] = fma(c, d[1], o[1]); o[2] = fma(c, d[2], o[2]);
+    o[3] = fma(c, d[3], o[3]); o[4] = fma(c, d[4], o[4]); o[5] = fma(c, d[5], o[5]);
+    o[6] = fma(c * t, d[0], o[6]); o[7] = fma(c * t, d[1], o[7]); o[8] = fma(c * t, d[3], o[8]);
+    o[9] = fma(c * t * t, d[0], o[9]); o[10] = fma(c, d[6], o[10]);
+#pragma unroll
+    for (int i = 0; i < 11; ++i) J[(size_t)i * P] = o[i];
+}
+// index moments -> raw moments where they stand
+__device__ __forceinline__ void raw_in_place(double *J, int P, const VelGrid &vg, const double uc[3]) {
+    double Jv[11], m[BGK_NMOM];
+#pragma unroll
+    for (int i = 0; i < 11; ++i) Jv[i] = J[(size_t)i * P];
+    index_to_raw(Jv, vg, uc, m);
+#pragma unroll
+    for (int i = 0; i < BGK_NMOM; ++i) J[(size_t)i * P] = m[i];
+}
+
+// Raw moments of an FP32 state on the stepping path: lines' and planes' sums
+// as FP32 pairs, the stage epilogue's operations in its velocity order, so the
+// partials equal what an epilogue yields for the same values.  A thread takes
+// the two points p and p + 256: one packed instruction serves both, loads stay
+// coalesced for every P, and 2 x 8 loads per thread are in flight.  The FP64
+// index moments of finished planes stay in the partials buffer, which the
+// thread owns for its points (a block of lines spans few planes), leaving the
+// registers to loads.  1.16 -> 0.40 ms for the state above (2.3 TB/s; latency
+// of the sum chains at 24 warps per SM); with two blocks per SM 0.45, with 4
+// velocities 0.43.
+template <int C>
+__global__ void __launch_bounds__(MT, 3) k_moments_f32(const float *f, double *part, VelGrid vg, int Nu, int P, int Kblk) {
+    constexpr int NL = C == 2 ? 4 : 3, NQ = C == 2 ? 7 : 6;
+    constexpr int MCH = C == 2 ? 4 : 8;                  // with G, eight would spill
+    const int pa = blockIdx.x * (2 * MT) + threadIdx.x, pb = pa + MT;
+    if (pa >= P) return;
+    const bool two = pb < P;
+    const float *fa = f + pa, *fb = f + (two ? pb : pa);
+    const int vb = blockIdx.y;
+    const int k0 = vb * Kblk, k1 = min(Nu, k0 + Kblk);
+    const int vn1 = vg.n[0], vn2 = vg.n[1];
+    const int jc[3] = {(vn1 - 1) / 2, (vn2 - 1) / 2, (vg.n[2] - 1) / 2};
+    const size_t GO = (size_t)Nu * P;                    // offset of the G component
+    double *Ja = part + (size_t)vb * BGK_NMOM * P + pa;
+    double *Jb = part + (size_t)vb * BGK_NMOM * P + (two ? pb : pa);
+    float2 Pl[NQ], Pe[NQ];
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) Pl[i] = Pe[i] = dup2(0.f);
+    bool first = true;
+    auto flush = [&](int j3) {
+        const double c = trap3(j3, vg), t = (float)(j3 - jc[2]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (h == 1 && !two) break;
+            double d[7];
+#pragma unroll
+            for (int i = 0; i < 7; ++i)
+                d[i] = i < NQ ? (double)(h ? Pl[i].y : Pl[i].x) + (double)(h ? Pe[i].y : Pe[i].x) : 0.0;
+            plane_to_part(h ? Jb : Ja, P, c, t, d, first);
+        }
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) Pl[i] = Pe[i] = dup2(0.f);
+        first = false;
+    };
+    int j3cur = (k0 / vn1) / vn2;
+    for (int kl = k0; kl < k1; kl += vn1) {
+        const int line = kl / vn1;
+        const int j2 = line % vn2, j3 = line / vn2;
+        if (j3 != j3cur) { flush(j3cur); j3cur = j3; }
+        float2 L[NL], E[NL];
+#pragma unroll
+        for (int i = 0; i < NL; ++i) L[i] = E[i] = dup2(0.f);
+        const size_t off = (size_t)kl * P;
+        for (int j0 = 0; j0 < vn1; j0 += MCH) {
+            float2 F[MCH], G[C == 2 ? MCH : 1];
+#pragma unroll
+            for (int i = 0; i < MCH; ++i) {
+                if (j0 + i < vn1) {
+                    const size_t o = off + (size_t)(j0 + i) * P;
+                    F[i] = make_float2(__ldcs(fa + o), __ldcs(fb + o));
+                    if (C == 2) G[C == 2 ? i : 0] = make_float2(__ldcs(fa + GO + o), __ldcs(fb + GO + o));
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < MCH; ++i) {
+                const int j1 = j0 + i;
+                if (j1 < vn1) {
+                    const float jt = (float)(j1 - jc[0]), cj = trap(j1, vn1);
+                    const float2 cF = __fmul2_rn(dup2(cj), F[i]);
+                    sum2x2(L[0], E[0], cF);
+                    const float2 p1 = __fmul2_rn(cF, dup2(jt));
+                    sum2x2(L[1], E[1], p1);
+                    E[1] = sub2(E[1], __ffma2_rn(cF, dup2(-jt), p1));
+                    const float jj = __fmul_rn(jt, jt);                  // exact
+                    const float2 p2 = __fmul2_rn(cF, dup2(jj));
+                    sum2x2(L[2], E[2], p2);
+                    E[2] = sub2(E[2], __ffma2_rn(cF, dup2(-jj), p2));
+                    if (C == 2) sum2x2(L[NL - 1], E[NL - 1], __fmul2_rn(dup2(cj), G[C == 2 ? i : 0]));
+                }
+            }
+        }
+        const float c2 = trap(j2, vn2), t2 = (float)(j2 - jc[1]);
+        const float b = __fmul_rn(c2, t2), bb = __fmul_rn(b, t2);       // exact
+        plane_add2(Pl[0], Pe[0], c2, L[0], E[0]);
+        plane_add2(Pl[1], Pe[1], c2, L[1], E[1]);
+        plane_add2(Pl[2], Pe[2], c2, L[2], E[2]);
+        plane_add2(Pl[3], Pe[3], b, L[0], E[0]);
+        plane_add2(Pl[4], Pe[4], b, L[1], E[1]);
+        plane_add2(Pl[5], Pe[5], bb, L[0], E[0]);
+        if (C == 2) plane_add2(Pl[NQ - 1], Pe[NQ - 1], c2, L[NL - 1], E[NL - 1]);
+    }
+    flush(j3cur);
+    const double uc[3] = {vg.lo[0] + jc[0] * vg.h[0], vg.lo[1] + jc[1] * vg.h[1], vg.lo[2] + jc[2] * vg.h[2]};
+    raw_in_place(Ja, P, vg, uc);
+    if (two) raw_in_place(Jb, P, vg, uc);
+}
+
+// Sum of eight pairs of values v with errors e: a balanced tree of TwoSums
+// (independent at each level, so no serial chain), the errors summed along.
+// s + c is within about 2^-51 of the sum of magnitudes.
+__device__ __forceinline__ void tree8(float2 (&v)[8], float2 (&e)[8], float2 &s, float2 &c) {
+#pragma unroll
+    for (int w = 4; w > 0; w >>= 1)
+#pragma unroll
+        for (int i = 0; i < w; ++i) {
+            const float2 a = v[i], b = v[i + w];
+            const float2 t = __fadd2_rn(a, b);
+            const float2 bp = sub2(t, a);
+            const float2 r = __fadd2_rn(sub2(a, sub2(t, bp)), sub2(b, bp));
+            v[i] = t;
+            e[i] = __fadd2_rn(__fadd2_rn(e[i], e[i + w]), r);
+        }
+    s = v[0];
+    c = e[0];
+}
+
+// Raw moments of an FP32 state for the diagnostic entry points, accurate as
+// FP64 sums are: eight velocities at a time as FP32 pair sums (tree8), those in
+// FP64.  1.75 FP64 instructions per value (0.63 ms of the FP64 pipe for the
+// state above, 0.90 in all) where a direct FP64 sum of the raw moments took 17
+// (7.18 ms).  Pair sums over whole lines are cheaper (0.45 ms) but lose up to
+// ten times more than FP64 sums do when lines are long and few.
+template <int C>
+__global__ void __launch_bounds__(MT, 2) k_moments_f32_diag(const float *f, double *part, VelGrid vg, int Nu, int P,
+                                                            int Kblk) {
+    constexpr int NL = C == 2 ? 4 : 3, NQ = C == 2 ? 7 : 6;
+    const int pa = blockIdx.x * (2 * MT) + threadIdx.x, pb = pa + MT;
+    if (pa >= P) return;
+    const bool two = pb < P;
+    const float *fa = f + pa, *fb = f + (two ? pb : pa);
+    const int vb = blockIdx.y;
+    const int k0 = vb * Kblk, k1 = min(Nu, k0 + Kblk);
+    const int vn1 = vg.n[0], vn2 = vg.n[1];
+    const int jc[3] = {(vn1 - 1) / 2, (vn2 - 1) / 2, (vg.n[2] - 1) / 2};
+    const size_t GO = (size_t)Nu * P;
+    double *Ja = part + (size_t)vb * BGK_NMOM * P + pa;
+    double *Jb = part + (size_t)vb * BGK_NMOM * P + (two ? pb : pa);
+    double Pd[2][NQ];
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) Pd[0][i] = Pd[1][i] = 0.0;
+    bool first = true;
+    auto flush = [&](int j3) {
+        const double c = trap3(j3, vg), t = (float)(j3 - jc[2]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (h == 1 && !two) break;
+            double d[7];
+#pragma unroll
+            for (int i = 0; i < 7; ++i) d[i] = i < NQ ? Pd[h][i] : 0.0;
+            plane_to_part(h ? Jb : Ja, P, c, t, d, first);
+        }
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) Pd[0][i] = Pd[1][i] = 0.0;
+        first = false;
+    };
+    int j3cur = (k0 / vn1) / vn2;
+    for (int kl = k0; kl < k1; kl += vn1) {
+        const int line = kl / vn1;
+        const int j2 = line % vn2, j3 = line / vn2;
+        if (j3 != j3cur) { flush(j3cur); j3cur = j3; }
+        double T[2][NL];
+#pragma unroll
+        for (int i = 0; i < NL; ++i) T[0][i] = T[1][i] = 0.0;
+        const size_t off = (size_t)kl * P;
+        for (int j0 = 0; j0 < vn1; j0 += 8) {
+            float2 F[8], v[8], e[8], s, c;
+            auto join = [&](int i) {
+                T[0][i] += (double)s.x + (double)c.x;
+                T[1][i] += (double)s.y + (double)c.y;
+            };
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                F[i] = dup2(0.f);
+                if (j0 + i < vn1) {
+                    const size_t o = off + (size_t)(j0 + i) * P;
+                    F[i] = make_float2(__ldcs(fa + o), __ldcs(fb + o));
+                }
+            }
+            float2 G[C == 2 ? 8 : 1];
+            if constexpr (C == 2) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    G[i] = dup2(0.f);
+                    if (j0 + i < vn1) {
+                        const size_t o = GO + off + (size_t)(j0 + i) * P;
+                        G[i] = make_float2(__ldcs(fa + o), __ldcs(fb + o));
+                        G[i] = __fmul2_rn(dup2(trap(j0 + i, vn1)), G[i]);            // exact
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (j0 + i < vn1) F[i] = __fmul2_rn(dup2(trap(j0 + i, vn1)), F[i]);   // exact
+                v[i] = F[i];
+                e[i] = dup2(0.f);
+            }
+            tree8(v, e, s, c);
+            join(0);
+#pragma unroll
+            for (int q = 1; q <= 2; ++q) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float t = (float)(j0 + i - jc[0]), w = q == 1 ? t : __fmul_rn(t, t);    // exact
+                    v[i] = __fmul2_rn(F[i], dup2(w));
+                    e[i] = __ffma2_rn(F[i], dup2(w), neg2(v[i]));
+                }
+                tree8(v, e, s, c);
+                join(q);
+            }
+            if constexpr (C == 2) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) { v[i] = G[i]; e[i] = dup2(0.f); }
+                tree8(v, e, s, c);
+                join(NL - 1);
+            }
+        }
+        const double cd = trap(j2, vn2), t2 = (double)(j2 - jc[1]), bd = cd * t2, bbd = bd * t2;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            Pd[h][0] = fma(cd, T[h][0], Pd[h][0]); Pd[h][1] = fma(cd, T[h][1], Pd[h][1]); Pd[h][2] = fma(cd, T[h][2], Pd[h][2]);
+            Pd[h][3] = fma(bd, T[h][0], Pd[h][3]); Pd[h][4] = fma(bd, T[h][1], Pd[h][4]);
+            Pd[h][5] = fma(bbd, T[h][0], Pd[h][5]);
+            if (C == 2) Pd[h][NQ - 1] = fma(cd, T[h][NL - 1], Pd[h][NQ - 1]);
+        }
+    }
+    flush(j3cur);
+    const double uc[3] = {vg.lo[0] + jc[0] * vg.h[0], vg.lo[1] + jc[1] * vg.h[1], vg.lo[2] + jc[2] * vg.h[2]};
+    raw_in_place(Ja, P, vg, uc);
+    if (two) raw_in_place(Jb, P, vg, uc);
+}
+
+// The diagnostic entry points' second look: partials that are not finite (an
+// infinity or NaN in the state, or FP32 sums out of range) are summed again
+// in FP64, which keeps an infinite or huge value's moments what they are.
+__global__ void __launch_bounds__(MT) k_moments_redo(const float *f, double *part, const double *vtab, int Nu, int P,
+                                                     int Kblk, int C) {
+    const int p = blockIdx.x * MT + threadIdx.x, vb = blockIdx.y;
+    if (p >= P) return;
+    double *out = part + (size_t)vb * BGK_NMOM * P + p;
+    if (isfinite(out[0] + out[(size_t)4 * P] + out[(size_t)5 * P] + out[(size_t)6 * P] + out[(size_t)10 * P])) return;
+    const int k0 = vb * Kblk, k1 = min(Nu, k0 + Kblk);
+    double m[BGK_NMOM];
+#pragma unroll
+    for (int j = 0; j < BGK_NMOM; ++j) m[j] = 0.0;
+    for (int k = k0; k < k1; ++k) {
+        const double *v = vtab + (size_t)k * BGK_VTAB;
+        const double u1 = v[0], u2 = v[1], u3 = v[2], w = v[3];
+        const double wF = w * (double)f[(size_t)k * P + p];
+        m[0] += wF;
+        m[1] = fma(wF, u1, m[1]);
+        m[2] = fma(wF, u2, m[2]);
+        m[3] = fma(wF, u3, m[3]);
+        m[4] = fma(wF * u1, u1, m[4]);
+        m[5] = fma(wF * u2, u2, m[5]);
+        m[6] = fma(wF * u3, u3, m[6]);
+        m[7] = fma(wF * u1, u2, m[7]);
+        m[8] = fma(wF * u1, u3, m[8]);
+        m[9] = fma(wF * u2, u3, m[9]);
+        if (C == 2) m[10] = fma(w, (double)f[((size_t)Nu + k) * P + p], m[10]);
+    }
+#pragma unroll
+    for (int j = 0; j < BGK_NMOM; ++j) out[(size_t)j * P] = m[j];
+}
+
+// Raw moments of an FP64 state: per line T_m = sum_j c jt^m F (m <= 2) and
+// sum_j c G, three (four) FP64 instructions per value instead of the 17 of a
+// direct sum of the raw moments; folded per line into the centred index
+// moments.  The FP64 pipe still bounds it: 1.1e8 values in 1.09 ms (0.83 TB/s),
+// 0.54 of it the pipe's own time, against about 3 before.
+template <int C>
+__global__ void __launch_bounds__(MT) k_moments_f64(const double *f, double *part, VelGrid vg, int Nu, int P, int Kblk) {
+    const int p = blockIdx.x * MT + threadIdx.x;
+    __shared__ double2 sj[BGK_MAXV];                     // (jt, jt^2) of the first-axis nodes
+    const int vn1 = vg.n[0], vn2 = vg.n[1];
+    const int jc[3] = {(vn1 - 1) / 2, (vn2 - 1) / 2, (vg.n[2] - 1) / 2};
+    for (int j = threadIdx.x; j < vn1; j += MT) {
+        const double t = j - jc[0];
+        sj[j] = make_double2(t, t * t);
+    }
+    __syncthreads();
+    if (p >= P) return;
+    const int vb = blockIdx.y;
+    const int k0 = vb * Kblk, k1 = min(Nu, k0 + Kblk);
+    double J[11];
+#pragma unroll
+    for (int i = 0; i < 11; ++i) J[i] = 0.0;
+    for (int kl = k0; kl < k1; kl += vn1) {
+        const int line = kl / vn1;
+        const int j2 = line % vn2, j3 = line / vn2;
+        const double *fl = f + (size_t)kl * P + p, *gl = fl + (size_t)Nu * P;
+        double T0 = 0.0, T1 = 0.0, T2 = 0.0, TG = 0.0;
+        for (int j0 = 0; j0 < vn1; j0 += MCH) {
+            double F[MCH], G[C == 2 ? MCH : 1];
+#pragma unroll
+            for (int i = 0; i < MCH; ++i)
+                if (j0 + i < vn1) {
+                    F[i] = __ldcs(fl + (size_t)(j0 + i) * P);
+                    if (C == 2) G[C == 2 ? i : 0] = __ldcs(gl + (size_t)(j0 + i) * P);
+                }
+#pragma unroll
+            for (int i = 0; i < MCH; ++i) {
+                const int j1 = j0 + i;
+                if (j1 < vn1) {
+                    if (j1 == 0 || j1 == vn1 - 1) {      // trapezoid half weight
+                        F[i] *= 0.5;
+                        if (C == 2) G[C == 2 ? i : 0] *= 0.5;
+                    }
+                    const double2 t = sj[j1];
+                    T0 += F[i];
+                    T1 = fma(t.x, F[i], T1);
+                    T2 = fma(t.y, F[i], T2);
+                    if (C == 2) TG += G[C == 2 ? i : 0];
+                }
+            }
+        }
+        const double c = (double)trap(j2, vn2) * (double)trap3(j3, vg), t2 = j2 - jc[1], t3 = j3 - jc[2];
+        const double cT0 = c * T0, cT1 = c * T1;
+        J[0] += cT0; J[1] += cT1; J[2] = fma(c, T2, J[2]);
+        J[3] = fma(t2, cT0, J[3]); J[4] = fma(t2, cT1, J[4]); J[5] = fma(t2 * t2, cT0, J[5]);
+        J[6] = fma(t3, cT0, J[6]); J[7] = fma(t3, cT1, J[7]); J[8] = fma(t2 * t3, cT0, J[8]);
+        J[9] = fma(t3 * t3, cT0, J[9]);
+        if (C == 2) J[10] = fma(c, TG, J[10]);
+    }
+    const double uc[3] = {vg.lo[0] + jc[0] * vg.h[0], vg.lo[1] + jc[1] * vg.h[1], vg.lo[2] + jc[2] * vg.h[2]};
+    double m[BGK_NMOM];
+    index_to_raw(J, vg, uc, m);
+#pragma unroll
+    for (int i = 0; i < BGK_NMOM; ++i) part[((size_t)vb * BGK_NMOM + i) * P + p] = m[i];
+}
+
+// Sums over the velocity blocks, one thread per (slot, point): ACROSS writes
+// m_out[p][slot] (bgk_moments), else out[slot][p] (a shard's partials).
+template <bool ACROSS>
+__global__ void __launch_bounds__(MT) k_reduce_moments(const double *part, int n_vblk, int P, double *out) {
+    const int p = blockIdx.x * MT + threadIdx.x, j = blockIdx.y;
+    if (p >= P) return;
+    const double *q = part + (size_t)j * P + p;
+    double s = 0.0;
+#pragma unroll 8
+    for (int vb = 0; vb < n_vblk; ++vb) s += q[(size_t)vb * BGK_NMOM * P];
+    out[ACROSS ? (size_t)p * BGK_NMOM + j : (size_t)j * P + p] = s;
+}
+
+// ---- entropy ---------------------------------------------------------------
+// ln x of a normal FP32 x as an unevaluated pair s + c (table-driven, after
+// Tang 1990): x = 2^e m with m in [1, 2), k_i = 1/m to 9 bits for the 256
+// subintervals of m, so r = m k_i - 1 is exact in FP32 (33 bits of m k_i less
+// the 9 that cancel, |r| <= 2^-8), and
+//   ln x = e ln2 - ln k_i + r - r^2/2 + r^3 (1/3 - r/4 + r^2/5 - ...).
+// ln2 is split so that e times its two leading parts is exact; the large
+// terms are added with their rounding errors kept (TwoSum).  The pair is good
+// to about 2^-47 of max(|ln x|, 1); on two values at once.
+struct LogTab { float k, hi, lo, pad; };                 // k_i, -ln k_i = hi + lo
+__device__ __forceinline__ void two_sum2(float2 &s, float2 &c, float2 v) {
+    const float2 t = __fadd2_rn(s, v);
+    const float2 bp = sub2(t, s);
+    c = __fadd2_rn(c, __fadd2_rn(sub2(s, sub2(t, bp)), sub2(v, bp)));
+    s = t;
+}
+__device__ __forceinline__ void log_pair2(const LogTab *tab, float2 x, float2 &s, float2 &c) {
+    const unsigned ba = __float_as_uint(x.x), bb = __float_as_uint(x.y);
+    const float4 ta = *reinterpret_cast<const float4 *>(tab + ((ba >> 15) & 255u));
+    const float4 tb = *reinterpret_cast<const float4 *>(tab + ((bb >> 15) & 255u));
+    const float2 m = make_float2(__uint_as_float((ba & 0x007fffffu) | 0x3f800000u),
+                                 __uint_as_float((bb & 0x007fffffu) | 0x3f800000u));
+    // the exponent as a float: 2^23 + biased exponent, minus 2^23 + 127 (exact)
+    const float2 e = __fadd2_rn(make_float2(__uint_as_float((ba >> 23) | 0x4b000000u),
+                                            __uint_as_float((bb >> 23) | 0x4b000000u)), dup2(-8388735.f));
+    const float2 r = __ffma2_rn(m, make_float2(ta.x, tb.x), dup2(-1.f));             // exact
+    const float2 q = __fmul2_rn(r, r);
+    const float2 qe = __ffma2_rn(r, r, neg2(q));                                     // r^2 = q + qe
+    float2 t = __ffma2_rn(r, dup2(-1.f / 6.f), dup2(0.2f));
+    t = __ffma2_rn(r, t, dup2(-0.25f));
+    t = __ffma2_rn(r, t, dup2(1.f / 3.f));
+    t = __fmul2_rn(__fmul2_rn(r, q), t);
+    s = __fmul2_rn(e, dup2(0.693145751953125f));                                     // exact
+    c = dup2(0.f);
+    two_sum2(s, c, make_float2(ta.y, tb.y));
+    two_sum2(s, c, r);
+    two_sum2(s, c, __fmul2_rn(e, dup2(LN2_MID)));                                    // exact product
+    two_sum2(s, c, __fmul2_rn(q, dup2(-0.5f)));
+    float2 w = __ffma2_rn(qe, dup2(-0.5f), t);
+    w = __fadd2_rn(w, make_float2(ta.z, tb.z));
+    w = __ffma2_rn(e, dup2(LN2_LO), w);
+    c = __fadd2_rn(c, w);
+}
+
+// Discrete entropy of the F component, partial over velocity blocks:
+// part[vb][p] = sum_{k in block vb} w_k F ln F; a non-positive F (or NaN) has
+// no entropy and is counted in *nonpos instead.  Two points per thread, the
+// logarithm and the line sums as FP32 pairs, one FP64 update per line: the
+// FP64 log and sum of every value took 12 ms for 2.3e8 values (25 FP64
+// instructions each), this is bound by FP32 issue (about 45 per value).
+__global__ void __launch_bounds__(MT, 4) k_entropy_f32(const float *f, VelGrid vg, int Nu, int P, int Kblk, double *part,
+                                                       unsigned int *nonpos) {
+    __shared__ __align__(16) LogTab tab[256];
+    for (int i = threadIdx.x; i < 256; i += MT) {
+        const double k = rint(512.0 / (1.0 + (i + 0.5) / 256.0)) / 512.0;
+        const double l = -log(k);
+        tab[i].k = (float)k;
+        tab[i].hi = (float)l;
+        tab[i].lo = (float)(l - (double)(float)l);
+        tab[i].pad = 0.f;
+    }
+    __syncthreads();
+    const int pa = blockIdx.x * (2 * MT) + threadIdx.x, pb = pa + MT;
+    if (pa >= P) return;
+    const bool two = pb < P;
+    const float *fa = f + pa, *fb = f + (two ? pb : pa);
+    const int vb = blockIdx.y;
+    const int k0 = vb * Kblk, k1 = min(Nu, k0 + Kblk);
+    const int vn1 = vg.n[0], vn2 = vg.n[1];
+    double h[2] = {0.0, 0.0};
+    unsigned int bad = 0;
+    for (int kl = k0; kl < k1; kl += vn1) {
+        const int line = kl / vn1;
+        const double c23 = (double)trap(line % vn2, vn2) * (double)trap3(line / vn2, vg);
+        float2 L = dup2(0.f), E = dup2(0.f);
+        for (int j0 = 0; j0 < vn1; j0 += MCH) {
+            float2 F[MCH];
+#pragma unroll
+            for (int i = 0; i < MCH; ++i)
+                if (j0 + i < vn1) {
+                    const size_t o = (size_t)(kl + j0 + i) * P;
+                    F[i] = make_float2(__ldcs(fa + o), __ldcs(fb + o));
+                }
+#pragma unroll
+            for (int i = 0; i < MCH; ++i) {
+                if (j0 + i >= vn1) continue;
+                const float cj = trap(j0 + i, vn1);
+                // outside the positive normal range: subnormal and infinite
+                // values by the FP64 log, anything else is counted
+                if ((__float_as_uint(F[i].x) - 0x00800000u) >= 0x7f000000u || (__float_as_uint(F[i].y) - 0x00800000u) >= 0x7f000000u) {
+                    for (int q = 0; q < 2; ++q) {
+                        const float v = q ? F[i].y : F[i].x;
+                        if ((__float_as_uint(v) - 0x00800000u) < 0x7f000000u) continue;
+                        if (v > 0.f) h[q] = fma(c23 * (double)cj * (double)v, log((double)v), h[q]);
+                        else if (q == 0 || two) ++bad;
+                        if (q) F[i].y = 1.f;
+                        else F[i].x = 1.f;                       // ln 1 = 0: no term
+                    }
+                }
+                float2 ls, lc;
+                log_pair2(tab, F[i], ls, lc);
+                const float2 cF = __fmul2_rn(dup2(cj), F[i]);                        // exact
+                const float2 p = __fmul2_rn(cF, ls);
+                sum2x2(L, E, p);
+                E = __fadd2_rn(E, __ffma2_rn(cF, lc, __ffma2_rn(cF, ls, neg2(p))));
+            }
+        }
+        h[0] = fma(c23, (double)L.x + (double)E.x, h[0]);
+        h[1] = fma(c23, (double)L.y + (double)E.y, h[1]);
+    }
+    const double W = vg.h[0] * vg.h[1] * vg.h[2];
+    part[(size_t)vb * P + pa] = W * h[0];
+    if (two) part[(size_t)vb * P + pb] = W * h[1];
+    if (bad) atomicAdd(nonpos, bad);
+}
+
+// The same of an FP64 state.  ln F by the same table in FP64, r = m k_i - 1
+// with one rounding and the series to r^7 (2^-67 of the next term): 12 FP64
+// instructions per value in place of the library log()'s path (36 ms for
+// 1.1e8 values); the FP64 pipe bounds it.
+__global__ void __launch_bounds__(MT) k_entropy_f64(const double *f, VelGrid vg, int Nu, int P, int Kblk, double *part,
+                                                    unsigned int *nonpos) {
+    __shared__ double2 tab[256];                         // (k_i, -ln k_i)
+    for (int i = threadIdx.x; i < 256; i += MT) {
+        const double k = rint(512.0 / (1.0 + (i + 0.5) / 256.0)) / 512.0;
+        tab[i] = make_double2(k, -log(k));
+    }
+    __syncthreads();
+    const int p = blockIdx.x * MT + threadIdx.x;
+    if (p >= P) return;
+    const int vb = blockIdx.y;
+    const int k0 = vb * Kblk, k1 = min(Nu, k0 + Kblk);
+    const int vn1 = vg.n[0], vn2 = vg.n[1];
+    double h = 0.0;
+    unsigned int bad = 0;
+    for (int kl = k0; kl < k1; kl += vn1) {
+        const int line = kl / vn1;
+        double T = 0.0;
+        for (int j0 = 0; j0 < vn1; j0 += MCH) {
+            double Fc[MCH];
+#pragma unroll
+            for (int i = 0; i < MCH; ++i)
+                if (j0 + i < vn1) Fc[i] = __ldcs(f + (size_t)(kl + j0 + i) * P + p);
+#pragma unroll
+            for (int i = 0; i < MCH; ++i) {
+                const int j1 = j0 + i;
+                if (j1 >= vn1) continue;
+                const double F = Fc[i];
+                const unsigned hi = (unsigned)__double2hiint(F);
+                double l;
+                if (hi - 0x00100000u >= 0x7fe00000u) {           // not a positive normal value
+                    if (!(F > 0.0)) { ++bad; continue; }
+                    l = log(F);
+                } else {
+                    const double2 t = tab[(hi >> 12) & 255u];
+                    const double m = __hiloint2double((hi & 0x000fffffu) | 0x3ff00000u, __double2loint(F));
+                    // 2^52 + biased exponent, minus 2^52 + 1023 (exact)
+                    const double e = __hiloint2double(0x43300000, hi >> 20) - 4503599627371519.0;
+                    const double r = fma(m, t.x, -1.0);
+                    double q = fma(r, 1.0 / 7.0, -1.0 / 6.0);
+                    q = fma(r, q, 0.2);
+                    q = fma(r, q, -0.25);
+                    q = fma(r, q, 1.0 / 3.0);
+                    q = fma(r, q, -0.5);
+                    l = fma(e, 0.69314718055994530942, t.y) + fma(r * r, q, r);
+                }
+                T = fma(j1 == 0 || j1 == vn1 - 1 ? 0.5 * F : F, l, T);
+            }
+        }
+        h = fma((double)trap(line % vn2, vn2) * (double)trap3(line / vn2, vg), T, h);
+    }
+    part[(size_t)vb * P + p] = vg.h[0] * vg.h[1] * vg.h[2] * h;
+    if (bad) atomicAdd(nonpos, bad);
+}
+
+// ---- domain totals -----------------------------------------------------------
+// sum_p W_p (rho, rho U, E) of the moments mom[P][11] and, with ent, sum_p W_p
+// sum_vb ent[vb][p]: W_p the quadrature weight (node weights times |J_e| on the
+// box, geo[p][10] on a curvilinear mesh).  Fixed grid and order, so equal
+// states give equal totals; blocks write six sums each, one block adds them.
+constexpr int TOT_BLOCKS = 152;
+__global__ void __launch_bounds__(MT) k_totals(const double *mom, const double *ent, int n_vblk, int P, FROps fr,
+                                               double jac, const double *geo, double *blk) {
+    const int q = fr.q, Ns = q * q * q;
+    double t[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int p = blockIdx.x * MT + threadIdx.x; p < P; p += gridDim.x * MT) {
+        const int s = p % Ns;
+        const double W = geo ? geo[(size_t)p * BGK_NGEO + 10] : fr.wq[s % q] * fr.wq[(s / q) % q] * fr.wq[s / (q * q)] * jac;
+        const double *m = mom + (size_t)p * BGK_NMOM;
+        t[0] = fma(W, m[0], t[0]); t[1] = fma(W, m[1], t[1]); t[2] = fma(W, m[2], t[2]); t[3] = fma(W, m[3], t[3]);
+        t[4] = fma(W, 0.5 * (m[4] + m[5] + m[6]) + m[10], t[4]);
+        if (ent) {
+            double h = 0.0;
+#pragma unroll 4
+            for (int vb = 0; vb < n_vblk; ++vb) h += ent[(size_t)vb * P + p];
+            t[5] = fma(W, h, t[5]);
+        }
+    }
+    __shared__ double red[6][MT / 32];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        for (int o = 16; o > 0; o >>= 1) t[j] += __shfl_xor_sync(0xffffffffu, t[j], o);
+        if ((threadIdx.x & 31) == 0) red[j][threadIdx.x >> 5] = t[j];
+    }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        double s = 0.0;
+        for (int w = 0; w < MT / 32; ++w) s += red[threadIdx.x][w];
+        blk[(size_t)blockIdx.x * 6 + threadIdx.x] = s;
+    }
+}
+__global__ void k_totals_sum(const double *blk, int n, double *out) {
+    if (threadIdx.x < 6) {
+        double s = 0.0;
+        for (int b = 0; b < n; ++b) s += blk[(size_t)b * 6 + threadIdx.x];
+        out[threadIdx.x] = s;
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_moments_f64(const MomentArgs64 &a, const VelGrid &vg, int n_vblk, cudaStream_t s) {
+    dim3 grid((a.P + MT - 1) / MT, n_vblk);
+    if (a.C == 1) k_moments_f64<1><<<grid, MT, 0, s>>>(a.f, a.part, vg, a.Nu, a.P, a.Kblk);
+    else k_moments_f64<2><<<grid, MT, 0, s>>>(a.f, a.part, vg, a.Nu, a.P, a.Kblk);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_moments_f32(const float *f, double *part, const double *vtab, const VelGrid &vg, int Nu, int P,
+                               int Kblk, int C, int n_vblk, bool check, cudaStream_t s) {
+    const dim3 grid((P + 2 * MT - 1) / (2 * MT), n_vblk);
+    if (!check) {
+        if (C == 1) k_moments_f32<1><<<grid, MT, 0, s>>>(f, part, vg, Nu, P, Kblk);
+        else k_moments_f32<2><<<grid, MT, 0, s>>>(f, part, vg, Nu, P, Kblk);
+        return cudaGetLastError();
+    }
+    if (C == 1) k_moments_f32_diag<1><<<grid, MT, 0, s>>>(f, part, vg, Nu, P, Kblk);
+    else k_moments_f32_diag<2><<<grid, MT, 0, s>>>(f, part, vg, Nu, P, Kblk);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_moments_redo<<<dim3((P + MT - 1) / MT, n_vblk), MT, 0, s>>>(f, part, vtab, Nu, P, Kblk, C);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sum_partials(const double *part, int n_vblk, int P, double *out, cudaStream_t s) {
+    k_reduce_moments<false><<<dim3((P + MT - 1) / MT, BGK_NMOM), MT, 0, s>>>(part, n_vblk, P, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reduce_moments(const double *part, int n_vblk, int P, double *m_out, cudaStream_t s) {
+    k_reduce_moments<true><<<dim3((P + MT - 1) / MT, BGK_NMOM), MT, 0, s>>>(part, n_vblk, P, m_out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_entropy_f32(const float *f, const VelGrid &vg, int Nu, int P, int Kblk, int n_vblk, double *part,
+                               unsigned int *nonpos, cudaStream_t s) {
+    k_entropy_f32<<<dim3((P + 2 * MT - 1) / (2 * MT), n_vblk), MT, 0, s>>>(f, vg, Nu, P, Kblk, part, nonpos);
+    return cudaGetLastError();
+}
+cudaError_t launch_entropy_f64(const double *f, const VelGrid &vg, int Nu, int P, int Kblk, int n_vblk, double *part,
+                               unsigned int *nonpos, cudaStream_t s) {
+    k_entropy_f64<<<dim3((P + MT - 1) / MT, n_vblk), MT, 0, s>>>(f, vg, Nu, P, Kblk, part, nonpos);
+    return cudaGetLastError();
+}
+
+size_t totals_scratch() { return (size_t)(TOT_BLOCKS + 1) * 6; }
+cudaError_t launch_totals(const double *mom, const double *ent, int n_vblk, int P, const FROps &fr, double jac,
+                          const double *geo, double *scratch, cudaStream_t s) {
+    const int nb = std::min(TOT_BLOCKS, (P + MT - 1) / MT);
+    k_totals<<<nb, MT, 0, s>>>(mom, ent, n_vblk, P, fr, jac, geo, scratch + 6);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_totals_sum<<<1, 32, 0, s>>>(scratch + 6, nb, scratch);
+    return cudaGetLastError();
+}
