@@ -38,7 +38,9 @@ struct bgk_ctx {
     std::vector<double> geo_h;        // [P][BGK_NGEO]
     double *geo, *fvec;               // FP64 metric terms and face vectors
     float *geo32, *fvec32;            // their FP32 copies (mixed form)
+    float *geop;                      // the same in the FP32 stage kernel's thread order
     double *rho_w;                    // [Ne][6][q*q] diffuse-wall densities
+    float2 *rho_w2, *bc2;             // rho_w and bcval as FP32 pairs (mixed form)
     CurvOps32 cops;                   // FP32 tables of the mixed-form curvilinear stage
     int *wall_ef;                     // [n_wall][2] (element, face) pairs on diffuse faces
     int n_wall;
@@ -307,7 +309,8 @@ void set_geometry<double>(bgk_ctx *ctx, StageArgs<double> &s) {
 }
 template <>
 void set_geometry<float>(bgk_ctx *ctx, StageArgs<float> &s) {
-    s.geo = ctx->geo32; s.fvec = ctx->fvec32; s.rho_w = ctx->rho_w;
+    s.geo = ctx->geo32; s.fvec = ctx->fvec32; s.geop = ctx->geop; s.rho_w = ctx->rho_w;
+    s.rho_w2 = ctx->rho_w2; s.bc2 = ctx->bc2;
     s.cops = ctx->cops;
 }
 
@@ -348,6 +351,13 @@ void build_curv_ops32(const FROps &fr, CurvOps32 &c) {
                           (1.0 - slp) * fr.wq[j] * (double)c.dgR[j] - (1.0 - slm) * fr.wq[j] * (double)c.dgL[j];
         c.def[j] = (float)(dj / wsum);
     }
+    for (int i = 0; i < q; ++i)
+        for (int j = 0; j < q; ++j) {
+            const double k = (double)c.D[i][j] - (double)c.def[j] - (double)c.dgR[i] * (double)c.lp[j] -
+                             (double)c.dgL[i] * (double)c.lm[j];
+            c.kh[i][j] = (float)k;
+            c.kl[i][j] = (float)(k - (double)c.kh[i][j]);
+        }
 }
 
 template <typename T>
@@ -376,11 +386,11 @@ bgk_status run_stage(bgk_ctx *ctx, const void *fn, const void *fs, void *fo, dou
         if (ctx->precision == BGK_FP64)
             CU(launch_wall_density<double>((const double *)fs, ctx->fvec, ctx->bcval, ctx->vtab, ctx->wall_ef,
                                            ctx->n_wall, ctx->q, ctx->Ne, ctx->Nu, ctx->C, ctx->fr, ctx->rho_w,
-                                           ctx->stream));
+                                           nullptr, ctx->stream));
         else
             CU(launch_wall_density<float>((const float *)fs, ctx->fvec32, ctx->bcval, ctx->vtab, ctx->wall_ef,
                                           ctx->n_wall, ctx->q, ctx->Ne, ctx->Nu, ctx->C, ctx->fr, ctx->rho_w,
-                                          ctx->stream));
+                                          ctx->rho_w2, ctx->stream));
     }
     LaunchScope ls(ctx, BGK_K_STAGE);
     if (ctx->precision == BGK_FP64)
@@ -634,7 +644,8 @@ bgk_status create_ctx(bgk_ctx **out, const bgk_mesh_desc *mesh, const bgk_vgrid_
     std::memcpy(ctx->bc, mesh->bc_state, sizeof ctx->bc);
     build_fr(ctx->p, ctx->fr);
     ctx->curved = curved;
-    ctx->geo = ctx->fvec = nullptr; ctx->geo32 = ctx->fvec32 = nullptr;
+    ctx->geo = ctx->fvec = nullptr; ctx->geo32 = ctx->fvec32 = ctx->geop = nullptr;
+    ctx->rho_w2 = ctx->bc2 = nullptr;
     ctx->rho_w = nullptr; ctx->wall_ef = nullptr; ctx->n_wall = 0;
     std::vector<double> fvec_h;
     std::vector<int> wall_h;
@@ -835,6 +846,19 @@ bgk_status create_ctx(bgk_ctx **out, const bgk_mesh_desc *mesh, const bgk_vgrid_
         if (st == BGK_OK) cu(cudaMalloc(&ctx->fvec32, nf * sizeof(float)), "cudaMalloc(fvec32)");
         if (st == BGK_OK) cu(cudaMalloc(&ctx->rho_w, (size_t)ctx->Ne * 6 * ctx->q * ctx->q * sizeof(double)), "cudaMalloc(rho_w)");
         if (st == BGK_OK && ctx->n_wall) cu(cudaMalloc(&ctx->wall_ef, wall_h.size() * sizeof(int)), "cudaMalloc(wall)");
+        if (st == BGK_OK && precision == BGK_MIXED) {
+            std::vector<float> gp;
+            curved_geop(q, g32.data(), f32.data(), ctx->mesh, ctx->cops, gp);
+            cu(cudaMalloc(&ctx->geop, gp.size() * sizeof(float)), "cudaMalloc(geop)");
+            if (st == BGK_OK) cu(cudaMemcpy(ctx->geop, gp.data(), gp.size() * sizeof(float), cudaMemcpyHostToDevice), "upload geop");
+            std::vector<float2> b2(bcv.size());
+            for (size_t i = 0; i < bcv.size(); ++i) b2[i] = make_float2((float)bcv[i], (float)(bcv[i] - (double)(float)bcv[i]));
+            const size_t nw = (size_t)ctx->Ne * 6 * ctx->q * ctx->q * sizeof(float2);
+            if (st == BGK_OK) cu(cudaMalloc(&ctx->bc2, b2.size() * sizeof(float2)), "cudaMalloc(bc2)");
+            if (st == BGK_OK) cu(cudaMalloc(&ctx->rho_w2, nw), "cudaMalloc(rho_w2)");
+            if (st == BGK_OK) cu(cudaMemcpy(ctx->bc2, b2.data(), b2.size() * sizeof(float2), cudaMemcpyHostToDevice), "upload bc2");
+            if (st == BGK_OK) cu(cudaMemset(ctx->rho_w2, 0, nw), "memset rho_w2");
+        }
         if (st == BGK_OK) cu(cudaMemcpy(ctx->geo, ctx->geo_h.data(), ng * sizeof(double), cudaMemcpyHostToDevice), "upload geo");
         if (st == BGK_OK) cu(cudaMemcpy(ctx->fvec, fvec_h.data(), nf * sizeof(double), cudaMemcpyHostToDevice), "upload fvec");
         if (st == BGK_OK) cu(cudaMemcpy(ctx->geo32, g32.data(), g32.size() * sizeof(float), cudaMemcpyHostToDevice), "upload geo32");
@@ -948,7 +972,8 @@ bgk_status bgk_destroy(bgk_ctx *ctx) {
     cudaFree(ctx->iters); cudaFree(ctx->eq32); cudaFree(ctx->vtab); cudaFree(ctx->vtab32); cudaFree(ctx->bcval); cudaFree(ctx->status);
     if (ctx->shard) { cudaFree(ctx->vtab_q); cudaFree(ctx->vtab32_q); }
     cudaFree(ctx->stats);
-    cudaFree(ctx->geo); cudaFree(ctx->fvec); cudaFree(ctx->geo32); cudaFree(ctx->fvec32);
+    cudaFree(ctx->geo); cudaFree(ctx->fvec); cudaFree(ctx->geo32); cudaFree(ctx->fvec32); cudaFree(ctx->geop);
+    cudaFree(ctx->rho_w2); cudaFree(ctx->bc2);
     cudaFree(ctx->rho_w); cudaFree(ctx->wall_ef);
     cudaFree(ctx->mlp_w); cudaFree(ctx->mlp_w16); cudaFree(ctx->mlp_norm); cudaFree(ctx->mlp_m); cudaFree(ctx->mlp_v);
     cudaFree(ctx->mlp_grad); cudaFree(ctx->mlp_loss); cudaFree(ctx->log); cudaFree(ctx->log_count);

@@ -183,6 +183,10 @@ struct CurvOps32 {
     float lp[BGK_MAXQ], lm[BGK_MAXQ];
     float dgL[BGK_MAXQ], dgR[BGK_MAXQ];
     float def[BGK_MAXQ];
+    // kappa_ij = D_ij - def_j - g_R'_i l_j(+1) - g_L'_i l_j(-1), the coefficient
+    // of Ft_j - Ft_i in t_i with those of the traces and defects folded in, of
+    // the FP32 entries above in FP64, as an unevaluated FP32 pair kh + kl
+    float kh[BGK_MAXQ][BGK_MAXQ], kl[BGK_MAXQ][BGK_MAXQ];
 };
 
 // Arguments of the fused stage kernel:  f_out = a f_n + b f_s + c R(f_s).
@@ -200,7 +204,10 @@ struct StageArgs {
     // curvilinear meshes (all null on the uniform box)
     const T *geo;            // [P][BGK_NGEO]
     const T *fvec;           // [Ne][6][Q*Q][3] face vectors, oriented +xi_d
+    const float *geop;       // FP32 geometry in the curvilinear stage kernel's thread order (curved_geop)
     const double *rho_w;     // [Ne][6][Q*Q] diffuse-wall densities of this stage's input
+    const float2 *rho_w2;    // the same, and bcval, as FP32 pairs hi + lo (mixed form)
+    const float2 *bc2;
     CurvOps32 cops;          // FP32 operator tables (mixed form)
     unsigned int *status;    // device status word (BGK_DEV_* bits)
     double a, b, c;
@@ -265,11 +272,12 @@ bool build_curved_geometry(const FROps &fr, const int n[3], const int periodic[3
                            std::vector<double> &geo, std::vector<double> &fvec, std::string &err);
 
 // Diffuse-wall densities of a state (wall.cu): rho_w[e][f][fp] for the n_wall
-// (element, face) pairs in wall_ef[2 * i], wall_ef[2 * i + 1].
+// (element, face) pairs in wall_ef[2 * i], wall_ef[2 * i + 1]; rho_w2 (may be
+// null) the same as FP32 pairs.
 template <typename T>
 cudaError_t launch_wall_density(const T *f, const T *fvec, const double *bcval, const double *vtab,
                                 const int *wall_ef, int n_wall, int q, int Ne, int Nu, int C, FROps fr,
-                                double *rho_w, cudaStream_t s);
+                                double *rho_w, float2 *rho_w2, cudaStream_t s);
 
 // Launchers: the Q' solve and its tensor refinement (kernels_qprime.cu); the
 // FP64 stage and Maxwellian (kernels_f64.cu); the FP32 stage and Maxwellian
@@ -282,6 +290,11 @@ cudaError_t launch_maxwellian_f64(double *f, const double *q, const double *vtab
                                   int C, double delta, cudaStream_t s);
 cudaError_t launch_stage_f32(const StageArgs<float> &a, int C, int n_vblk, int variant, int depth,
                              cudaStream_t s);
+// the curvilinear FP32 stage (kernels_f32_curved.cu) and its host-built geometry:
+// from geo32[P][BGK_NGEO32] and fvec32[Ne][6][q*q][3], the vectors S of every
+// scalar u . S a thread of the kernel needs, [scalar][3][thread]
+cudaError_t launch_stage_f32_curved(const StageArgs<float> &a, int C, int n_vblk, cudaStream_t s);
+void curved_geop(int q, const float *geo32, const float *fvec32, const MeshInfo &mesh, const CurvOps32 &co, std::vector<float> &out);
 bool stage_f32_tma_supported(const StageArgs<float> &a, int C, int depth);
 // line kernels: kind 0 line, 1 line_wide, 2 half, 3 half_wide
 bool stage_f32_line_supported(const StageArgs<float> &a, int C, int kind, int depth);

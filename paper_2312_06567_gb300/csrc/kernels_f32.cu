@@ -33,7 +33,9 @@ __device__ __forceinline__ float2 psub(float2 x, float2 y) { return __ffma2_rn(y
 // R = -div + (g' - f)/tau.  g' = exp(c0) * exp2(-log2(e)/2 c^T A c) with the
 // per-point factor exp(c0) from FP64 and the exponent in FP32.
 //
-// Curvilinear elements (CURV): the transformed-flux form of the FP64 stage
+// Curvilinear elements (CURV; p = 4 with F and G only, where the line kernel of
+// kernels_f32_curved.cu spills: 1.85 against 2.9 ms per stage on 48 warped
+// elements, 18^3 velocities): the transformed-flux form of the FP64 stage
 // kernel (kernels_f64.cu) in FP32, regrouped so that every rounding acts on
 // deviations (see CurvOps32).  a_d = u . S^d per node is staged beside f; per
 // direction, with w_j = a_j (f_j - f_i),
@@ -48,8 +50,7 @@ __device__ __forceinline__ float2 psub(float2 x, float2 y) { return __ffma2_rn(y
 // telescoping of the element quadrature survive the FP32 arithmetic.
 template <int Q, int C, bool CURV>
 // Held to 128 registers (two blocks, 16 warps per SM; the curvilinear
-// instantiation keeps its geometry in shared memory): 1.7x faster on the
-// sphere O-grid at p = 1 than one block of 8 warps without the cap.
+// instantiation keeps its geometry in shared memory).
 #ifndef BGK_PLAIN_MINB
 #define BGK_PLAIN_MINB 2
 #endif
@@ -371,60 +372,6 @@ __global__ void __launch_bounds__(256, BGK_PLAIN_MINB) k_stage_f32(StageArgs<flo
                     const float *sfc = sf[buf][c];
                     const float fi = fself[c];
                     float div = 0.f;
-                    if constexpr (CURV) {
-#pragma unroll
-                        for (int d = 0; d < 3; ++d) {
-                            const float *own = sfc + le * NS + base[d];
-                            const float *ownA = sA[buf][d] + le * NS + base[d];
-                            float dF = 0.f, E = 0.f, trL = 0.f, trR = 0.f, fmL = 0.f, fmR = 0.f;
-#pragma unroll
-                            for (int m = 1; m < Q; ++m) {
-                                const int j = (id[d] + m) % Q;
-                                const float dfj = own[j * stride[d]] - fi;
-                                const float wj = ownA[j * stride[d]] * dfj;
-                                dF = fmaf(cD[id[d]][j], wj, dF);
-                                E = fmaf(cdef[j], wj, E);
-                                trL = fmaf(cl[1][j], wj, trL);
-                                trR = fmaf(cl[0][j], wj, trR);
-                                fmL = fmaf(cl[1][j], dfj, fmL);
-                                fmR = fmaf(cl[0][j], dfj, fmR);
-                            }
-                            float X[2];
-#pragma unroll
-                            for (int side = 0; side < 2; ++side) {
-                                const int fpi = d == 0 ? id[1] + Q * id[2] : (d == 1 ? id[0] + Q * id[2] : id[0] + Q * id[1]);
-                                const float A = sAf[buf][(le * 6 + 2 * d + side) * Q * Q + fpi];
-                                const float un = side ? A : -A;           // outward
-                                const int en = en_[d][side];
-                                const int kind = a.mesh.face_kind[2 * d + side];
-                                float dev;
-                                if (en < 0 && kind == BGK_FK_CLOSED) {
-                                    dev = -fi;                            // F^I = 0
-                                } else if (un > 0.f) {
-                                    dev = side ? fmR : fmL;
-                                } else if (en >= e0 && en < e0 + EB) {
-                                    const float *nb = sfc + (en - e0) * NS + base[d];
-                                    dev = 0.f;
-#pragma unroll
-                                    for (int j = 0; j < Q; ++j) dev = fmaf(cl[side][j], nb[j * stride[d]] - fi, dev);
-                                } else if (en >= 0) {
-                                    const float *nb = fs + (size_t)en * NS + base[d];
-                                    dev = 0.f;
-#pragma unroll
-                                    for (int j = 0; j < Q; ++j) dev = fmaf(cl[side][j], __ldg(nb + j * stride[d]) - fi, dev);
-                                } else {
-                                    double fpd = __ldg(a.bcval + ((size_t)(2 * d + side) * C + c) * a.Nu + k);
-                                    if (kind == BGK_FK_DIFFUSE)
-                                        fpd *= __ldg(a.rho_w + ((size_t)e * 6 + 2 * d + side) * Q * Q + fpi);
-                                    dev = (float)fpd - fi;
-                                }
-                                X[side] = fmaf(A, dev, -(side ? trR : trL));
-                            }
-                            div += fmaf(X[1], cg[1][id[d]], fmaf(X[0], cg[0][id[d]], dF - E));
-                        }
-                        div = fmaf(fi, fmaf(u[0], sG[tid][9], fmaf(u[1], sG[tid][10], u[2] * sG[tid][11])), div);
-                        div *= sG[tid][12];
-                    } else {
 #pragma unroll
                     for (int d = 0; d < 3; ++d) {
                         const int side = u[d] > 0.f ? 0 : 1;
@@ -464,7 +411,6 @@ __global__ void __launch_bounds__(256, BGK_PLAIN_MINB) k_stage_f32(StageArgs<flo
                         }
                         t = fmaf(sdg[side][id[d]], dn, fmaf(seps[side][id[d]], fi, t));
                         div = fmaf(toh[d] * u[d], t, div);
-                    }
                     }
                     const float eqv = (c == 0) ? g32 : __fmul_rn(gfac, g32);
                     const float eqc = (c == 0) ? gc : __fmul_rn(gfac, gc);
@@ -708,20 +654,24 @@ static cudaError_t stage32_q(const StageArgs<float> &a, int C, int n_vblk, cudaS
     constexpr int NS = Q * Q * Q, EB = 256 / NS;
     dim3 grid((a.mesh.Ne + EB - 1) / EB, n_vblk);
     if (a.geo) {
-        // the curvilinear instantiations' moment accumulators (dynamic shared memory)
-        const size_t dyn = (size_t)EB * NS * (11 * sizeof(double) + 14 * sizeof(float));
-        static SmemLimit lim;
-        size_t *attr = lim.slot();
-        if (!attr) return cudaErrorInvalidDevice;
-        if (dyn > *attr) {
-            cudaError_t e = cudaFuncSetAttribute(k_stage_f32<Q, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_stage_f32<Q, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-            if (e != cudaSuccess) return e;
-            *attr = dyn;
+        if constexpr (Q == 5) {
+            if (C == 2) {
+                // the curvilinear instantiation's moment accumulators (dynamic shared memory)
+                const size_t dyn = (size_t)EB * NS * (11 * sizeof(double) + 14 * sizeof(float));
+                static SmemLimit lim;
+                size_t *attr = lim.slot();
+                if (!attr) return cudaErrorInvalidDevice;
+                if (dyn > *attr) {
+                    const cudaError_t e =
+                        cudaFuncSetAttribute(k_stage_f32<Q, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+                    if (e != cudaSuccess) return e;
+                    *attr = dyn;
+                }
+                k_stage_f32<Q, 2, true><<<grid, EB * NS, dyn, s>>>(a);
+                return cudaGetLastError();
+            }
         }
-        if (C == 1) k_stage_f32<Q, 1, true><<<grid, EB * NS, dyn, s>>>(a);
-        else k_stage_f32<Q, 2, true><<<grid, EB * NS, dyn, s>>>(a);
+        return launch_stage_f32_curved(a, C, n_vblk, s);
     } else {
         if (C == 1) k_stage_f32<Q, 1, false><<<grid, EB * NS, 0, s>>>(a);
         else k_stage_f32<Q, 2, false><<<grid, EB * NS, 0, s>>>(a);
@@ -765,7 +715,7 @@ static bool any_specular(const MeshInfo &m) {
 bool stage_f32_tma_supported(const StageArgs<float> &a, int C, int depth) {
     if (a.fr.q != 2 && a.fr.q != 4) return false;          // element slabs of whole 16-byte units
     if (any_specular(a.mesh)) return false;                 // reflected traces are not staged
-    if (a.geo) return false;                                // curvilinear: the plain kernel only
+    if (a.geo) return false;                                // curvilinear: kernels of their own
     if (depth < 2 || depth > BGK_MAX_DEPTH) return false;
     if (!aligned16(a.f_s) || (a.a32 != 0.f && !aligned16(a.f_n))) return false;
     const size_t smem = a.fr.q == 2 ? (C == 1 ? tma_smem<2, 1>(depth) : tma_smem<2, 2>(depth))

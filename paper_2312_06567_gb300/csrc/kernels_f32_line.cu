@@ -242,19 +242,6 @@ __device__ __forceinline__ void add_pair(LineAcc<C> &A, LineAcc<C> &B, float cj1
     }
 }
 
-// Plane pairs of one point in shared memory: P[q] at P[q * n], errors at
-// P[(NQ + q) * n]; the same operations as IndexMoments::plane_add/end_line.
-template <int NQ>
-__device__ __forceinline__ void plane_add_s(float *P, int n, int q, float c, float sum, float err) {
-    float ps = P[q * n], pc = P[(NQ + q) * n];
-    const float pr = __fmul_rn(c, sum);
-    sum2(ps, pc, pr);
-    pc = __fadd_rn(pc, fmaf(c, sum, -pr));
-    pc = fmaf(c, err, pc);
-    P[q * n] = ps;
-    P[(NQ + q) * n] = pc;
-}
-
 // BC = false: the mesh is periodic in every direction, so no face is a
 // Dirichlet face and the per-direction tests drop out.
 template <int Q, int C, int EB, int NPT, bool BC>
@@ -935,7 +922,7 @@ bool stage_f32_line_supported(const StageArgs<float> &a, int C, int kind, int de
     if (Q == 3 && (kind != 0 || a.mesh.n[0] % 4 != 0)) return false;
     for (int f = 0; f < 6; ++f)
         if (a.mesh.specular[f]) return false;               // reflected traces are not staged
-    if (a.geo) return false;                                // curvilinear: the plain kernel only
+    if (a.geo) return false;                                // curvilinear: kernels of their own
     if (!aligned_to(a.f_s, 16) || (a.a32 != 0.f && !aligned_to(a.f_n, 16)) || !aligned_to(a.f_out, 16)) return false;
     size_t smem = 0;
     line_any(kind, false, a, C, 0, depth, nullptr, &smem);

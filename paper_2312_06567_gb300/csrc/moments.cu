@@ -38,29 +38,6 @@ __device__ __forceinline__ void plane_add2(float2 &P, float2 &Pe, float c, float
     Pe = __ffma2_rn(c2, e, Pe);
 }
 
-// the plane's seven sums (00 10 20 01 11 02 G) of one point into its index
-// moments J in the partials buffer, weight c, centred third index t
-__device__ __forceinline__ void plane_to_part(double *J, int P, double c, double t, const double (&d)[7], bool first) {
-    double o[11];
-#pragma unroll
-    for (int i = 0; i < 11; ++i) o[i] = first ? 0.0 : J[(size_t)i * P];
-    o[0] = fma(c, d[0], o[0]); o[1] = fma(c, d[1], o[1]); o[2] = fma(c, d[2], o[2]);
-    o[3] = fma(c, d[3], o[3]); o[4] = fma(c, d[4], o[4]); o[5] = fma(c, d[5], o[5]);
-    o[6] = fma(c * t, d[0], o[6]); o[7] = fma(c * t, d[1], o[7]); o[8] = fma(c * t, d[3], o[8]);
-    o[9] = fma(c * t * t, d[0], o[9]); o[10] = fma(c, d[6], o[10]);
-#pragma unroll
-    for (int i = 0; i < 11; ++i) J[(size_t)i * P] = o[i];
-}
-// index moments -> raw moments where they stand
-__device__ __forceinline__ void raw_in_place(double *J, int P, const VelGrid &vg, const double uc[3]) {
-    double Jv[11], m[BGK_NMOM];
-#pragma unroll
-    for (int i = 0; i < 11; ++i) Jv[i] = J[(size_t)i * P];
-    index_to_raw(Jv, vg, uc, m);
-#pragma unroll
-    for (int i = 0; i < BGK_NMOM; ++i) J[(size_t)i * P] = m[i];
-}
-
 // Raw moments of an FP32 state on the stepping path: lines' and planes' sums
 // as FP32 pairs, the stage epilogue's operations in its velocity order, so the
 // partials equal what an epilogue yields for the same values.  A thread takes

@@ -57,6 +57,42 @@ __device__ __forceinline__ void index_to_raw(const double J[11], const VelGrid &
     m[10] = W * J[10];
 }
 
+// the plane's seven sums (00 10 20 01 11 02 G) of one point into its index
+// moments J in the partials buffer, weight c, centred third index t
+__device__ __forceinline__ void plane_to_part(double *J, int P, double c, double t, const double (&d)[7], bool first) {
+    double o[11];
+#pragma unroll
+    for (int i = 0; i < 11; ++i) o[i] = first ? 0.0 : J[(size_t)i * P];
+    o[0] = fma(c, d[0], o[0]); o[1] = fma(c, d[1], o[1]); o[2] = fma(c, d[2], o[2]);
+    o[3] = fma(c, d[3], o[3]); o[4] = fma(c, d[4], o[4]); o[5] = fma(c, d[5], o[5]);
+    o[6] = fma(c * t, d[0], o[6]); o[7] = fma(c * t, d[1], o[7]); o[8] = fma(c * t, d[3], o[8]);
+    o[9] = fma(c * t * t, d[0], o[9]); o[10] = fma(c, d[6], o[10]);
+#pragma unroll
+    for (int i = 0; i < 11; ++i) J[(size_t)i * P] = o[i];
+}
+// index moments -> raw moments where they stand
+__device__ __forceinline__ void raw_in_place(double *J, int P, const VelGrid &vg, const double uc[3]) {
+    double Jv[11], m[BGK_NMOM];
+#pragma unroll
+    for (int i = 0; i < 11; ++i) Jv[i] = J[(size_t)i * P];
+    index_to_raw(Jv, vg, uc, m);
+#pragma unroll
+    for (int i = 0; i < BGK_NMOM; ++i) J[(size_t)i * P] = m[i];
+}
+
+// Plane pairs of one point in shared memory: P[q] at P[q * n], errors at
+// P[(NQ + q) * n]; the same operations as IndexMoments::plane_add/end_line.
+template <int NQ>
+__device__ __forceinline__ void plane_add_s(float *P, int n, int q, float c, float sum, float err) {
+    float ps = P[q * n], pc = P[(NQ + q) * n];
+    const float pr = __fmul_rn(c, sum);
+    sum2(ps, pc, pr);
+    pc = __fadd_rn(pc, fmaf(c, sum, -pr));
+    pc = fmaf(c, err, pc);
+    P[q * n] = ps;
+    P[(NQ + q) * n] = pc;
+}
+
 // The Runge--Kutta update (a + b) f + a (f^n - f) + c R of the mixed form,
 // with one rounding at the level of f: the two small terms are summed first
 // (their roundings are relative to themselves) and added to f last.  Adding

@@ -16,7 +16,7 @@ constexpr int WT = 256;
 template <typename T, int Q>
 __global__ void __launch_bounds__(WT) k_wall_density(const T *f, const T *fvec, const double *bcval,
                                                     const double *vtab, const int *wall_ef, int Ne, int Nu,
-                                                    int C, FROps fr, double *rho_w) {
+                                                    int C, FROps fr, double *rho_w, float2 *rho_w2) {
     constexpr int NS = Q * Q * Q, NF = Q * Q;
     __shared__ double red[WT / 32][2 * NF];
     __shared__ double nv[NF][3];
@@ -70,14 +70,17 @@ __global__ void __launch_bounds__(WT) k_wall_density(const T *f, const T *fvec, 
     if (threadIdx.x < NF) {
         double a = 0.0, b = 0.0;
         for (int w = 0; w < WT / 32; ++w) { a += red[w][threadIdx.x]; b += red[w][NF + threadIdx.x]; }
-        rho_w[((size_t)e * 6 + face) * NF + threadIdx.x] = b < 0.0 ? -a / b : 0.0;
+        const double r = b < 0.0 ? -a / b : 0.0;
+        const size_t o = ((size_t)e * 6 + face) * NF + threadIdx.x;
+        rho_w[o] = r;
+        if (rho_w2) rho_w2[o] = make_float2((float)r, (float)(r - (double)(float)r));
     }
 }
 
 template <typename T, int Q>
 cudaError_t launch_q(const T *f, const T *fvec, const double *bcval, const double *vtab, const int *wall_ef,
-                     int n_wall, int Ne, int Nu, int C, const FROps &fr, double *rho_w, cudaStream_t s) {
-    k_wall_density<T, Q><<<n_wall, WT, 0, s>>>(f, fvec, bcval, vtab, wall_ef, Ne, Nu, C, fr, rho_w);
+                     int n_wall, int Ne, int Nu, int C, const FROps &fr, double *rho_w, float2 *rho_w2, cudaStream_t s) {
+    k_wall_density<T, Q><<<n_wall, WT, 0, s>>>(f, fvec, bcval, vtab, wall_ef, Ne, Nu, C, fr, rho_w, rho_w2);
     return cudaGetLastError();
 }
 
@@ -86,18 +89,18 @@ cudaError_t launch_q(const T *f, const T *fvec, const double *bcval, const doubl
 template <typename T>
 cudaError_t launch_wall_density(const T *f, const T *fvec, const double *bcval, const double *vtab,
                                 const int *wall_ef, int n_wall, int q, int Ne, int Nu, int C, FROps fr,
-                                double *rho_w, cudaStream_t s) {
+                                double *rho_w, float2 *rho_w2, cudaStream_t s) {
     if (n_wall == 0) return cudaSuccess;
     switch (q) {
-        case 2: return launch_q<T, 2>(f, fvec, bcval, vtab, wall_ef, n_wall, Ne, Nu, C, fr, rho_w, s);
-        case 3: return launch_q<T, 3>(f, fvec, bcval, vtab, wall_ef, n_wall, Ne, Nu, C, fr, rho_w, s);
-        case 4: return launch_q<T, 4>(f, fvec, bcval, vtab, wall_ef, n_wall, Ne, Nu, C, fr, rho_w, s);
-        case 5: return launch_q<T, 5>(f, fvec, bcval, vtab, wall_ef, n_wall, Ne, Nu, C, fr, rho_w, s);
+        case 2: return launch_q<T, 2>(f, fvec, bcval, vtab, wall_ef, n_wall, Ne, Nu, C, fr, rho_w, rho_w2, s);
+        case 3: return launch_q<T, 3>(f, fvec, bcval, vtab, wall_ef, n_wall, Ne, Nu, C, fr, rho_w, rho_w2, s);
+        case 4: return launch_q<T, 4>(f, fvec, bcval, vtab, wall_ef, n_wall, Ne, Nu, C, fr, rho_w, rho_w2, s);
+        case 5: return launch_q<T, 5>(f, fvec, bcval, vtab, wall_ef, n_wall, Ne, Nu, C, fr, rho_w, rho_w2, s);
         default: return cudaErrorInvalidValue;
     }
 }
 
 template cudaError_t launch_wall_density<double>(const double *, const double *, const double *, const double *,
-                                                 const int *, int, int, int, int, int, FROps, double *, cudaStream_t);
+                                                 const int *, int, int, int, int, int, FROps, double *, float2 *, cudaStream_t);
 template cudaError_t launch_wall_density<float>(const float *, const float *, const double *, const double *,
-                                                const int *, int, int, int, int, int, FROps, double *, cudaStream_t);
+                                                const int *, int, int, int, int, int, FROps, double *, float2 *, cudaStream_t);
