@@ -1660,12 +1660,12 @@ bgk_status bgk_mlp_weights(bgk_ctx *ctx, float *buf, int load) {
     return BGK_OK;
 }
 
-// Upload x[n][9], t[n][5] (host) and run the training kernel over all n samples.
-static bgk_status mlp_batch_pass(bgk_ctx *ctx, const float *dx, const float *dt, const int *didx, int n,
+// The training kernel over all n samples (device arrays), sums into scratch.
+static bgk_status mlp_batch_pass(bgk_ctx *ctx, const float *dx, const float *dt, const int *didx, int n, void *scratch,
                                  int bf16) {
     MlpParams p{ctx->mlp_w, ctx->mlp_norm, nullptr};   // training rounds the master weights itself
     LaunchScope ls(ctx, BGK_K_OTHER);
-    CU(launch_mlp_train(p, dx, dt, didx, n, ctx->mlp_grad, ctx->mlp_loss, bf16, ctx->stream));
+    CU(launch_mlp_train(p, dx, dt, didx, n, scratch, bf16, ctx->stream));
     return BGK_OK;
 }
 
@@ -1679,19 +1679,21 @@ bgk_status bgk_mlp_grad(bgk_ctx *ctx, const float *x, const float *t, int n, int
     CU(cudaMallocAsync((void **)&dx, (size_t)n * MLP_IN * sizeof(float), ctx->stream));
     CU(cudaMallocAsync((void **)&dt, (size_t)n * MLP_OUT * sizeof(float), ctx->stream));
     CU(cudaMallocAsync((void **)&didx, (size_t)n * sizeof(int), ctx->stream));
+    void *scratch = nullptr;
+    CU(cudaMallocAsync(&scratch, mlp_train_scratch(n), ctx->stream));
     CU(cudaMemcpyAsync(dx, x, (size_t)n * MLP_IN * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
     CU(cudaMemcpyAsync(dt, t, (size_t)n * MLP_OUT * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
     CU(cudaMemcpyAsync(didx, idx.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaMemsetAsync(ctx->mlp_grad, 0, MLP_NPARAM * sizeof(float), ctx->stream));
     CU(cudaMemsetAsync(ctx->mlp_loss, 0, sizeof(double), ctx->stream));
-    bgk_status st = mlp_batch_pass(ctx, dx, dt, didx, n, bf16);
+    bgk_status st = mlp_batch_pass(ctx, dx, dt, didx, n, scratch, bf16);
     if (st) return st;
+    CU(launch_mlp_grad_sum(scratch, n, ctx->mlp_grad, ctx->mlp_loss, ctx->stream));
     CU(cudaMemcpyAsync(grad, ctx->mlp_grad, MLP_NPARAM * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
     CU(cudaMemcpyAsync(loss, ctx->mlp_loss, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     CU(cudaFreeAsync(dx, ctx->stream));
     CU(cudaFreeAsync(dt, ctx->stream));
     CU(cudaFreeAsync(didx, ctx->stream));
-    CU(cudaMemsetAsync(ctx->mlp_grad, 0, MLP_NPARAM * sizeof(float), ctx->stream));
+    CU(cudaFreeAsync(scratch, ctx->stream));
     CU(cudaStreamSynchronize(ctx->stream));
     return BGK_OK;
 }
@@ -1772,54 +1774,60 @@ bgk_status bgk_mlp_train(bgk_ctx *ctx, int epochs, int batch, float lr, unsigned
         for (int i = 0; i < fan[l][0] * fan[l][1]; ++i) w[off + i] = (float)(nd(rng) * sc);
         off += (size_t)fan[l][0] * fan[l][1] + fan[l][1];
     }
-    float *dx = nullptr, *dt = nullptr;
-    int *didx = nullptr;
-    CU(cudaMalloc(&dx, hx.size() * sizeof(float)));
-    CU(cudaMalloc(&dt, ht.size() * sizeof(float)));
-    CU(cudaMalloc(&didx, (size_t)n * sizeof(int)));
-    CU(cudaMemcpyAsync(dx, hx.data(), hx.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaMemcpyAsync(dt, ht.data(), ht.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
+    // one block of device memory: features, targets, the epoch's order, and the
+    // batch's gradient rows (given back at the end)
+    const size_t bx = hx.size() * sizeof(float), bt = ht.size() * sizeof(float), bi = ((size_t)n * sizeof(int) + 15) & ~(size_t)15;
+    char *dev = nullptr;
+    CU(cudaMallocAsync((void **)&dev, mlp_train_scratch(batch) + 8 + bx + bt + bi, ctx->stream));
+    struct Free {
+        void *p;
+        cudaStream_t s;
+        ~Free() { cudaFreeAsync(p, s); }
+    } release{dev, ctx->stream};
+    void *scratch = dev;
+    float *dx = (float *)(dev + ((mlp_train_scratch(batch) + 7) & ~(size_t)7)), *dt = dx + hx.size();
+    int *didx = (int *)(dt + ht.size());
+    CU(cudaMemcpyAsync(dx, hx.data(), bx, cudaMemcpyHostToDevice, ctx->stream));
+    CU(cudaMemcpyAsync(dt, ht.data(), bt, cudaMemcpyHostToDevice, ctx->stream));
     CU(cudaMemcpyAsync(ctx->mlp_w, w.data(), MLP_NPARAM * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
     CU(cudaMemcpyAsync(ctx->mlp_norm, norm.data(), MLP_NNORM * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
     CU(cudaMemsetAsync(ctx->mlp_m, 0, MLP_NPARAM * sizeof(float), ctx->stream));
     CU(cudaMemsetAsync(ctx->mlp_v, 0, MLP_NPARAM * sizeof(float), ctx->stream));
-    CU(cudaMemsetAsync(ctx->mlp_grad, 0, MLP_NPARAM * sizeof(float), ctx->stream));
     ctx->mlp_ready = true;
     std::vector<int> perm((size_t)n);
     for (long long i = 0; i < n; ++i) perm[i] = (int)i;
     const long long nbatch = n / batch;
     const long long total = (long long)epochs * nbatch;
     long long step = 0;
-    double last = 0.0;
     for (int ep = 0; ep < epochs; ++ep) {
         std::shuffle(perm.begin(), perm.end(), rng);
         CU(cudaMemcpyAsync(didx, perm.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice, ctx->stream));
         CU(cudaMemsetAsync(ctx->mlp_loss, 0, sizeof(double), ctx->stream));
         for (long long b = 0; b < nbatch; ++b) {
-            st = mlp_batch_pass(ctx, dx, dt, didx + b * batch, batch, bf16);
+            st = mlp_batch_pass(ctx, dx, dt, didx + b * batch, batch, scratch, bf16);
             if (st) break;
             ++step;
             const double frac = (double)(step - 1) / (double)std::max(1ll, total - 1);
             const float lr_t = (float)(lr * (0.1 + 0.45 * (1.0 + std::cos(M_PI * frac))));
             LaunchScope ls(ctx, BGK_K_OTHER);
-            cudaError_t e = launch_mlp_adam(ctx->mlp_w, ctx->mlp_m, ctx->mlp_v, ctx->mlp_grad, MLP_NPARAM, lr_t,
-                                            0.9f, 0.999f, 1e-8f, (int)step, ctx->stream);
+            cudaError_t e = launch_mlp_adam(ctx->mlp_w, ctx->mlp_m, ctx->mlp_v, scratch, batch, ctx->mlp_loss, lr_t, 0.9f,
+                                            0.999f, 1e-8f, (int)step, ctx->stream);
             if (e != cudaSuccess) { st = fail(ctx, BGK_ECUDA, "adam: %s", cudaGetErrorString(e)); break; }
         }
         if (st) break;
-        double ls_sum = 0.0;
-        cudaMemcpyAsync(&ls_sum, ctx->mlp_loss, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
-        cudaStreamSynchronize(ctx->stream);
-        last = ls_sum / (double)nbatch;
     }
+    // the last epoch's loss
+    double ls_sum = 0.0;
+    if (!st) {
+        CU(cudaMemcpyAsync(&ls_sum, ctx->mlp_loss, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+        CU(cudaStreamSynchronize(ctx->stream));
+    }
+    const double last = ls_sum / (double)nbatch;
     if (!st) {
         const cudaError_t e = launch_mlp_round(ctx->mlp_w, ctx->mlp_w16, MLP_NPARAM, ctx->stream);
         if (e != cudaSuccess) st = fail(ctx, BGK_ECUDA, "mlp round: %s", cudaGetErrorString(e));
     }
     cudaStreamSynchronize(ctx->stream);
-    cudaFree(dx);
-    cudaFree(dt);
-    cudaFree(didx);
     if (st) return st;
     if (final_loss) *final_loss = last;
     return BGK_OK;

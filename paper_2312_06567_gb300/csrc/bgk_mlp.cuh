@@ -73,10 +73,15 @@ __device__ __forceinline__ void mlp_infer_warp(const MlpParams &p, const float x
 // batched inference on tensor cores (mlp_tc.cu): delta[n][5] from raw features x[n][9]
 cudaError_t launch_mlp_infer_tc(const MlpParams &p, const float *x, long long n, float *delta, unsigned int *status,
                                 cudaStream_t s);
-size_t mlp_train_smem();
-cudaError_t launch_mlp_train(const MlpParams &p, const float *x, const float *t, const int *idx, int nb,
-                             float *grad, double *loss, int bf16, cudaStream_t s);
+// One batch's forward and backward pass (mlp.cu): per-block sums of the
+// gradients and the loss in scratch (mlp_train_scratch(nb) bytes), which
+// launch_mlp_adam turns into an update (the loss added to *loss) and
+// launch_mlp_grad_sum into the gradient.
+size_t mlp_train_scratch(int nb);
+cudaError_t launch_mlp_train(const MlpParams &p, const float *x, const float *t, const int *idx, int nb, void *scratch,
+                             int bf16, cudaStream_t s);
+cudaError_t launch_mlp_grad_sum(const void *scratch, int nb, float *grad, double *loss, cudaStream_t s);
 // w16[i] = w[i] rounded to BF16 (held in FP32), the copy BF16 inference reads
 cudaError_t launch_mlp_round(const float *w, float *w16, int n, cudaStream_t s);
-cudaError_t launch_mlp_adam(float *w, float *m, float *v, float *grad, int n, float lr, float b1, float b2,
-                            float eps, int step, cudaStream_t s);
+cudaError_t launch_mlp_adam(float *w, float *m, float *v, const void *scratch, int nb, double *loss, float lr, float b1,
+                            float b2, float eps, int step, cudaStream_t s);
