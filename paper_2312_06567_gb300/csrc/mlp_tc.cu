@@ -97,6 +97,28 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);      // a in the low half (lower address)
     return *reinterpret_cast<const uint32_t *>(&h);
 }
+// SiLU z / (1 + e^-z) of two values.  e^-z is held below 2^60 (beyond z = -41,
+// where the result is under 1e-16 either way), so that one reciprocal serves
+// both denominators, 1/d_a = d_b / (d_a d_b); each quotient is then corrected by
+// its exact remainder (Markstein 1990), which gives the correctly rounded
+// division but for rare last bits.  The IEEE divisions this replaces were half
+// of the kernel's instructions.
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float2 silu2(float2 z) {
+    const float2 e = make_float2(fminf(__expf(-z.x), 1.15292150460684698e18f), fminf(__expf(-z.y), 1.15292150460684698e18f));
+    const float2 d = __fadd2_rn(e, make_float2(1.f, 1.f));
+    const float r = rcp_approx(__fmul_rn(d.x, d.y));
+    const float2 r2 = __fmul2_rn(make_float2(r, r), make_float2(d.y, d.x));
+    const float2 q = __fmul2_rn(z, r2);
+    const float2 rem = __ffma2_rn(make_float2(-q.x, -q.y), d, z);
+    const float2 c = __ffma2_rn(rem, r2, q);
+    // an infinite z: the remainder is not a number, the quotient is the result
+    return make_float2(fabsf(z.x) <= 3.0e38f ? c.x : q.x, fabsf(z.y) <= 3.0e38f ? c.y : q.y);
+}
 // SiLU of 32 accumulator columns plus bias, rounded to BF16, written as four
 // 16-byte chunks of this thread's row of a K = 64 operand (chunks c0 .. c0+3)
 __device__ __forceinline__ void silu_row(const float (&z)[32], const float *bias, uint8_t *A, int row, int c0) {
@@ -106,8 +128,8 @@ __device__ __forceinline__ void silu_row(const float (&z)[32], const float *bias
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
             const int j = 8 * c + 2 * h;
-            const float a = z[j] + bias[j], b = z[j + 1] + bias[j + 1];
-            w[h] = pack_bf16(a / (1.f + __expf(-a)), b / (1.f + __expf(-b)));
+            const float2 v = silu2(__fadd2_rn(make_float2(z[j], z[j + 1]), *reinterpret_cast<const float2 *>(bias + j)));
+            w[h] = pack_bf16(v.x, v.y);
         }
         *reinterpret_cast<uint4 *>(A + kmaj(row, 8 * (c0 + c), 1024)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
@@ -123,20 +145,21 @@ __global__ void __launch_bounds__(TM, 4) k_mlp_infer_tc(MlpParams p, const float
     int *abort_flag = reinterpret_cast<int *>(tslot + 1);
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
 
-    // ---- weights as BF16 B operands (row = output unit, K = input unit) and the FP32 biases
+    // ---- weights as BF16 B operands (row = output unit, K = input unit; read
+    // along rows of the weight matrices) and the FP32 biases
     const float *W1 = p.w, *b1 = W1 + MLP_IN * MLP_H, *W2 = b1 + MLP_H, *b2 = W2 + MLP_H * MLP_H;
     const float *W3 = b2 + MLP_H, *b3 = W3 + MLP_H * MLP_OUT;
     for (int i = tid; i < MLP_H * K1; i += TM) {
-        const int n_ = i / K1, k = i % K1;
+        const int n_ = i % MLP_H, k = i / MLP_H;
         const float v = k < MLP_IN ? W1[k * MLP_H + n_] : 0.f;
         *reinterpret_cast<__nv_bfloat16 *>(sm + OFF_B1 + kmaj(n_, k, 256)) = __float2bfloat16_rn(v);
     }
     for (int i = tid; i < MLP_H * MLP_H; i += TM) {
-        const int n_ = i / MLP_H, k = i % MLP_H;
+        const int n_ = i % MLP_H, k = i / MLP_H;
         *reinterpret_cast<__nv_bfloat16 *>(sm + OFF_B2 + kmaj(n_, k, 1024)) = __float2bfloat16_rn(W2[k * MLP_H + n_]);
     }
     for (int i = tid; i < N3 * MLP_H; i += TM) {
-        const int n_ = i / MLP_H, k = i % MLP_H;
+        const int n_ = i % N3, k = i / N3;
         const float v = n_ < MLP_OUT ? W3[k * MLP_OUT + n_] : 0.f;
         *reinterpret_cast<__nv_bfloat16 *>(sm + OFF_B3 + kmaj(n_, k, 1024)) = __float2bfloat16_rn(v);
     }
@@ -189,6 +212,15 @@ __global__ void __launch_bounds__(TM, 4) k_mlp_infer_tc(MlpParams p, const float
     };
 
     const long long n_tiles = (n + TM - 1) / TM;
+    // the features of the next tile are requested a tile ahead (their latency
+    // was a third of the kernel's stalls)
+    float xr[MLP_IN];
+    auto request = [&](long long tile) {
+        const long long pt = tile * TM + tid;
+#pragma unroll
+        for (int f = 0; f < MLP_IN; ++f) xr[f] = tile < n_tiles && pt < n ? __ldg(x + pt * MLP_IN + f) : 0.f;
+    };
+    request(blockIdx.x);
     for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         const long long pt = tile * TM + tid;
         const bool live = pt < n;
@@ -199,8 +231,9 @@ __global__ void __launch_bounds__(TM, 4) k_mlp_infer_tc(MlpParams p, const float
             for (int f = 0; f < K1; ++f) xn[f] = 0.f;
             if (live) {
 #pragma unroll
-                for (int f = 0; f < MLP_IN; ++f) xn[f] = (__ldg(x + pt * MLP_IN + f) - xm[f]) / xs[f];
+                for (int f = 0; f < MLP_IN; ++f) xn[f] = (xr[f] - xm[f]) / xs[f];
             }
+            request(tile + gridDim.x);
 #pragma unroll
             for (int c = 0; c < 2; ++c)
                 *reinterpret_cast<uint4 *>(sm + OFF_A0 + kmaj(tid, 8 * c, 256)) =
