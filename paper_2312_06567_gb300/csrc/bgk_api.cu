@@ -1191,6 +1191,10 @@ bgk_status bgk_tune_stage(bgk_ctx *ctx, double dt, int reps, int *variant_out, i
     for (int v : {BGK_STAGE_ASYNC, BGK_STAGE_LINE, BGK_STAGE_LINE_WIDE, BGK_STAGE_HALF, BGK_STAGE_HALF_WIDE})
         for (int d : {2, 3, 4, 6, 8, 12, 16})
             if (stage_f32_variant_supported(sa, ctx->C, v, d)) cands.push_back({v, d});
+    // the line kernel reading directly, where that is what AUTO would run
+    int auto_depth = 0;
+    if (!ctx->curved && !stage_f32_auto_ring(sa, ctx->C, &auto_depth) && stage_f32_direct_supported(sa))
+        cands.push_back({BGK_STAGE_AUTO, ctx->stage_depth});
     cudaEvent_t ea = nullptr, eb = nullptr;
     CU(cudaEventCreate(&ea));
     CU(cudaEventCreate(&eb));
@@ -1245,7 +1249,7 @@ bgk_status bgk_tune_stage(bgk_ctx *ctx, double dt, int reps, int *variant_out, i
         set_blocking(ctx, pick_nb);
         // then the ring depths of that kernel again, at the chosen blocking
         // (the first search timed them at the default one); stage time only
-        if (!st && err == cudaSuccess && pick.v != BGK_STAGE_PLAIN) {
+        if (!st && err == cudaSuccess && pick.v != BGK_STAGE_PLAIN && pick.v != BGK_STAGE_AUTO) {
             StageArgs<float> sn = sp;
             sn.Kblk = ctx->Kblk;
             double best_d = 1e300;

@@ -299,6 +299,11 @@ bool stage_f32_tma_supported(const StageArgs<float> &a, int C, int depth);
 // line kernels: kind 0 line, 1 line_wide, 2 half, 3 half_wide
 bool stage_f32_line_supported(const StageArgs<float> &a, int C, int kind, int depth);
 cudaError_t launch_stage_f32_line(const StageArgs<float> &a, int C, int n_vblk, int kind, int depth, cudaStream_t s);
+// the line kernel without the copy ring (any order, element count and box face)
+bool stage_f32_direct_supported(const StageArgs<float> &a);
+// whether BGK_STAGE_AUTO takes the ring form on this mesh, and its depth
+bool stage_f32_auto_ring(const StageArgs<float> &a, int C, int *depth);
+cudaError_t launch_stage_f32_direct(const StageArgs<float> &a, int C, int n_vblk, cudaStream_t s);
 // any FP32 stage variant: is it available for these arguments
 bool stage_f32_variant_supported(const StageArgs<float> &a, int C, int variant, int depth);
 cudaError_t launch_maxwellian_f32(float *f, const double *q, const double *vtab, int Nu, int P, int C,

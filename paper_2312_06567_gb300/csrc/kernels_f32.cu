@@ -739,11 +739,16 @@ bool stage_f32_variant_supported(const StageArgs<float> &a, int C, int variant, 
 cudaError_t launch_stage_f32(const StageArgs<float> &a, int C, int n_vblk, int variant, int depth, cudaStream_t s) {
     if (variant >= BGK_STAGE_LINE && variant <= BGK_STAGE_HALF_WIDE)
         return launch_stage_f32_line(a, C, n_vblk, variant - BGK_STAGE_LINE, depth, s);
-    if ((variant == BGK_STAGE_AUTO || variant == BGK_STAGE_ASYNC) && stage_f32_tma_supported(a, C, depth)) {
+    if (variant == BGK_STAGE_ASYNC) {
+        if (!stage_f32_tma_supported(a, C, depth)) return cudaErrorInvalidValue;
         if (a.fr.q == 2) return C == 1 ? stage32_tma<2, 1>(a, n_vblk, depth, s) : stage32_tma<2, 2>(a, n_vblk, depth, s);
         return C == 1 ? stage32_tma<4, 1>(a, n_vblk, depth, s) : stage32_tma<4, 2>(a, n_vblk, depth, s);
     }
-    if (variant == BGK_STAGE_ASYNC) return cudaErrorInvalidValue;
+    if (variant == BGK_STAGE_AUTO && !a.geo) {
+        int d = 0;
+        if (stage_f32_auto_ring(a, C, &d)) return launch_stage_f32_line(a, C, n_vblk, 0, d, s);
+        if (stage_f32_direct_supported(a)) return launch_stage_f32_direct(a, C, n_vblk, s);
+    }
     switch (a.fr.q) {
         case 2: return stage32_q<2>(a, C, n_vblk, s);
         case 3: return stage32_q<3>(a, C, n_vblk, s);

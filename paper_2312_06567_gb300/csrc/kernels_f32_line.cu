@@ -77,6 +77,11 @@ __device__ __forceinline__ void ld_vec<3>(const float *p, float (&v)[3]) {
     v[0] = p[0]; v[1] = p[1]; v[2] = p[2];               // 4-byte aligned only
 }
 template <>
+__device__ __forceinline__ void ld_vec<5>(const float *p, float (&v)[5]) {
+#pragma unroll
+    for (int i = 0; i < 5; ++i) v[i] = p[i];
+}
+template <>
 __device__ __forceinline__ void ld_vec<1>(const float *p, float (&v)[1]) {
     v[0] = *p;
 }
@@ -93,6 +98,11 @@ __device__ __forceinline__ void st_vec<2>(float *p, const float (&v)[2]) {
 template <>
 __device__ __forceinline__ void st_vec<3>(float *p, const float (&v)[3]) {
     p[0] = v[0]; p[1] = v[1]; p[2] = v[2];
+}
+template <>
+__device__ __forceinline__ void st_vec<5>(float *p, const float (&v)[5]) {
+#pragma unroll
+    for (int i = 0; i < 5; ++i) p[i] = v[i];
 }
 template <>
 __device__ __forceinline__ void st_vec<1>(float *p, const float (&v)[1]) {
@@ -243,8 +253,15 @@ __device__ __forceinline__ void add_pair(LineAcc<C> &A, LineAcc<C> &B, float cj1
 }
 
 // BC = false: the mesh is periodic in every direction, so no face is a
-// Dirichlet face and the per-direction tests drop out.
-template <int Q, int C, int EB, int NPT, bool BC>
+// Dirichlet or specular face and the per-direction tests drop out.
+// RING = false: the same work per thread on values read straight from global
+// memory (no copies, no barriers, any run of elements): meshes whose element
+// runs are not whole 16-byte units (p = 4, p = 2 with odd rows) or short, and
+// those that reflect specularly (the mirrored velocity's trace is not staged).
+// Bit-identical too.  Against the plain kernel: p = 4, 588 for 1399 us per stage
+// (7500 points, 4608 velocities); specular p = 2, 1107 for 1987 us (5670 points,
+// 10,560 velocities; the reflected lines are read where they are used).
+template <int Q, int C, int EB, int NPT, bool BC, bool RING = true>
 __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, EB, NPT>::MINB) k_stage_f32_line(StageArgs<float> a, int S) {
     using SG = StageGeom<Q, C, EB>;
     using LG = LineGeom<Q, C, EB, NPT>;
@@ -252,7 +269,7 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
     constexpr int NCT = LG::NCT, NQ = LG::NQ, NH = LG::NH, NTT = Q * Q * NH;
     extern __shared__ __align__(128) float sbuf[];
     // [S][STAGE] copy ring | [NPT][2 NQ][NCT] plane pairs | 2S mbarriers | [S] release counts | [S] fills
-    float *Psm = sbuf + (size_t)S * STAGE;
+    float *Psm = sbuf + (RING ? (size_t)S * STAGE : 0);
     unsigned long long *bars = reinterpret_cast<unsigned long long *>(Psm + NPT * 2 * NQ * NCT);
     unsigned int *rel = reinterpret_cast<unsigned int *>(bars + 2 * S);
     unsigned int *fills = rel + S;
@@ -278,14 +295,14 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
     constexpr int NW = LG::NW;
     const int tid = threadIdx.x;
     RunGeom g;
-    g.init(a.mesh, EB, blockIdx.x);
+    if (RING) g.init(a.mesh, EB, blockIdx.x);
     const int vb = blockIdx.y;
     const int k0 = vb * a.Kblk, k1 = min(a.Nu, k0 + a.Kblk);
     const int nk = k1 - k0;
     const size_t slab = (size_t)a.P;
     const VelGrid &vg = a.vg;
     const int vn1 = vg.n[0], vn2 = vg.n[1], vn3 = vg.n[2];
-    if (tid == 0) {
+    if (RING && tid == 0) {
         ring_init(bars, S, NW);
         s_exited = 0;
         s_wait_ns = a.wait_ns;
@@ -322,11 +339,25 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
     const int r = rem / NH, h = rem - r * NH;
     const int jy = r % Q, kz = r / Q;
     const int i0 = NPT * h;                              // first node of this thread on its line
-    const bool active = l < g.nel;
-    const int pb = (g.e0 + l) * NS + Q * r + i0;         // point of local node i: pb + i
-    const int bcm = !BC ? 0
-                        : (l == 0 && g.xn0 < 0 ? 1 : 0) | (l == g.nel - 1 && g.xn1 < 0 ? 2 : 0) | (g.yn0 < 0 ? 4 : 0) |
-                              (g.yn1 < 0 ? 8 : 0) | (g.zn0 < 0 ? 16 : 0) | (g.zn1 < 0 ? 32 : 0);
+    const int el = RING ? g.e0 + l : min((int)blockIdx.x * EB + l, a.mesh.Ne - 1);      // the thread's element
+    const bool active = RING ? l < g.nel : (tid < EB * NTT && (int)blockIdx.x * EB + l < a.mesh.Ne);
+    const int pb = el * NS + Q * r + i0;                 // point of local node i: pb + i
+    // Dirichlet (and, without the ring, specular) faces of this element: bit
+    // 2d + side; without the ring the neighbours' offsets from the element
+    int bcm = !BC || !RING ? 0
+                           : (l == 0 && g.xn0 < 0 ? 1 : 0) | (l == g.nel - 1 && g.xn1 < 0 ? 2 : 0) | (g.yn0 < 0 ? 4 : 0) |
+                                 (g.yn1 < 0 ? 8 : 0) | (g.zn0 < 0 ? 16 : 0) | (g.zn1 < 0 ? 32 : 0);
+    int nbo[RING ? 1 : 6];
+    if constexpr (!RING) {
+        const int n1 = a.mesh.n[0], n2 = a.mesh.n[1], n3 = a.mesh.n[2];
+        const int ec[3] = {el % n1, (el / n1) % n2, el / (n1 * n2)}, es[3] = {1, n1, n1 * n2}, nn[3] = {n1, n2, n3};
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            nbo[2 * d] = ec[d] > 0 ? -es[d] : (nn[d] - 1) * es[d];
+            nbo[2 * d + 1] = ec[d] < nn[d] - 1 ? es[d] : -(nn[d] - 1) * es[d];
+            if (BC && !a.mesh.periodic[d]) bcm |= (ec[d] == 0 ? 1 << 2 * d : 0) | (ec[d] == nn[d] - 1 ? 2 << 2 * d : 0);
+        }
+    }
     const int own_off = (l + SG::PAD) * NS;              // own element within a component's stage region
     const int ln = Q * r;                                // own line within an element
     const bool mom = a.part != nullptr;
@@ -427,16 +458,29 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
         float jt1 = (float)(-jc[0]);
         for (int j1 = 0; j1 < vn1; ++j1, jt1 += 1.f) {
             const int k = kl + j1;
-            ok = __all_sync(0xffffffffu, mbar_wait_s(smem_u32(bars + slot), par, &s_wait_ns));
-            if (!ok) break;
+            if constexpr (RING) {
+                ok = __all_sync(0xffffffffu, mbar_wait_s(smem_u32(bars + slot), par, &s_wait_ns));
+                if (!ok) break;
+            }
             // every thread computes (an idle one, past the end of a short run,
             // on stage slots that hold no element of its own: finite or not,
             // its values are never stored), so the loop body does not diverge;
             // only the stores depend on `active`
             {
-                const float *st = sbuf + (size_t)slot * STAGE;
+                const float *st = RING ? sbuf + (size_t)slot * STAGE : a.f_s + (size_t)k * slab + (size_t)el * NS;
+                // component stride, and the offsets of the element, its upwind
+                // neighbours and f^n from st (f^n from a base of its own without the ring)
+                const size_t cstr = RING ? (size_t)PER_C : (size_t)a.Nu * slab;
                 const float u1 = su1c[j1].x;
                 const int sx = u1 > 0.f ? 0 : 1;
+                const int o_own = RING ? own_off : 0;
+                const int o_x = RING ? own_off + (sx ? NS : -NS) : nbo[RING ? 0 : sx] * NS;
+                const int o_y = RING ? (SLOTS + l) * NS : nbo[RING ? 0 : 2 + sy] * NS;
+                const int o_z = RING ? (SLOTS + EB + l) * NS : nbo[RING ? 0 : 4 + sz] * NS;
+                const float *fnb = RING ? st + (SLOTS + 2 * EB + l) * NS : a.f_n + (size_t)k * slab + (size_t)el * NS;
+                // specular faces: the element's own line at the mirrored velocity
+                // (direction d), with the weights of that outflow
+                auto mirrored = [&](int d) { return a.f_s + (size_t)mirror_velocity(k, d, vg.n) * slab + (size_t)el * NS; };
                 float outv[C][NPT];
                 if constexpr (C == 2 && NPT == Q && NPT % 2 == 1) {
                     // F and G of each point as one packed FP32 pair: every
@@ -444,16 +488,16 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                     // body below (x - y as fma(y, -1, x), the same rounding), so
                     // the results are the same bit for bit; the equilibrium is
                     // evaluated once for both
-                    const float *s0 = st, *s1 = st + PER_C;
+                    const float *s0 = st, *s1 = st + cstr;
                     auto ld2 = [&](int off, int n, float2 *v) {
                         for (int i = 0; i < n; ++i) v[i] = make_float2(s0[off + i], s1[off + i]);
                     };
                     float2 F2[NPT], div2[NPT];
-                    ld2(own_off + ln + i0, NPT, F2);
+                    ld2(o_own + ln + i0, NPT, F2);
                     // ---- first direction
                     {
                         float2 F[Q], t[NPT];
-                        ld2(own_off + ln, Q, F);
+                        ld2(o_own + ln, Q, F);
                         float2 dv[Q][Q];
 #pragma unroll
                         for (int i = 0; i < Q; ++i)
@@ -473,7 +517,7 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                         float2 dn[NPT];
                         if (!BC || !((bcm >> sx) & 1)) {
                             float2 NB[Q];
-                            ld2(own_off + (sx ? NS : -NS) + ln, Q, NB);
+                            ld2(o_x + ln, Q, NB);
                             float Lr[Q];
                             ld_vec<Q>(&slam[sx][0], Lr);
 #pragma unroll
@@ -483,6 +527,15 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
 #pragma unroll
                                 for (int i = 0; i < NPT; ++i)
                                     dn[i] = __ffma2_rn(dup2(Lr[j]), sub2(NB[j], F2[i]), dn[i]);
+                        } else if (!RING && a.mesh.specular[sx]) {
+                            const float *m0 = mirrored(0) + ln, *m1 = m0 + cstr;
+#pragma unroll
+                            for (int i = 0; i < NPT; ++i) dn[i] = __fmul2_rn(dup2(sdlam[1 - sx]), F2[i]);
+#pragma unroll
+                            for (int j = 0; j < Q; ++j)
+#pragma unroll
+                                for (int i = 0; i < NPT; ++i)
+                                    dn[i] = __ffma2_rn(dup2(slam[1 - sx][j]), sub2(make_float2(m0[j], m1[j]), F2[i]), dn[i]);
                         } else {
                             const float2 bv = make_float2((float)__ldg(a.bcval + ((size_t)(0 + sx) * C + 0) * a.Nu + k),
                                                           (float)__ldg(a.bcval + ((size_t)(0 + sx) * C + 1) * a.Nu + k));
@@ -513,7 +566,7 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                         for (int m = 1; m < Q; ++m) {
                             const int jq = (nd + m) % Q;
                             float2 Gv[NPT];
-                            ld2(own_off + (dd == 1 ? Q * (jq + Q * kz) : Q * (jy + Q * jq)) + i0, NPT, Gv);
+                            ld2(o_own + (dd == 1 ? Q * (jq + Q * kz) : Q * (jy + Q * jq)) + i0, NPT, Gv);
 #pragma unroll
                             for (int i = 0; i < NPT; ++i) t[i] = __ffma2_rn(dup2(Dr[m]), sub2(Gv[i], F2[i]), t[i]);
                         }
@@ -525,10 +578,20 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
 #pragma unroll
                             for (int jq = 0; jq < Q; ++jq) {
                                 float2 H[NPT];
-                                ld2((dd == 1 ? (SLOTS + l) * NS + Q * (jq + Q * kz) : (SLOTS + EB + l) * NS + Q * (jy + Q * jq)) + i0,
-                                    NPT, H);
+                                ld2((dd == 1 ? o_y + Q * (jq + Q * kz) : o_z + Q * (jy + Q * jq)) + i0, NPT, H);
 #pragma unroll
                                 for (int i = 0; i < NPT; ++i) dn[i] = __ffma2_rn(dup2(Lr[jq]), sub2(H[i], F2[i]), dn[i]);
+                            }
+                        } else if (!RING && a.mesh.specular[2 * dd + sd]) {
+                            const float *m0 = mirrored(dd) + i0, *m1 = m0 + cstr;
+#pragma unroll
+                            for (int i = 0; i < NPT; ++i) dn[i] = __fmul2_rn(dup2(sdlam[1 - sd]), F2[i]);
+#pragma unroll
+                            for (int jq = 0; jq < Q; ++jq) {
+                                const int o = dd == 1 ? Q * (jq + Q * kz) : Q * (jy + Q * jq);
+#pragma unroll
+                                for (int i = 0; i < NPT; ++i)
+                                    dn[i] = __ffma2_rn(dup2(slam[1 - sd][jq]), sub2(make_float2(m0[o + i], m1[o + i]), F2[i]), dn[i]);
                             }
                         } else {
                             const float2 bv = make_float2((float)__ldg(a.bcval + ((size_t)(2 * dd + sd) * C + 0) * a.Nu + k),
@@ -545,7 +608,10 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                     }
                     // ---- equilibrium (once for both), source and Runge--Kutta update
                     float2 FN[NPT];
-                    if (fa != 0.f) ld2((SLOTS + 2 * EB + l) * NS + ln + i0, NPT, FN);
+                    if (fa != 0.f) {
+#pragma unroll
+                        for (int i = 0; i < NPT; ++i) FN[i] = make_float2(fnb[ln + i0 + i], fnb[cstr + ln + i0 + i]);
+                    }
 #pragma unroll
                     for (int i = 0; i < NPT; ++i) {
                         const float c1 = __fsub_rn(u1, V1[i]);
@@ -568,14 +634,14 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                 } else {
 #pragma unroll
                 for (int c = 0; c < C; ++c) {
-                    const float *sc = st + c * PER_C;
+                    const float *sc = st + c * cstr;
                     float Fi[NPT];                       // this thread's nodes
-                    ld_vec<NPT>(sc + own_off + ln + i0, Fi);
+                    ld_vec<NPT>(sc + o_own + ln + i0, Fi);
                     float div[NPT];
                     // ---- first direction: the line itself and the upwind neighbour's line
                     {
                         float F[Q];
-                        ld_vec<Q>(sc + own_off + ln, F);
+                        ld_vec<Q>(sc + o_own + ln, F);
                         float t[NPT];
                         if (NPT == Q) {
                             // deviations formed once per pair: f_i - f_j = -(f_j - f_i) exactly
@@ -614,7 +680,7 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                         float dn[NPT];
                         if (!BC || !((bcm >> sx) & 1)) {
                             float NB[Q];
-                            ld_vec<Q>(sc + own_off + (sx ? NS : -NS) + ln, NB);
+                            ld_vec<Q>(sc + o_x + ln, NB);
                             float Lr[Q];
                             ld_vec<Q>(&slam[sx][0], Lr);
                             scale_vec<NPT>(dn, sdlam[sx], Fi);
@@ -624,6 +690,17 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
 #pragma unroll
                                 for (int i = 0; i < NPT; ++i) NBj[i] = NB[j];
                                 acc_dev<NPT>(dn, Lr[j], NBj, Fi);
+                            }
+                        } else if (!RING && a.mesh.specular[sx]) {
+                            float NB[Q];
+                            ld_vec<Q>(mirrored(0) + c * cstr + ln, NB);
+                            scale_vec<NPT>(dn, sdlam[1 - sx], Fi);
+#pragma unroll
+                            for (int j = 0; j < Q; ++j) {
+                                float NBj[NPT];
+#pragma unroll
+                                for (int i = 0; i < NPT; ++i) NBj[i] = NB[j];
+                                acc_dev<NPT>(dn, slam[1 - sx][j], NBj, Fi);
                             }
                         } else {
                             const float bv = (float)__ldg(a.bcval + ((size_t)(0 + sx) * C + c) * a.Nu + k);
@@ -647,7 +724,7 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                         for (int m = 1; m < Q; ++m) {
                             const int jp = (jy + m) % Q;             // the canonical order
                             float Gv[NPT];
-                            ld_vec<NPT>(sc + own_off + Q * (jp + Q * kz) + i0, Gv);
+                            ld_vec<NPT>(sc + o_own + Q * (jp + Q * kz) + i0, Gv);
                             acc_dev<NPT>(t, Dr[m], Gv, Fi);
                         }
                         if (!BC || !((bcm >> (2 + sy)) & 1)) {
@@ -657,8 +734,16 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
 #pragma unroll
                             for (int jp = 0; jp < Q; ++jp) {
                                 float H[NPT];
-                                ld_vec<NPT>(sc + (SLOTS + l) * NS + Q * (jp + Q * kz) + i0, H);
+                                ld_vec<NPT>(sc + o_y + Q * (jp + Q * kz) + i0, H);
                                 acc_dev<NPT>(dn, Lr[jp], H, Fi);
+                            }
+                        } else if (!RING && a.mesh.specular[2 + sy]) {
+                            scale_vec<NPT>(dn, sdlam[1 - sy], Fi);
+#pragma unroll
+                            for (int jp = 0; jp < Q; ++jp) {
+                                float H[NPT];
+                                ld_vec<NPT>(mirrored(1) + c * cstr + Q * (jp + Q * kz) + i0, H);
+                                acc_dev<NPT>(dn, slam[1 - sy][jp], H, Fi);
                             }
                         } else {
                             const float bv = (float)__ldg(a.bcval + ((size_t)(2 + sy) * C + c) * a.Nu + k);
@@ -682,7 +767,7 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                         for (int m = 1; m < Q; ++m) {
                             const int kp = (kz + m) % Q;             // the canonical order
                             float Gv[NPT];
-                            ld_vec<NPT>(sc + own_off + Q * (jy + Q * kp) + i0, Gv);
+                            ld_vec<NPT>(sc + o_own + Q * (jy + Q * kp) + i0, Gv);
                             acc_dev<NPT>(t, Dr[m], Gv, Fi);
                         }
                         if (!BC || !((bcm >> (4 + sz)) & 1)) {
@@ -692,8 +777,16 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
 #pragma unroll
                             for (int kp = 0; kp < Q; ++kp) {
                                 float H[NPT];
-                                ld_vec<NPT>(sc + (SLOTS + EB + l) * NS + Q * (jy + Q * kp) + i0, H);
+                                ld_vec<NPT>(sc + o_z + Q * (jy + Q * kp) + i0, H);
                                 acc_dev<NPT>(dn, Lr[kp], H, Fi);
+                            }
+                        } else if (!RING && a.mesh.specular[4 + sz]) {
+                            scale_vec<NPT>(dn, sdlam[1 - sz], Fi);
+#pragma unroll
+                            for (int jp = 0; jp < Q; ++jp) {
+                                float H[NPT];
+                                ld_vec<NPT>(mirrored(2) + c * cstr + Q * (jy + Q * jp) + i0, H);
+                                acc_dev<NPT>(dn, slam[1 - sz][jp], H, Fi);
                             }
                         } else {
                             const float bv = (float)__ldg(a.bcval + ((size_t)(4 + sz) * C + c) * a.Nu + k);
@@ -707,7 +800,7 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                     }
                     // ---- equilibrium, source and Runge--Kutta update
                     float FN[NPT];
-                    if (fa != 0.f) ld_vec<NPT>(sc + (SLOTS + 2 * EB + l) * NS + ln + i0, FN);
+                    if (fa != 0.f) ld_vec<NPT>(fnb + c * cstr + ln + i0, FN);
                     if constexpr (NPT % 2 == 0) {
                         // the same operations on pairs of points
                         const float2 u12 = dup2(u1);
@@ -764,31 +857,33 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                     }
                 }
             }
-            // release the slot; the warp that releases it last refills it with
-            // the velocity S ahead
-            __syncwarp();
-            int go = 0;
-            if (lane == 0) {
-                __threadfence_block();
-                if (atom_add_shared(&rel[slot], 1u) == NW - 1) {
-                    rel[slot] = 0;
+            if constexpr (RING) {
+                // release the slot; the warp that releases it last refills it with
+                // the velocity S ahead
+                __syncwarp();
+                int go = 0;
+                if (lane == 0) {
                     __threadfence_block();
-                    go = (k - k0) + S < *(volatile int *)&s_nfill ? 2 : 1;
+                    if (atom_add_shared(&rel[slot], 1u) == NW - 1) {
+                        rel[slot] = 0;
+                        __threadfence_block();
+                        go = (k - k0) + S < *(volatile int *)&s_nfill ? 2 : 1;
+                    }
                 }
-            }
-            // the whole warp refills the slot (warp-uniform operands; one
-            // elected lane issues the copies)
-            if (__shfl_sync(0xffffffffu, go, 0) == 2) {
-                // velocity k + S by its axis indices (velocity blocks are whole lines)
-                int i1 = j1 + S, i2 = j2, i3 = j3;
-                while (i1 >= vn1) {
-                    i1 -= vn1;
-                    if (++i2 == vn2) { i2 = 0; ++i3; }
+                // the whole warp refills the slot (warp-uniform operands; one
+                // elected lane issues the copies)
+                if (__shfl_sync(0xffffffffu, go, 0) == 2) {
+                    // velocity k + S by its axis indices (velocity blocks are whole lines)
+                    int i1 = j1 + S, i2 = j2, i3 = j3;
+                    while (i1 >= vn1) {
+                        i1 -= vn1;
+                        if (++i2 == vn2) { i2 = 0; ++i3; }
+                    }
+                    ring_issue_u<Q, C, EB, true, true>(a, g, sbuf, bars, slot, k + S, make_float3(su1c[i1].x, su2[i2], su3[i3]));
+                    if (lane == 0) fills[slot] += 1;
                 }
-                ring_issue_u<Q, C, EB, true, true>(a, g, sbuf, bars, slot, k + S, make_float3(su1c[i1].x, su2[i2], su3[i3]));
-                if (lane == 0) fills[slot] += 1;
+                if (++slot == S) { slot = 0; par ^= 1u; }
             }
-            if (++slot == S) { slot = 0; par ^= 1u; }
         }
         if (!ok) break;
         if (mom && active) {
@@ -900,6 +995,32 @@ cudaError_t line_dispatch3(int kind, bool launch, const StageArgs<float> &a, int
     return launch ? line_launch<3, C, 16, 3>(a, n_vblk, depth, s) : cudaSuccess;
 }
 
+// without the ring: any order and element count, a thread per first-axis line
+template <int Q, int C>
+cudaError_t line_direct(const StageArgs<float> &a, int n_vblk, cudaStream_t s) {
+    constexpr int EB = Q == 2 ? 16 : Q == 3 ? 16 : Q == 4 ? 8 : 5;
+    using LG = LineGeom<Q, C, EB, Q>;
+    constexpr size_t smem = (size_t)Q * 2 * LG::NQ * LG::NCT * sizeof(float);
+    static SmemLimit lim;
+    size_t *attr = lim.slot();
+    if (!attr) return cudaErrorInvalidDevice;
+    if (smem > *attr) {
+        cudaError_t e = cudaFuncSetAttribute(k_stage_f32_line<Q, C, EB, Q, false, false>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_stage_f32_line<Q, C, EB, Q, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)smem);
+        if (e != cudaSuccess) return e;
+        *attr = smem;
+    }
+    const dim3 grid((a.mesh.Ne + EB - 1) / EB, n_vblk);
+    if (a.mesh.periodic[0] && a.mesh.periodic[1] && a.mesh.periodic[2])
+        k_stage_f32_line<Q, C, EB, Q, false, false><<<grid, LG::NTHR, smem, s>>>(a, 0);
+    else
+        k_stage_f32_line<Q, C, EB, Q, true, false><<<grid, LG::NTHR, smem, s>>>(a, 0);
+    return cudaGetLastError();
+}
+
 cudaError_t line_any(int kind, bool launch, const StageArgs<float> &a, int C, int n_vblk, int depth, cudaStream_t s,
                      size_t *smem) {
     if (a.fr.q == 4) return C == 1 ? line_dispatch<4, 1>(kind, launch, a, n_vblk, depth, s, smem)
@@ -933,4 +1054,40 @@ cudaError_t launch_stage_f32_line(const StageArgs<float> &a, int C, int n_vblk, 
     if (!stage_f32_line_supported(a, C, kind, depth)) return cudaErrorInvalidValue;
     size_t smem = 0;
     return line_any(kind, true, a, C, n_vblk, depth, s, &smem);
+}
+
+// The line kernel's form for a mesh: on the ring, or reading directly (us per
+// stage on a GB300, ring / direct; the node-per-thread asynchronous kernel that
+// was the default before in brackets).  A ring pays where its runs are full:
+//   p = 3, 8 elements a row, 24^3 velocities           1253 / 1626 [3058]
+//   p = 3, 6 elements a row (runs of 4: 3/4 full)        501 /  602 [1107]
+//   p = 3, 2 elements a row                               61 /   57 [  84]
+//   p = 2, F and G, 32 elements a row (runs of 16)       909 / 1445 [2480]
+//   p = 2, 8 elements a row                              806 /  490 [1639]
+//   p = 1, 9 elements a row / 12, F and G     230 / 201 [573], 841 / 752 [2295]
+//   p = 1, 512 points, 8^3 velocities                     29 /   19 [  75]
+// so: at p = 3 from 5/8 full, at p = 2 from 3/4, at p = 1 never.  Two slots are
+// enough but for F and G at p = 3 (222 against 210 with three).
+bool stage_f32_auto_ring(const StageArgs<float> &a, int C, int *depth) {
+    const int Q = a.fr.q, eb = Q == 4 ? 4 : 16, n1 = a.mesh.n[0];
+    const int slots = (n1 + eb - 1) / eb * eb;           // elements the row's runs have room for
+    *depth = Q == 4 && C == 2 ? 3 : 2;
+    if (Q == 2 || Q == 5 || (Q == 4 ? 8 * n1 < 5 * slots : 4 * n1 < 3 * slots)) return false;
+    return stage_f32_line_supported(a, C, 0, *depth);
+}
+
+bool stage_f32_direct_supported(const StageArgs<float> &a) {
+    // vector loads of a line: whole 16-byte lines at p = 3, 8-byte ones at p = 1
+    const uintptr_t n = a.fr.q == 4 ? 16 : a.fr.q == 2 ? 8 : 4;
+    return !a.geo && a.eq32 && aligned_to(a.f_s, n) && (a.a32 == 0.f || aligned_to(a.f_n, n)) && aligned_to(a.f_out, n);
+}
+
+cudaError_t launch_stage_f32_direct(const StageArgs<float> &a, int C, int n_vblk, cudaStream_t s) {
+    switch (a.fr.q) {
+        case 2: return C == 1 ? line_direct<2, 1>(a, n_vblk, s) : line_direct<2, 2>(a, n_vblk, s);
+        case 3: return C == 1 ? line_direct<3, 1>(a, n_vblk, s) : line_direct<3, 2>(a, n_vblk, s);
+        case 4: return C == 1 ? line_direct<4, 1>(a, n_vblk, s) : line_direct<4, 2>(a, n_vblk, s);
+        case 5: return C == 1 ? line_direct<5, 1>(a, n_vblk, s) : line_direct<5, 2>(a, n_vblk, s);
+        default: return cudaErrorInvalidValue;
+    }
 }
