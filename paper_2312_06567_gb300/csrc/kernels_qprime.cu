@@ -144,15 +144,20 @@ struct PointState {
     float feat[MLP_IN];
 };
 
-// One thread: the point's moments (sum of the velocity-block partials) and
-// everything derived from them.
-__device__ __forceinline__ void point_prologue(const QPrimeArgs &a, int p, PointState &ps) {
-#pragma unroll
-    for (int j = 0; j < BGK_NMOM; ++j) ps.m[j] = 0.0;
-    for (int vb = 0; vb < a.n_vblk; ++vb) {
-#pragma unroll
-        for (int j = 0; j < BGK_NMOM; ++j) ps.m[j] += a.part[((size_t)vb * BGK_NMOM + j) * a.P + p];
-    }
+// Moment slot j of point p: the sum of the velocity-block partials, in order.
+// One thread per (slot, point): with one per point, the loads of a block were
+// 64 round trips of 11 values in a row (on a small grid of 64 velocity blocks a
+// tenth of the kernel).
+__device__ __forceinline__ double moment_slot(const QPrimeArgs &a, int p, int j) {
+    const double *q = a.part + (size_t)j * a.P + p;
+    double s = 0.0;
+#pragma unroll 8
+    for (int vb = 0; vb < a.n_vblk; ++vb) s += q[(size_t)vb * BGK_NMOM * a.P];
+    return s;
+}
+
+// One thread: everything derived from the point's moments ps.m.
+__device__ __forceinline__ void point_prologue(const QPrimeArgs &a, PointState &ps) {
     const double *m = ps.m;
     const GasInfo &gs = a.gas;
     const double rho = m[0];
@@ -995,10 +1000,12 @@ __device__ __forceinline__ void fused_pass(const QPrimeArgs &a, int lane, const 
 // point (QW warps take the batch's points in turn); the per-point algebra
 // (prologue, Newton step, correction fit, epilogue) runs one lane of warp 0
 // per point, so the FP64 work of a point issues once rather than on 32 lanes.
-constexpr int QB = 32;
+// QB: up to 32 points, whose algebra issues together on GB300's slow FP64 pipe (a
+// warp instruction takes 16 SM cycles whatever its active lanes); fewer where 32
+// would leave multiprocessors idle or half a wave empty (qprime_batch).
 constexpr int QW = 8;
 
-template <bool F32>
+template <bool F32, int QB>
 struct QPShared {
     using MT = typename std::conditional<F32, float, double>::type;
     PointState ps[QB];
@@ -1018,9 +1025,9 @@ struct QPShared {
 
 __device__ __forceinline__ Sym3 load_sym3(const double *t) { return Sym3{t[0], t[1], t[2], t[3], t[4], t[5]}; }
 
-template <bool F32>
-__global__ void __launch_bounds__(QB * QW, 2) k_qprime(QPrimeArgs a) {
-    __shared__ QPShared<F32> S;
+template <bool F32, int QB>
+__global__ void __launch_bounds__(32 * QW, 2) k_qprime(QPrimeArgs a) {
+    __shared__ QPShared<F32, QB> S;
     __shared__ float su1[BGK_MAXV];          // u1 of the first-axis velocity nodes (the same on every line)
     extern __shared__ double dyn_tab[];      // FP64 engine: [QW][n1][5] tables w1 ut1^m; FP32: [QW][2 n1] float4
     const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1029,8 +1036,11 @@ __global__ void __launch_bounds__(QB * QW, 2) k_qprime(QPrimeArgs a) {
     const double tol = F32 ? a.tol32 : a.tol;
     const double Pr = a.gas.Pr;
     for (int j = threadIdx.x; j < a.vg.n[0]; j += blockDim.x) su1[j] = __ldg(a.vtab32 + j).x;
-    // -- prologue: one lane per point
-    if (wib == 0 && lane < nb) point_prologue(a, p0 + lane, S.ps[lane]);
+    // -- prologue: the moments, one thread per slot and point; the rest, one lane per point
+    for (int i = threadIdx.x; i < QB * BGK_NMOM; i += 32 * QW)
+        if (i % QB < nb) S.ps[i % QB].m[i / QB] = moment_slot(a, p0 + i % QB, i / QB);
+    __syncthreads();
+    if (wib == 0 && lane < nb) point_prologue(a, S.ps[lane]);
     __syncthreads();
     // -- starting points: one warp per point (the network runs on the warp)
     for (int i = wib; i < nb; i += QW) {
@@ -1312,7 +1322,9 @@ __global__ void __launch_bounds__(QW * 32) k_qprime_tensor(QPrimeArgs a) {
     const int p = blockIdx.x * QW + wib;
     if (p >= a.P) return;                       // whole warps; no block barrier follows
     PointState &ps = S.ps[wib];
-    if (lane == 0) point_prologue(a, p, ps);
+    if (lane < BGK_NMOM) ps.m[lane] = moment_slot(a, p, lane);
+    __syncwarp();
+    if (lane == 0) point_prologue(a, ps);
     __syncwarp();
     // targets in the frame ut = u - U0, and the start: the d+2 solution's record
     double t[10], b[10];
@@ -1466,20 +1478,44 @@ cudaError_t allow_dyn_smem(K kernel, SmemLimit &lim, size_t bytes) {
     return cudaSuccess;
 }
 
-cudaError_t launch_qprime(const QPrimeArgs &a, bool fp32_sums, cudaStream_t s) {
-    const unsigned grid = (unsigned)((a.P + QB - 1) / QB);
-    if (fp32_sums) {
-        static SmemLimit lim32;
-        const size_t dyn = (size_t)QW * 2 * a.vg.n[0] * sizeof(float4);      // the fused pass's tables
-        const cudaError_t e = allow_dyn_smem(k_qprime<true>, lim32, dyn);
-        if (e != cudaSuccess) return e;
-        k_qprime<true><<<grid, QB * QW, dyn, s>>>(a);
-    } else {
-        static SmemLimit lim64;
-        const size_t dyn = (size_t)QW * a.vg.n[0] * 5 * sizeof(double);
-        const cudaError_t e = allow_dyn_smem(k_qprime<false>, lim64, dyn);
-        if (e != cudaSuccess) return e;
-        k_qprime<false><<<grid, QB * QW, dyn, s>>>(a);
-    }
+template <bool F32, int QB>
+static cudaError_t qprime_launch(const QPrimeArgs &a, cudaStream_t s) {
+    static SmemLimit lim;
+    // the fused pass's tables (FP32 sums), the engine's first-axis table (FP64)
+    const size_t dyn = F32 ? (size_t)QW * 2 * a.vg.n[0] * sizeof(float4) : (size_t)QW * a.vg.n[0] * 5 * sizeof(double);
+    const cudaError_t e = allow_dyn_smem(k_qprime<F32, QB>, lim, dyn);
+    if (e != cudaSuccess) return e;
+    k_qprime<F32, QB><<<(unsigned)((a.P + QB - 1) / QB), 32 * QW, dyn, s>>>(a);
     return cudaGetLastError();
+}
+
+// Points per block: the batch (a multiple of the eight warps) whose waves of
+// two blocks per multiprocessor cost least, a block of QB points costing its QB
+// passes and about six passes' worth of algebra.  512 points, 8^3 velocities:
+// 0.211 ms with 32, 0.109 ms with 8; 6912 points, 40^3: 2.31 ms with 32 (216
+// blocks on 304 places), 1.80 with 24; 13,824 points, 32^3: 1.79 and 1.53.
+static int qprime_batch(int P, int sms) {
+    int best = 32;
+    long long cost = -1;
+    for (int qb = 32; qb >= 8; qb -= 8) {
+        const long long blocks = (P + qb - 1) / qb, waves = (blocks + 2 * sms - 1) / (2 * sms);
+        if (cost < 0 || waves * (qb + 6) < cost) {
+            cost = waves * (qb + 6);
+            best = qb;
+        }
+    }
+    return best;
+}
+
+cudaError_t launch_qprime(const QPrimeArgs &a, bool fp32_sums, cudaStream_t s) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    switch (qprime_batch(a.P, sms)) {
+        case 8: return fp32_sums ? qprime_launch<true, 8>(a, s) : qprime_launch<false, 8>(a, s);
+        case 16: return fp32_sums ? qprime_launch<true, 16>(a, s) : qprime_launch<false, 16>(a, s);
+        case 24: return fp32_sums ? qprime_launch<true, 24>(a, s) : qprime_launch<false, 24>(a, s);
+        default: return fp32_sums ? qprime_launch<true, 32>(a, s) : qprime_launch<false, 32>(a, s);
+    }
 }
