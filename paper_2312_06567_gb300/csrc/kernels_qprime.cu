@@ -1237,45 +1237,37 @@ __device__ __forceinline__ void tensor_phi(int a, int &p1, int &p2, int &p3) {
     p1 = e1[a]; p2 = e2[a]; p3 = e3[a];
 }
 
-// Gaussian elimination with partial pivoting, N x N, compile-time indices.
-template <int N>
-__device__ __forceinline__ bool solve_n(double (&J)[N][N], double (&r)[N]) {
+// The 10x10 system J x = r of one point on a warp: lane i < 10 holds row i in
+// a[] and its right-hand side in r; Gauss--Jordan with partial pivoting over the
+// rows, the pivot row broadcast.  Component c of the solution goes to x[c]
+// (shared memory).  False if singular.  One lane's elimination took 254
+// registers and three times the FP64 instructions.
+__device__ __forceinline__ bool solve10_warp(double (&a)[10], double r, int lane, double *x) {
+    bool free_row = lane < 10;
+    int mine = -1;
 #pragma unroll
-    for (int c = 0; c < N; ++c) {
-        int piv = c;
-        double best = fabs(J[c][c]);
+    for (int c = 0; c < 10; ++c) {
+        const double v = fabs(a[c]);
+        // the largest |a[c]| among the rows not used yet, by its high word
+        const unsigned key = free_row && v > 0.0 ? (unsigned)__double2hiint(v) + 1u : 0u;
+        const unsigned best = __reduce_max_sync(0xffffffffu, key);
+        if (best == 0u) return false;                    // (warp-uniform)
+        const int piv = __ffs(__ballot_sync(0xffffffffu, key == best)) - 1;
+        const double inv = 1.0 / __shfl_sync(0xffffffffu, a[c], piv);
+        const double l = lane == piv ? 0.0 : a[c] * inv;
 #pragma unroll
-        for (int i = c + 1; i < N; ++i) {
-            const double v = fabs(J[i][c]);
-            if (v > best) { best = v; piv = i; }
-        }
-        if (!(best > 0.0)) return false;
+        for (int j = c + 1; j < 10; ++j) a[j] = fma(-l, __shfl_sync(0xffffffffu, a[j], piv), a[j]);
+        r = fma(-l, __shfl_sync(0xffffffffu, r, piv), r);
+        if (lane == piv) {
+            mine = c;
+            free_row = false;
+            r *= inv;                                    // later columns do not change a finished row's pivot
 #pragma unroll
-        for (int i = c + 1; i < N; ++i) {
-            if (i == piv) {
-#pragma unroll
-                for (int j = 0; j < N; ++j) {
-                    const double t = J[c][j]; J[c][j] = J[i][j]; J[i][j] = t;
-                }
-                const double t = r[c]; r[c] = r[i]; r[i] = t;
-            }
-        }
-        const double inv = 1.0 / J[c][c];
-#pragma unroll
-        for (int i = c + 1; i < N; ++i) {
-            const double l = J[i][c] * inv;
-#pragma unroll
-            for (int j = c + 1; j < N; ++j) J[i][j] = fma(-l, J[c][j], J[i][j]);
-            r[i] = fma(-l, r[c], r[i]);
+            for (int j = c + 1; j < 10; ++j) a[j] *= inv;
         }
     }
-#pragma unroll
-    for (int c = N - 1; c >= 0; --c) {
-        double sacc = r[c];
-#pragma unroll
-        for (int j = c + 1; j < N; ++j) sacc = fma(-J[c][j], r[j], sacc);
-        r[c] = sacc / J[c][c];
-    }
+    if (mine >= 0) x[mine] = r;
+    __syncwarp();
     return true;
 }
 
@@ -1304,20 +1296,32 @@ __device__ __forceinline__ bool tensor_from_b(const PointState &ps, const double
     return true;
 }
 
+template <bool F32>
 struct TensorShared {
+    using MT = typename std::conditional<F32, float, double>::type;
     PointState ps[QW];
     double par[QW][10];       // c0, U'(3), A(6)
-    double M[QW][35];
+    double db[QW][10];        // the Newton step
+    double t[QW][10];         // targets
+    MT M[QW][35];
+    int jidx[10][10];         // slot of the moment of phi_i phi_j
     int go[QW];
 };
 
 template <bool F32>
-__global__ void __launch_bounds__(QW * 32) k_qprime_tensor(QPrimeArgs a) {
-    __shared__ TensorShared S;
+__global__ void __launch_bounds__(QW * 32, 2) k_qprime_tensor(QPrimeArgs a) {
+    __shared__ TensorShared<F32> S;
     __shared__ float su1[BGK_MAXV];
     extern __shared__ double dyn_tab[];
     const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int j = threadIdx.x; j < a.vg.n[0]; j += blockDim.x) su1[j] = __ldg(a.vtab32 + j).x;
+    if (threadIdx.x < 100) {
+        const int i = threadIdx.x / 10, j = threadIdx.x % 10;
+        int a1, a2, a3, b1, b2, b3;
+        tensor_phi(i, a1, a2, a3);
+        tensor_phi(j, b1, b2, b3);
+        S.jidx[i][j] = midx(a1 + b1, a2 + b2, a3 + b3);
+    }
     __syncthreads();
     const int p = blockIdx.x * QW + wib;
     if (p >= a.P) return;                       // whole warps; no block barrier follows
@@ -1327,11 +1331,12 @@ __global__ void __launch_bounds__(QW * 32) k_qprime_tensor(QPrimeArgs a) {
     if (lane == 0) point_prologue(a, ps);
     __syncwarp();
     // targets in the frame ut = u - U0, and the start: the d+2 solution's record
-    double t[10], b[10];
+    double b[10];
     double res = 1.0e300;
     int it = 0;
     bool conv = false;
     if (lane == 0) {
+        double *t = S.t[wib];
         const double ip = 1.0 / a.gas.Pr;
         t[0] = ps.m[0];
         t[1] = ps.m[1] - ps.U0[0] * ps.m[0];
@@ -1354,78 +1359,77 @@ __global__ void __launch_bounds__(QW * 32) k_qprime_tensor(QPrimeArgs a) {
         const double *pr = S.par[wib];
         const Sym3 A{pr[4], pr[5], pr[6], pr[7], pr[8], pr[9]};
         const double x[5] = {0.0, pr[1], pr[2], pr[3], 0.0};
-        double M[35];
-        if (F32) {
-            Engine32 e32;
-            float Mf[35];
-            e32.moments(a.vg, ps, x, A, pr[0], lane, Mf);
+        {
+            typename TensorShared<F32>::MT M[35];
+            if constexpr (F32) {
+                Engine32 e32;
+                e32.moments(a.vg, ps, x, A, pr[0], lane, M);
+            } else {
+                e64.moments(a.vg, ps, x, A, pr[0], lane, M);
+            }
+            __syncwarp();                                // the last evaluation's rows have been read
+            if (lane == 0) {
 #pragma unroll
-            for (int j = 0; j < 35; ++j) M[j] = Mf[j];
-        } else {
-            e64.moments(a.vg, ps, x, A, pr[0], lane, M);
+                for (int j = 0; j < 35; ++j) S.M[wib][j] = M[j];
+            }
+            __syncwarp();
         }
+        // lane i < 10: row i of R = sum w phi g - t and J = sum w phi phi^T g
+        const int row = min(lane, 9);
+        double Jr[10];
+#pragma unroll
+        for (int j = 0; j < 10; ++j) Jr[j] = (double)S.M[wib][S.jidx[row][j]];
+        const double R = Jr[0] - S.t[wib][row];          // phi_0 = 1
+        double rs = fabs(R) * (row == 0 ? ps.sc_rho : row < 4 ? ps.sc_mom : 1.0 / (ps.rho * ps.theta));
+        if (!(rs >= 0.0)) rs = 1.0e300;                  // not a number
+        double r_mom = row >= 1 && row < 4 ? rs : 0.0, r_oth = row >= 1 && row < 4 ? 0.0 : rs;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {                // lanes 10..31 repeat row 9
+            r_mom = fmax(r_mom, __shfl_xor_sync(0xffffffffu, r_mom, o));
+            r_oth = fmax(r_oth, __shfl_xor_sync(0xffffffffu, r_oth, o));
+        }
+        res = fmax(r_mom, r_oth);
+        const double tol = F32 ? a.tol32 : a.tol;
+        double tol_mom = tol;
+        if (F32) {            // the momentum rows' FP32 floor, as in k_qprime
+            const double um = fmax(fabs(pr[1]), fmax(fabs(pr[2]), fabs(pr[3])));
+            tol_mom = fmax(tol, 8.0 * 0x1p-24 * um * sqrt(fmax(A.t11 + A.t22 + A.t33, 0.0) / 3.0));
+        }
+        // (lanes 0..15 hold the maxima over rows 0..9; lane 0 decides for all)
+        const bool done = __shfl_sync(0xffffffffu, (int)(r_oth <= tol && r_mom <= tol_mom), 0) != 0;
+        const bool num = __shfl_sync(0xffffffffu, (int)(res < 1.0e300), 0) != 0;
+        bool solved = false;
+        if (!done && it < a.max_iter && num) solved = solve10_warp(Jr, -R, lane, S.db[wib]);
         if (lane == 0) {
-#pragma unroll
-            for (int j = 0; j < 35; ++j) S.M[wib][j] = M[j];
-            double R[10], J[10][10];
-#pragma unroll
-            for (int i = 0; i < 10; ++i) {
-                int a1, a2, a3;
-                tensor_phi(i, a1, a2, a3);
-                R[i] = M[midx(a1, a2, a3)] - t[i];
-#pragma unroll
-                for (int j = 0; j < 10; ++j) {
-                    int b1, b2, b3;
-                    tensor_phi(j, b1, b2, b3);
-                    J[i][j] = M[midx(a1 + b1, a2 + b2, a3 + b3)];
-                }
-            }
-            const double sq = 1.0 / (ps.rho * ps.theta);
-            double r_mom = 0.0, r_oth = fabs(R[0]) * ps.sc_rho;
-#pragma unroll
-            for (int i = 1; i < 4; ++i) r_mom = fmax(r_mom, fabs(R[i]) * ps.sc_mom);
-#pragma unroll
-            for (int i = 4; i < 10; ++i) r_oth = fmax(r_oth, fabs(R[i]) * sq);
-            res = fmax(r_mom, r_oth);
-            const double tol = F32 ? a.tol32 : a.tol;
-            double tol_mom = tol;
-            if (F32) {        // the momentum rows' FP32 floor, as in k_qprime
-                const double um = fmax(fabs(pr[1]), fmax(fabs(pr[2]), fabs(pr[3])));
-                tol_mom = fmax(tol, 8.0 * 0x1p-24 * um * sqrt(fmax(A.t11 + A.t22 + A.t33, 0.0) / 3.0));
-            }
             bool go = false;
-            if (r_oth <= tol && r_mom <= tol_mom) {
+            if (done) {
                 conv = true;
-            } else if (it < a.max_iter && res == res) {
-                double db[10];
+            } else if (solved) {
+                const double *db = S.db[wib];
+                double lam = 1.0, bt[10], c0n = 0.0, Un[3];
+                Sym3 An;
+                bool ok = false;
+                for (int h = 0; h < 60 && !ok; ++h) {
 #pragma unroll
-                for (int i = 0; i < 10; ++i) db[i] = -R[i];
-                if (solve_n<10>(J, db)) {
-                    double lam = 1.0, bt[10], c0n = 0.0, Un[3];
-                    Sym3 An;
-                    bool ok = false;
-                    for (int h = 0; h < 60 && !ok; ++h) {
+                    for (int i = 0; i < 10; ++i) bt[i] = fma(lam, db[i], b[i]);
+                    ok = tensor_from_b(ps, bt, c0n, Un, An);
+                    if (!ok) lam *= 0.5;
+                }
+                if (ok) {
 #pragma unroll
-                        for (int i = 0; i < 10; ++i) bt[i] = fma(lam, db[i], b[i]);
-                        ok = tensor_from_b(ps, bt, c0n, Un, An);
-                        if (!ok) lam *= 0.5;
-                    }
-                    if (ok) {
-#pragma unroll
-                        for (int i = 0; i < 10; ++i) b[i] = bt[i];
-                        S.par[wib][0] = c0n;
-                        S.par[wib][1] = Un[0]; S.par[wib][2] = Un[1]; S.par[wib][3] = Un[2];
-                        S.par[wib][4] = An.t11; S.par[wib][5] = An.t22; S.par[wib][6] = An.t33;
-                        S.par[wib][7] = An.t12; S.par[wib][8] = An.t13; S.par[wib][9] = An.t23;
-                        ++it;
-                        go = true;
-                    }
+                    for (int i = 0; i < 10; ++i) b[i] = bt[i];
+                    S.par[wib][0] = c0n;
+                    S.par[wib][1] = Un[0]; S.par[wib][2] = Un[1]; S.par[wib][3] = Un[2];
+                    S.par[wib][4] = An.t11; S.par[wib][5] = An.t22; S.par[wib][6] = An.t33;
+                    S.par[wib][7] = An.t12; S.par[wib][8] = An.t13; S.par[wib][9] = An.t23;
+                    go = true;
                 }
             }
             S.go[wib] = go;
         }
         __syncwarp();
         if (!S.go[wib]) break;
+        ++it;
     }
     // the converged Gaussian: x = (rho', U', theta' = tr T'/3) for the record and qp
     const double *pr = S.par[wib];
