@@ -259,8 +259,12 @@ __device__ __forceinline__ void add_pair(LineAcc<C> &A, LineAcc<C> &B, float cj1
 // runs are not whole 16-byte units (p = 4, p = 2 with odd rows) or short, and
 // those that reflect specularly (the mirrored velocity's trace is not staged).
 // Bit-identical too.  Against the plain kernel: p = 4, 588 for 1399 us per stage
-// (7500 points, 4608 velocities); specular p = 2, 1107 for 1987 us (5670 points,
-// 10,560 velocities; the reflected lines are read where they are used).
+// (7500 points, 4608 velocities); specular p = 2, 829 for 1987 us (5670 points,
+// 10,560 velocities).  A reflecting face is no case of its own there: its upwind
+// operand is the element itself at the mirrored velocity, so the threads of a
+// warp differ in an address and a row of weights, not in a branch (1107 us with
+// a branch per direction).  On the ring the pointers would cost 1.6% (p = 2, F
+// and G), so it keeps offsets.
 template <int Q, int C, int EB, int NPT, bool BC, bool RING = true>
 __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, EB, NPT>::MINB) k_stage_f32_line(StageArgs<float> a, int S) {
     using SG = StageGeom<Q, C, EB>;
@@ -478,9 +482,29 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                 const int o_y = RING ? (SLOTS + l) * NS : nbo[RING ? 0 : 2 + sy] * NS;
                 const int o_z = RING ? (SLOTS + EB + l) * NS : nbo[RING ? 0 : 4 + sz] * NS;
                 const float *fnb = RING ? st + (SLOTS + 2 * EB + l) * NS : a.f_n + (size_t)k * slab + (size_t)el * NS;
-                // specular faces: the element's own line at the mirrored velocity
-                // (direction d), with the weights of that outflow
-                auto mirrored = [&](int d) { return a.f_s + (size_t)mirror_velocity(k, d, vg.n) * slab + (size_t)el * NS; };
+                // upwind operand of each direction: the neighbour, or at a specular
+                // face the element itself at the mirrored velocity, with the weights
+                // of that outflow (the other side's)
+                const float *px = st + o_x, *py = st + o_y, *pz = st + o_z;
+                int wx = sx, wy = sy, wz = sz, dirichlet = bcm;
+                if constexpr (BC && !RING) {
+                    const float *self = a.f_s + (size_t)el * NS;
+                    if ((bcm >> sx & 1) && a.mesh.specular[sx]) {
+                        px = self + (size_t)(kl + vn1 - 1 - j1) * slab;
+                        wx = 1 - sx;
+                        dirichlet &= ~(1 << sx);
+                    }
+                    if ((bcm >> (2 + sy) & 1) && a.mesh.specular[2 + sy]) {
+                        py = self + (size_t)(k + (vn2 - 1 - 2 * j2) * vn1) * slab;
+                        wy = 1 - sy;
+                        dirichlet &= ~(1 << (2 + sy));
+                    }
+                    if ((bcm >> (4 + sz) & 1) && a.mesh.specular[4 + sz]) {
+                        pz = self + ((size_t)k + (ptrdiff_t)(vn3 - 1 - 2 * j3) * vn1 * vn2) * slab;
+                        wz = 1 - sz;
+                        dirichlet &= ~(1 << (4 + sz));
+                    }
+                }
                 float outv[C][NPT];
                 if constexpr (C == 2 && NPT == Q && NPT % 2 == 1) {
                     // F and G of each point as one packed FP32 pair: every
@@ -515,27 +539,20 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                             }
                         }
                         float2 dn[NPT];
-                        if (!BC || !((bcm >> sx) & 1)) {
+                        if (!BC || !((dirichlet >> sx) & 1)) {
                             float2 NB[Q];
-                            ld2(o_x + ln, Q, NB);
+                            if constexpr (RING) ld2(o_x + ln, Q, NB);
+                            else
+                                for (int i = 0; i < Q; ++i) NB[i] = make_float2(px[ln + i], px[cstr + ln + i]);
                             float Lr[Q];
-                            ld_vec<Q>(&slam[sx][0], Lr);
+                            ld_vec<Q>(&slam[wx][0], Lr);
 #pragma unroll
-                            for (int i = 0; i < NPT; ++i) dn[i] = __fmul2_rn(dup2(sdlam[sx]), F2[i]);
+                            for (int i = 0; i < NPT; ++i) dn[i] = __fmul2_rn(dup2(sdlam[wx]), F2[i]);
 #pragma unroll
                             for (int j = 0; j < Q; ++j)
 #pragma unroll
                                 for (int i = 0; i < NPT; ++i)
                                     dn[i] = __ffma2_rn(dup2(Lr[j]), sub2(NB[j], F2[i]), dn[i]);
-                        } else if (!RING && a.mesh.specular[sx]) {
-                            const float *m0 = mirrored(0) + ln, *m1 = m0 + cstr;
-#pragma unroll
-                            for (int i = 0; i < NPT; ++i) dn[i] = __fmul2_rn(dup2(sdlam[1 - sx]), F2[i]);
-#pragma unroll
-                            for (int j = 0; j < Q; ++j)
-#pragma unroll
-                                for (int i = 0; i < NPT; ++i)
-                                    dn[i] = __ffma2_rn(dup2(slam[1 - sx][j]), sub2(make_float2(m0[j], m1[j]), F2[i]), dn[i]);
                         } else {
                             const float2 bv = make_float2((float)__ldg(a.bcval + ((size_t)(0 + sx) * C + 0) * a.Nu + k),
                                                           (float)__ldg(a.bcval + ((size_t)(0 + sx) * C + 1) * a.Nu + k));
@@ -570,28 +587,22 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
 #pragma unroll
                             for (int i = 0; i < NPT; ++i) t[i] = __ffma2_rn(dup2(Dr[m]), sub2(Gv[i], F2[i]), t[i]);
                         }
-                        if (!BC || !((bcm >> (2 * dd + sd)) & 1)) {
+                        if (!BC || !((dirichlet >> (2 * dd + sd)) & 1)) {
                             float Lr[Q];
-                            ld_vec<Q>(&slam[sd][0], Lr);
+                            ld_vec<Q>(&slam[dd == 1 ? wy : wz][0], Lr);
 #pragma unroll
-                            for (int i = 0; i < NPT; ++i) dn[i] = __fmul2_rn(dup2(cf.x), F2[i]);
+                            for (int i = 0; i < NPT; ++i) dn[i] = __fmul2_rn(dup2(RING ? cf.x : sdlam[dd == 1 ? wy : wz]), F2[i]);
 #pragma unroll
                             for (int jq = 0; jq < Q; ++jq) {
                                 float2 H[NPT];
-                                ld2((dd == 1 ? o_y + Q * (jq + Q * kz) : o_z + Q * (jy + Q * jq)) + i0, NPT, H);
+                                const int o = dd == 1 ? Q * (jq + Q * kz) : Q * (jy + Q * jq);
+                                if constexpr (RING) ld2((dd == 1 ? o_y : o_z) + o + i0, NPT, H);
+                                else {
+                                    const float *ph = (dd == 1 ? py : pz) + o + i0;
+                                    for (int i = 0; i < NPT; ++i) H[i] = make_float2(ph[i], ph[cstr + i]);
+                                }
 #pragma unroll
                                 for (int i = 0; i < NPT; ++i) dn[i] = __ffma2_rn(dup2(Lr[jq]), sub2(H[i], F2[i]), dn[i]);
-                            }
-                        } else if (!RING && a.mesh.specular[2 * dd + sd]) {
-                            const float *m0 = mirrored(dd) + i0, *m1 = m0 + cstr;
-#pragma unroll
-                            for (int i = 0; i < NPT; ++i) dn[i] = __fmul2_rn(dup2(sdlam[1 - sd]), F2[i]);
-#pragma unroll
-                            for (int jq = 0; jq < Q; ++jq) {
-                                const int o = dd == 1 ? Q * (jq + Q * kz) : Q * (jy + Q * jq);
-#pragma unroll
-                                for (int i = 0; i < NPT; ++i)
-                                    dn[i] = __ffma2_rn(dup2(slam[1 - sd][jq]), sub2(make_float2(m0[o + i], m1[o + i]), F2[i]), dn[i]);
                             }
                         } else {
                             const float2 bv = make_float2((float)__ldg(a.bcval + ((size_t)(2 * dd + sd) * C + 0) * a.Nu + k),
@@ -678,29 +689,18 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                             }
                         }
                         float dn[NPT];
-                        if (!BC || !((bcm >> sx) & 1)) {
+                        if (!BC || !((dirichlet >> sx) & 1)) {
                             float NB[Q];
-                            ld_vec<Q>(sc + o_x + ln, NB);
+                            ld_vec<Q>(px + c * cstr + ln, NB);
                             float Lr[Q];
-                            ld_vec<Q>(&slam[sx][0], Lr);
-                            scale_vec<NPT>(dn, sdlam[sx], Fi);
+                            ld_vec<Q>(&slam[wx][0], Lr);
+                            scale_vec<NPT>(dn, sdlam[wx], Fi);
 #pragma unroll
                             for (int j = 0; j < Q; ++j) {
                                 float NBj[NPT];
 #pragma unroll
                                 for (int i = 0; i < NPT; ++i) NBj[i] = NB[j];
                                 acc_dev<NPT>(dn, Lr[j], NBj, Fi);
-                            }
-                        } else if (!RING && a.mesh.specular[sx]) {
-                            float NB[Q];
-                            ld_vec<Q>(mirrored(0) + c * cstr + ln, NB);
-                            scale_vec<NPT>(dn, sdlam[1 - sx], Fi);
-#pragma unroll
-                            for (int j = 0; j < Q; ++j) {
-                                float NBj[NPT];
-#pragma unroll
-                                for (int i = 0; i < NPT; ++i) NBj[i] = NB[j];
-                                acc_dev<NPT>(dn, slam[1 - sx][j], NBj, Fi);
                             }
                         } else {
                             const float bv = (float)__ldg(a.bcval + ((size_t)(0 + sx) * C + c) * a.Nu + k);
@@ -727,23 +727,15 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                             ld_vec<NPT>(sc + o_own + Q * (jp + Q * kz) + i0, Gv);
                             acc_dev<NPT>(t, Dr[m], Gv, Fi);
                         }
-                        if (!BC || !((bcm >> (2 + sy)) & 1)) {
+                        if (!BC || !((dirichlet >> (2 + sy)) & 1)) {
                             float Lr[Q];
-                            ld_vec<Q>(&slam[sy][0], Lr);
-                            scale_vec<NPT>(dn, cf.x, Fi);
+                            ld_vec<Q>(&slam[wy][0], Lr);
+                            scale_vec<NPT>(dn, RING ? cf.x : sdlam[wy], Fi);
 #pragma unroll
                             for (int jp = 0; jp < Q; ++jp) {
                                 float H[NPT];
-                                ld_vec<NPT>(sc + o_y + Q * (jp + Q * kz) + i0, H);
+                                ld_vec<NPT>(py + c * cstr + Q * (jp + Q * kz) + i0, H);
                                 acc_dev<NPT>(dn, Lr[jp], H, Fi);
-                            }
-                        } else if (!RING && a.mesh.specular[2 + sy]) {
-                            scale_vec<NPT>(dn, sdlam[1 - sy], Fi);
-#pragma unroll
-                            for (int jp = 0; jp < Q; ++jp) {
-                                float H[NPT];
-                                ld_vec<NPT>(mirrored(1) + c * cstr + Q * (jp + Q * kz) + i0, H);
-                                acc_dev<NPT>(dn, slam[1 - sy][jp], H, Fi);
                             }
                         } else {
                             const float bv = (float)__ldg(a.bcval + ((size_t)(2 + sy) * C + c) * a.Nu + k);
@@ -770,23 +762,15 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                             ld_vec<NPT>(sc + o_own + Q * (jy + Q * kp) + i0, Gv);
                             acc_dev<NPT>(t, Dr[m], Gv, Fi);
                         }
-                        if (!BC || !((bcm >> (4 + sz)) & 1)) {
+                        if (!BC || !((dirichlet >> (4 + sz)) & 1)) {
                             float Lr[Q];
-                            ld_vec<Q>(&slam[sz][0], Lr);
-                            scale_vec<NPT>(dn, cf.x, Fi);
+                            ld_vec<Q>(&slam[wz][0], Lr);
+                            scale_vec<NPT>(dn, RING ? cf.x : sdlam[wz], Fi);
 #pragma unroll
                             for (int kp = 0; kp < Q; ++kp) {
                                 float H[NPT];
-                                ld_vec<NPT>(sc + o_z + Q * (jy + Q * kp) + i0, H);
+                                ld_vec<NPT>(pz + c * cstr + Q * (jy + Q * kp) + i0, H);
                                 acc_dev<NPT>(dn, Lr[kp], H, Fi);
-                            }
-                        } else if (!RING && a.mesh.specular[4 + sz]) {
-                            scale_vec<NPT>(dn, sdlam[1 - sz], Fi);
-#pragma unroll
-                            for (int jp = 0; jp < Q; ++jp) {
-                                float H[NPT];
-                                ld_vec<NPT>(mirrored(2) + c * cstr + Q * (jy + Q * jp) + i0, H);
-                                acc_dev<NPT>(dn, slam[1 - sz][jp], H, Fi);
                             }
                         } else {
                             const float bv = (float)__ldg(a.bcval + ((size_t)(4 + sz) * C + c) * a.Nu + k);
