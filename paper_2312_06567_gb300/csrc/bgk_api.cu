@@ -385,11 +385,11 @@ bgk_status run_stage(bgk_ctx *ctx, const void *fn, const void *fs, void *fo, dou
         LaunchScope lw(ctx, BGK_K_WALL);
         if (ctx->precision == BGK_FP64)
             CU(launch_wall_density<double>((const double *)fs, ctx->fvec, ctx->bcval, ctx->vtab, ctx->wall_ef,
-                                           ctx->n_wall, ctx->q, ctx->Ne, ctx->Nu, ctx->C, ctx->fr, ctx->rho_w,
+                                           ctx->n_wall, ctx->q, ctx->Ne, ctx->Nu, ctx->vg.n[0], ctx->C, ctx->fr, ctx->rho_w,
                                            nullptr, ctx->stream));
         else
             CU(launch_wall_density<float>((const float *)fs, ctx->fvec32, ctx->bcval, ctx->vtab, ctx->wall_ef,
-                                          ctx->n_wall, ctx->q, ctx->Ne, ctx->Nu, ctx->C, ctx->fr, ctx->rho_w,
+                                          ctx->n_wall, ctx->q, ctx->Ne, ctx->Nu, ctx->vg.n[0], ctx->C, ctx->fr, ctx->rho_w,
                                           ctx->rho_w2, ctx->stream));
     }
     LaunchScope ls(ctx, BGK_K_STAGE);

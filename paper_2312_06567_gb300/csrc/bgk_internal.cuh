@@ -276,7 +276,7 @@ bool build_curved_geometry(const FROps &fr, const int n[3], const int periodic[3
 // null) the same as FP32 pairs.
 template <typename T>
 cudaError_t launch_wall_density(const T *f, const T *fvec, const double *bcval, const double *vtab,
-                                const int *wall_ef, int n_wall, int q, int Ne, int Nu, int C, FROps fr,
+                                const int *wall_ef, int n_wall, int q, int Ne, int Nu, int n1, int C, FROps fr,
                                 double *rho_w, float2 *rho_w2, cudaStream_t s);
 
 // Launchers: the Q' solve and its tensor refinement (kernels_qprime.cu); the
