@@ -31,6 +31,17 @@ constexpr double kTwoPi = 6.283185307179586476925286766559;
 // exponent is below -650, where the recurrence would underflow).
 // The block holds EB whole elements; their values for the current velocity
 // are staged in shared memory (double buffered, one barrier per velocity).
+// The FP64 pipe bounds the kernel, so on the box the outer trace of a face
+// point, which all Q nodes of the line behind it use, is formed once, by one
+// thread, before the barrier (a sum of Q products per line instead of per node:
+// 9 of 41 FP64 instructions per value at p = 3).  One Taylor-Green stage, 4096
+// points at 24^3 velocities, p = 3: 5.90 -> 4.82 ms; 60 elements at 20^3, p = 1 /
+// 2 / 3 / 4: 0.53 / 1.93 / 3.22 / 7.06 -> 0.45 / 1.44 / 2.66 / 5.70 ms, with F and
+// G 0.86 / 2.86 / 6.26 / 13.9 -> 0.79 / 2.37 / 5.11 / 9.76 ms.
+// The register bound of the box forms: one block per multiprocessor asked for
+// (150 to 196 registers, nothing spilled) is faster up to p = 2 and at p = 3 with
+// F and G (p = 2: 1.44 against 1.65 ms), the compiler's own choice (127, 128)
+// at p = 3 (2.66 against 3.00) and p = 4 (5.70 against 6.43).
 //
 // Curvilinear elements (CURV): the transformed flux Ft_d = a_d f with
 // a_d = u . S^d at each node (S^d = J grad xi_d), per direction and line
@@ -43,13 +54,17 @@ constexpr double kTwoPi = 6.283185307179586476925286766559;
 // shared memory beside f.  Boundary faces: Dirichlet (prescribed exterior
 // Maxwellian), diffuse wall (rho_w times the wall Maxwellian), closed (no flux).
 template <int Q, int C, bool CURV>
-__global__ void __launch_bounds__(256) k_stage_f64(StageArgs<double> a) {
+__global__ void __launch_bounds__(256, !CURV && (Q <= 3 || (Q == 4 && C == 2)) ? 1 : 0) k_stage_f64(StageArgs<double> a) {
     constexpr int NS = Q * Q * Q;
     constexpr int EB = 256 / NS;
     constexpr int NT = EB * NS;
     __shared__ double sf[2][C][NT];
     __shared__ double sFt[CURV ? 2 : 1][CURV ? C : 1][CURV ? 3 : 1][CURV ? NT : 1];
     __shared__ double sD[2][Q][Q];        // Dt_L, Dt_R (CURV: D, unused)
+    // box: the outer traces of the block's face points, direction d of local
+    // element le at (le * 3 + d) * Q * Q + face point
+    constexpr int NTR = CURV ? 1 : EB * 3 * Q * Q, TRT = CURV ? 1 : (NTR + NT - 1) / NT;
+    __shared__ double sTr[CURV ? 1 : 2][CURV ? 1 : C][NTR];
     __shared__ double sdg[2][Q];          // g_L', g_R'
     __shared__ double sl[2][Q];           // neighbour trace weights: l(+1) for left inflow, l(-1) for right
     const int tid = threadIdx.x;
@@ -87,6 +102,27 @@ __global__ void __launch_bounds__(256) k_stage_f64(StageArgs<double> a) {
         en_[d][0] = ec[d] > 0 ? e - estr[d] : (a.mesh.periodic[d] ? e + (nn[d] - 1) * estr[d] : -1);
         en_[d][1] = ec[d] < nn[d] - 1 ? e + estr[d] : (a.mesh.periodic[d] ? e - (nn[d] - 1) * estr[d] : -1);
         base[d] = s - id[d] * stride[d];
+    }
+    // the face points this thread forms the outer trace of: their direction,
+    // first node and stride of the line, and the elements behind the two sides
+    // (-1: a boundary face, -2: no point)
+    int td[TRT], tb[TRT], te[TRT], tn[TRT][2];
+    if constexpr (!CURV) {
+#pragma unroll
+        for (int q = 0; q < TRT; ++q) {
+            const int r = tid + q * NT, d = (r / (Q * Q)) % 3, fp = r % (Q * Q);
+            te[q] = e0 + r / (3 * Q * Q);
+            td[q] = d;
+            tb[q] = d == 0 ? Q * fp : d == 1 ? fp % Q + Q * Q * (fp / Q) : fp;
+            tn[q][0] = tn[q][1] = -2;
+            if (r < NTR && te[q] < a.mesh.Ne) {
+                const int x = d == 0 ? te[q] % n1 : d == 1 ? (te[q] / n1) % n2 : te[q] / (n1 * n2);
+                const int es = d == 0 ? 1 : d == 1 ? n1 : n1 * n2, nd = d == 0 ? n1 : d == 1 ? n2 : n3;
+                const int per = a.mesh.periodic[d];
+                tn[q][0] = x > 0 ? te[q] - es : (per ? te[q] + (nd - 1) * es : -1);
+                tn[q][1] = x < nd - 1 ? te[q] + es : (per ? te[q] - (nd - 1) * es : -1);
+            }
+        }
     }
     // curvilinear: the node's metric vectors, 1/J and the face vectors of the
     // flux nodes on its three lines (faces 2d and 2d + 1)
@@ -167,6 +203,32 @@ __global__ void __launch_bounds__(256) k_stage_f64(StageArgs<double> a) {
                     }
                 }
             }
+            if constexpr (!CURV) {
+                const double ut[3] = {__ldg(vt + 0), u2, u3};
+#pragma unroll
+                for (int q = 0; q < TRT; ++q) {
+                    const int side = (td[q] == 0 ? ut[0] : td[q] == 1 ? ut[1] : ut[2]) > 0.0 ? 0 : 1;
+                    const int en = side ? tn[q][1] : tn[q][0], st = td[q] == 0 ? 1 : td[q] == 1 ? Q : Q * Q;
+                    if (en == -2) continue;
+                    // the neighbour's trace, or the element's own on this face at
+                    // the mirrored velocity (specular), or the exterior value
+                    const bool mirror = en < 0 && a.mesh.specular[2 * td[q] + side];
+                    const double *l = sl[mirror ? 1 - side : side];
+                    const size_t kk = mirror ? mirror_velocity(k, td[q], a.vg.n) : k;
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        double fp = 0.0;
+                        if (en >= 0 || mirror) {
+                            const double *nb = a.f_s + ((size_t)c * a.Nu + kk) * slab + (size_t)(mirror ? te[q] : en) * NS + tb[q];
+#pragma unroll
+                            for (int j = 0; j < Q; ++j) fp = fma(l[j], __ldg(nb + j * st), fp);
+                        } else {
+                            fp = __ldg(a.bcval + ((size_t)(2 * td[q] + side) * C + c) * a.Nu + k);
+                        }
+                        sTr[buf][c][tid + q * NT] = fp;
+                    }
+                }
+            }
             // equilibrium value at this velocity
             const float qf = q0f + (float)j1 * (D0f + ahf * (float)(j1 - 1));
             if (qf < -650.0f) {
@@ -244,25 +306,8 @@ __global__ void __launch_bounds__(256) k_stage_f64(StageArgs<double> a) {
                         double t = 0.0;
 #pragma unroll
                         for (int j = 0; j < Q; ++j) t = fma(sD[side][id[d]][j], own[j * stride[d]], t);
-                        const int en = side ? en_[d][1] : en_[d][0];
-                        double fp = 0.0;
-                        if (en >= e0 && en < e0 + EB) {
-                            const double *nb = sfc + (en - e0) * NS + base[d];
-#pragma unroll
-                            for (int j = 0; j < Q; ++j) fp = fma(sl[side][j], nb[j * stride[d]], fp);
-                        } else if (en >= 0) {
-                            const double *nb = fs + (size_t)en * NS + base[d];
-#pragma unroll
-                            for (int j = 0; j < Q; ++j) fp = fma(sl[side][j], __ldg(nb + j * stride[d]), fp);
-                        } else if (a.mesh.specular[2 * d + side]) {
-                            // the element's own trace on this face at the mirrored velocity
-                            const double *mr = a.f_s + ((size_t)c * a.Nu + mirror_velocity(k, d, a.vg.n)) * slab +
-                                               (size_t)e * NS + base[d];
-#pragma unroll
-                            for (int j = 0; j < Q; ++j) fp = fma(sl[1 - side][j], __ldg(mr + j * stride[d]), fp);
-                        } else {
-                            fp = __ldg(a.bcval + ((size_t)(2 * d + side) * C + c) * a.Nu + k);
-                        }
+                        const int fpi = d == 0 ? id[1] + Q * id[2] : (d == 1 ? id[0] + Q * id[2] : id[0] + Q * id[1]);
+                        const double fp = sTr[buf][c][(le * 3 + d) * Q * Q + fpi];
                         t = fma(sdg[side][id[d]], fp, t);
                         div = fma(sc[d], t, div);
                     }
