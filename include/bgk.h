@@ -287,8 +287,9 @@ BGK_API bgk_status bgk_test_ring_stall(bgk_ctx *ctx, int after, double wait_seco
 
 /* Autotune the mixed-form stage kernel on this context's own problem (the
  * launch configuration only; every kernel candidate computes the same values):
- * time the plain kernel and every supported asynchronous variant at every ring
- * depth (2, 3, 4, 6, 8, 12, 16), each over `reps` stages with f^n and the moment
+ * time the plain kernel, the default (variant 0) where it reads directly, and
+ * every supported asynchronous variant at every ring depth (2, 3, 4, 6, 8, 12,
+ * 16), each over `reps` stages with f^n and the moment
  * epilogue (time step dt), from the current state into a scratch buffer, and
  * keep the fastest (as bgk_set_stage_kernel would); then, for that kernel, time
  * Q' solve + stage at the velocity blockings from the current count to four
