@@ -467,22 +467,24 @@ __global__ void __launch_bounds__(MT, 4) k_entropy_f32(const float *f, VelGrid v
 #pragma unroll
             for (int i = 0; i < MCH; ++i) {
                 if (j0 + i >= vn1) continue;
-                const float cj = trap(j0 + i, vn1);
+                float2 cj = dup2(trap(j0 + i, vn1));
                 // outside the positive normal range: subnormal and infinite
-                // values by the FP64 log, anything else is counted
+                // values by the FP64 log, anything else is counted.  Their place
+                // in the pair is taken by 1 with weight zero: log_pair2(1) is
+                // -2.2e-16, not 0, which F as small as these would not hide
                 if ((__float_as_uint(F[i].x) - 0x00800000u) >= 0x7f000000u || (__float_as_uint(F[i].y) - 0x00800000u) >= 0x7f000000u) {
                     for (int q = 0; q < 2; ++q) {
                         const float v = q ? F[i].y : F[i].x;
                         if ((__float_as_uint(v) - 0x00800000u) < 0x7f000000u) continue;
-                        if (v > 0.f) h[q] = fma(c23 * (double)cj * (double)v, log((double)v), h[q]);
+                        if (v > 0.f) h[q] = fma(c23 * (double)(q ? cj.y : cj.x) * (double)v, log((double)v), h[q]);
                         else if (q == 0 || two) ++bad;
-                        if (q) F[i].y = 1.f;
-                        else F[i].x = 1.f;                       // ln 1 = 0: no term
+                        if (q) { F[i].y = 1.f; cj.y = 0.f; }
+                        else { F[i].x = 1.f; cj.x = 0.f; }
                     }
                 }
                 float2 ls, lc;
                 log_pair2(tab, F[i], ls, lc);
-                const float2 cF = __fmul2_rn(dup2(cj), F[i]);                        // exact
+                const float2 cF = __fmul2_rn(cj, F[i]);                              // exact
                 const float2 p = __fmul2_rn(cF, ls);
                 sum2x2(L, E, p);
                 E = __fadd2_rn(E, __ffma2_rn(cF, lc, __ffma2_rn(cF, ls, neg2(p))));

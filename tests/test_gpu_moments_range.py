@@ -1,0 +1,57 @@
+"""Moments, totals and entropy where the values' range matters (GPU): dilute
+FP32 states whose tails are subnormal."""
+import numpy as np
+import pytest
+
+from oracle import stage as ostage
+from paper_2312_06567_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lib(libbgk, cuda_device):
+    from paper_2312_06567_gb300 import bgk
+    return bgk
+
+
+def _quadrature(wl):
+    """Nodes u[Nu, 3], weights w[Nu] and the points' weights W[P], long double."""
+    u = W.velocity_nodes(wl).astype(np.longdouble)
+    w = np.ones(1, dtype=np.longdouble)
+    for d in range(3):                                    # k1 fastest
+        c = np.full(wl.vel_n[d], (np.longdouble(wl.vel_hi[d]) - wl.vel_lo[d]) / (wl.vel_n[d] - 1))
+        c[0] *= 0.5
+        c[-1] *= 0.5
+        w = (c[:, None] * w[None, :]).reshape(-1)
+    wq = ostage.problem_from_workload(wl).fr.wq
+    jac = np.prod([(wl.mesh_hi[d] - wl.mesh_lo[d]) / wl.mesh_n[d] / 2 for d in range(3)])
+    return u, w, np.tile(np.einsum("i,j,k->ijk", wq, wq, wq).reshape(-1), wl.n_elem) * jac
+
+
+def _entropy(wl, f):
+    """The entropy of f's first component and the sum of the magnitudes of its terms, long double."""
+    _, w, Wp = _quadrature(wl)
+    F = f[0].reshape(wl.n_vel, -1).astype(np.longdouble)
+    t = F * np.log(F)
+    return Wp @ (w @ t), Wp @ (w @ np.abs(t))
+
+
+@pytest.mark.parametrize("rho", [1.0, 1e-4, 1e-8, 1e-12])
+def test_entropy_of_a_dilute_state_with_subnormal_tails(lib, rho):
+    """A Maxwellian whose tail ends just above the smallest subnormal: every
+    value counts at its own scale.  Bound: the FP64 sums' 1e-13."""
+    wl = W.reduced(W.taylor_green_box(), mesh_n=(2, 1, 1), vel_n=(24, 24, 24)).replace(p=1)
+    peak = rho / (2 * np.pi) ** 1.5
+    reach = np.sqrt(2 * np.log(peak / 3e-45) / 3)         # |u_d| at the grid's corner
+    wl = wl.replace(vel_lo=(-reach,) * 3, vel_hi=(reach,) * 3)
+    u = W.velocity_nodes(wl)
+    theta = 1 + 0.01 * np.arange(wl.n_elem * wl.n_sol) / (wl.n_elem * wl.n_sol)
+    F = rho / (2 * np.pi * theta) ** 1.5 * np.exp(-0.5 * (u ** 2).sum(1)[:, None] / theta)
+    f = F.astype(np.float32).reshape(1, wl.n_vel, wl.n_elem, wl.n_sol)
+    assert f.min() > 0 and np.mean(f < np.finfo(np.float32).tiny) > 0.005
+    with lib.Solver(wl, lib.BGK_MIXED) as s:
+        s.set_state(f)
+        H = s.entropy()
+    want, mag = _entropy(wl, f)
+    assert abs(H - float(want)) <= 1e-13 * float(mag)
