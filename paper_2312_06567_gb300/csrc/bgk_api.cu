@@ -1783,11 +1783,25 @@ bgk_status bgk_mlp_train(bgk_ctx *ctx, int epochs, int batch, float lr, unsigned
     const size_t bx = hx.size() * sizeof(float), bt = ht.size() * sizeof(float), bi = ((size_t)n * sizeof(int) + 15) & ~(size_t)15;
     char *dev = nullptr;
     CU(cudaMallocAsync((void **)&dev, mlp_train_scratch(batch) + 8 + bx + bt + bi, ctx->stream));
-    struct Free {
+    // Copies from these host arrays may still be under way when a call returns
+    // (pageable memory is staged only where the GPU cannot read it in place):
+    // the epochs' orders alternate between two lists, an event after each
+    // upload says when its list may be shuffled again, and no exit leaves
+    // before the stream has finished with all of them.
+    std::vector<int> perm[2];
+    double ls_sum = 0.0;
+    struct Release {
         void *p;
         cudaStream_t s;
-        ~Free() { cudaFreeAsync(p, s); }
-    } release{dev, ctx->stream};
+        cudaEvent_t up[2];
+        ~Release() {
+            cudaStreamSynchronize(s);
+            cudaFreeAsync(p, s);
+            for (cudaEvent_t e : up)
+                if (e) cudaEventDestroy(e);
+        }
+    } release{dev, ctx->stream, {nullptr, nullptr}};
+    for (cudaEvent_t &e : release.up) CU(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     void *scratch = dev;
     float *dx = (float *)(dev + ((mlp_train_scratch(batch) + 7) & ~(size_t)7)), *dt = dx + hx.size();
     int *didx = (int *)(dt + ht.size());
@@ -1798,14 +1812,18 @@ bgk_status bgk_mlp_train(bgk_ctx *ctx, int epochs, int batch, float lr, unsigned
     CU(cudaMemsetAsync(ctx->mlp_m, 0, MLP_NPARAM * sizeof(float), ctx->stream));
     CU(cudaMemsetAsync(ctx->mlp_v, 0, MLP_NPARAM * sizeof(float), ctx->stream));
     ctx->mlp_ready = true;
-    std::vector<int> perm((size_t)n);
-    for (long long i = 0; i < n; ++i) perm[i] = (int)i;
+    for (auto &l : perm) l.resize((size_t)n);
+    for (long long i = 0; i < n; ++i) perm[1][i] = (int)i;
     const long long nbatch = n / batch;
     const long long total = (long long)epochs * nbatch;
     long long step = 0;
     for (int ep = 0; ep < epochs; ++ep) {
-        std::shuffle(perm.begin(), perm.end(), rng);
-        CU(cudaMemcpyAsync(didx, perm.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice, ctx->stream));
+        std::vector<int> &order = perm[ep & 1];
+        if (ep >= 2) CU(cudaEventSynchronize(release.up[ep & 1]));
+        order = perm[(ep & 1) ^ 1];                      // (only read here, as its upload does)
+        std::shuffle(order.begin(), order.end(), rng);
+        CU(cudaMemcpyAsync(didx, order.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice, ctx->stream));
+        CU(cudaEventRecord(release.up[ep & 1], ctx->stream));
         CU(cudaMemsetAsync(ctx->mlp_loss, 0, sizeof(double), ctx->stream));
         for (long long b = 0; b < nbatch; ++b) {
             st = mlp_batch_pass(ctx, dx, dt, didx + b * batch, batch, scratch, bf16);
@@ -1821,7 +1839,6 @@ bgk_status bgk_mlp_train(bgk_ctx *ctx, int epochs, int batch, float lr, unsigned
         if (st) break;
     }
     // the last epoch's loss
-    double ls_sum = 0.0;
     if (!st) {
         CU(cudaMemcpyAsync(&ls_sum, ctx->mlp_loss, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
         CU(cudaStreamSynchronize(ctx->stream));

@@ -70,3 +70,22 @@ def test_inference_at_tile_edges_and_large_arguments(lib, n, scale):
     err = np.abs((d - n32[18:23]) / n32[23:28] - y)
     assert np.all(np.isfinite(d))
     assert np.max(err) <= 5e-3 * max(1.0, np.abs(y).max())
+
+
+def test_training_repeats_for_a_seed(lib):
+    """Several batches and epochs over a list of samples larger than a copy that
+    is staged at once: each epoch takes its own order of the samples, so equal
+    seeds give equal weights and losses bit for bit, and another seed others."""
+    wl = W.reduced(W.taylor_green_box(), mesh_n=(6, 5, 5), vel_n=(8, 8, 8)).replace(p=3)
+    with lib.Solver(wl, lib.BGK_MIXED) as s:
+        s.set_state(W.random_anisotropic_state(wl, seed=2).astype(np.float32))
+        s.mlp_log(True, 3 * s.n_points)
+        s.step(wl.dt(), 1)
+        s.mlp_log(False)
+        runs = []
+        for seed in (5, 5, 5, 6):
+            loss = s.mlp_train(epochs=9, batch=900, lr=1e-3, seed=seed)
+            runs.append((loss, [p.tobytes() for p in s.mlp_weights()[0]]))
+    assert np.isfinite(runs[0][0])
+    assert runs[1] == runs[0] and runs[2] == runs[0]
+    assert runs[3][1] != runs[0][1]
