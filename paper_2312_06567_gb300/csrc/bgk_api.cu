@@ -263,8 +263,8 @@ bgk_status check_device_status(bgk_ctx *ctx) {
 bgk_status run_moments(bgk_ctx *ctx, const void *f, bool check = false) {
     LaunchScope ls(ctx, BGK_K_MOMENTS);
     if (ctx->precision == BGK_FP64) {
-        MomentArgs64 a{(const double *)f, ctx->part, ctx->Nu, ctx->P, ctx->Kblk, ctx->C};
-        CU(launch_moments_f64(a, ctx->vg, ctx->n_vblk, ctx->stream));
+        MomentArgs64 a{(const double *)f, ctx->part, ctx->vtab, ctx->Nu, ctx->P, ctx->Kblk, ctx->C};
+        CU(launch_moments_f64(a, ctx->vg, ctx->n_vblk, check, ctx->stream));
     } else {
         CU(launch_moments_f32((const float *)f, ctx->part, ctx->vtab, ctx->vg, ctx->Nu, ctx->P, ctx->Kblk, ctx->C,
                               ctx->n_vblk, check, ctx->stream));

@@ -258,6 +258,7 @@ struct QPrimeArgs {
 struct MomentArgs64 {
     const double *f;
     double *part;
+    const double *vtab;
     int Nu, P, Kblk, C;
 };
 
@@ -312,8 +313,8 @@ cudaError_t launch_macro(const double *mom, double *out, int P, const MeshInfo &
                          const GasInfo &gas, const double face_rho[6], const double *geo, cudaStream_t s);
 // Moments, entropy and totals of a stored state (moments.cu).  check (the
 // diagnostic entry points): the FP32 state's lines fold in FP64, and a point
-// whose sums are not finite is summed again in FP64 throughout.
-cudaError_t launch_moments_f64(const MomentArgs64 &a, const VelGrid &vg, int n_vblk, cudaStream_t s);
+// whose sums are not finite (either precision) is summed again directly.
+cudaError_t launch_moments_f64(const MomentArgs64 &a, const VelGrid &vg, int n_vblk, bool check, cudaStream_t s);
 cudaError_t launch_moments_f32(const float *f, double *part, const double *vtab, const VelGrid &vg, int Nu, int P,
                                int Kblk, int C, int n_vblk, bool check, cudaStream_t s);
 // out[j][p] = sum over velocity blocks of part[vb][j][p]: a shard's partial raw

@@ -270,9 +270,11 @@ __global__ void __launch_bounds__(MT, 2) k_moments_f32_diag(const float *f, doub
 }
 
 // The diagnostic entry points' second look: partials that are not finite (an
-// infinity or NaN in the state, or FP32 sums out of range) are summed again
-// in FP64, which keeps an infinite or huge value's moments what they are.
-__global__ void __launch_bounds__(MT) k_moments_redo(const float *f, double *part, const double *vtab, int Nu, int P,
+// infinity or NaN in the state, or sums out of range) are summed again directly
+// in FP64: sums over centred indices make NaN of an infinite value (0 times it,
+// or its difference in index_to_raw), which keeps its moments infinite here.
+template <typename T>
+__global__ void __launch_bounds__(MT) k_moments_redo(const T *f, double *part, const double *vtab, int Nu, int P,
                                                      int Kblk, int C) {
     const int p = blockIdx.x * MT + threadIdx.x, vb = blockIdx.y;
     if (p >= P) return;
@@ -604,10 +606,13 @@ __global__ void k_totals_sum(const double *blk, int n, double *out) {
 
 }  // namespace
 
-cudaError_t launch_moments_f64(const MomentArgs64 &a, const VelGrid &vg, int n_vblk, cudaStream_t s) {
+cudaError_t launch_moments_f64(const MomentArgs64 &a, const VelGrid &vg, int n_vblk, bool check, cudaStream_t s) {
     dim3 grid((a.P + MT - 1) / MT, n_vblk);
     if (a.C == 1) k_moments_f64<1><<<grid, MT, 0, s>>>(a.f, a.part, vg, a.Nu, a.P, a.Kblk);
     else k_moments_f64<2><<<grid, MT, 0, s>>>(a.f, a.part, vg, a.Nu, a.P, a.Kblk);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || !check) return e;
+    k_moments_redo<double><<<grid, MT, 0, s>>>(a.f, a.part, a.vtab, a.Nu, a.P, a.Kblk, a.C);
     return cudaGetLastError();
 }
 
@@ -623,7 +628,7 @@ cudaError_t launch_moments_f32(const float *f, double *part, const double *vtab,
     else k_moments_f32_diag<2><<<grid, MT, 0, s>>>(f, part, vg, Nu, P, Kblk);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_moments_redo<<<dim3((P + MT - 1) / MT, n_vblk), MT, 0, s>>>(f, part, vtab, Nu, P, Kblk, C);
+    k_moments_redo<float><<<dim3((P + MT - 1) / MT, n_vblk), MT, 0, s>>>(f, part, vtab, Nu, P, Kblk, C);
     return cudaGetLastError();
 }
 

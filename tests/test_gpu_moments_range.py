@@ -1,5 +1,5 @@
 """Moments, totals and entropy where the values' range matters (GPU): dilute
-FP32 states whose tails are subnormal."""
+FP32 states whose tails are subnormal, infinite values."""
 import numpy as np
 import pytest
 
@@ -55,3 +55,28 @@ def test_entropy_of_a_dilute_state_with_subnormal_tails(lib, rho):
         H = s.entropy()
     want, mag = _entropy(wl, f)
     assert abs(H - float(want)) <= 1e-13 * float(mag)
+
+
+@pytest.mark.parametrize("delta", [0.0, 2.0])
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_an_infinite_value_makes_its_points_moments_and_the_energy_infinite(lib, prec, delta):
+    """At a velocity with no zero component, on a grid with a plane u_d = 0 in
+    each direction: the moments are infinite with the sign of their weight, as a
+    direct sum has them; the other points keep theirs."""
+    wl = W.reduced(W.taylor_green_box(), mesh_n=(3, 1, 1), vel_n=(9, 5, 7)).replace(p=2, delta=delta)
+    dt = np.float64 if prec == "fp64" else np.float32
+    f = W.random_anisotropic_state(wl, seed=4).astype(dt)
+    k, at = 7 + 9 * (1 + 5 * 2), 1 * wl.n_sol + 3
+    u = W.velocity_nodes(wl)[k]
+    assert np.all(u != 0)
+    with lib.Solver(wl, lib.BGK_FP64 if prec == "fp64" else lib.BGK_MIXED) as s:
+        s.set_state(f)
+        m0 = s.moments()
+        f[0, k, 1, 3] = np.inf
+        s.set_state(f)
+        m, t = s.moments(), s.totals()
+    psi = [1, u[0], u[1], u[2], u[0] ** 2, u[1] ** 2, u[2] ** 2, u[0] * u[1], u[0] * u[2], u[1] * u[2]]
+    assert np.array_equal(m[at, :10], np.inf * np.sign(psi))
+    assert abs(m[at, 10] - m0[at, 10]) <= 1e-14 * m0[at, 10]
+    assert np.array_equal(np.delete(m, at, 0), np.delete(m0, at, 0))
+    assert t[0] == np.inf and t[4] == np.inf and np.array_equal(t[1:4], np.inf * np.sign(u))
