@@ -1,5 +1,6 @@
 """Moments, totals and entropy where the values' range matters (GPU): dilute
-FP32 states whose tails are subnormal, infinite values."""
+FP32 states whose tails are subnormal, infinite values, velocity grids far
+from centred on the gas."""
 import numpy as np
 import pytest
 
@@ -80,3 +81,35 @@ def test_an_infinite_value_makes_its_points_moments_and_the_energy_infinite(lib,
     assert abs(m[at, 10] - m0[at, 10]) <= 1e-14 * m0[at, 10]
     assert np.array_equal(np.delete(m, at, 0), np.delete(m0, at, 0))
     assert t[0] == np.inf and t[4] == np.inf and np.array_equal(t[1:4], np.inf * np.sign(u))
+
+
+def _moments(wl, f):
+    """m[P, 11] and the sums of magnitudes that scale its errors, long double."""
+    u, w, _ = _quadrature(wl)
+    psi = [np.ones_like(w), u[:, 0], u[:, 1], u[:, 2], u[:, 0] ** 2, u[:, 1] ** 2, u[:, 2] ** 2, u[:, 0] * u[:, 1],
+           u[:, 0] * u[:, 2], u[:, 1] * u[:, 2]]
+    F = f[0].reshape(wl.n_vel, -1).astype(np.longdouble)
+    G = f[1].reshape(wl.n_vel, -1).astype(np.longdouble) if wl.n_comp == 2 else 0 * F
+    return np.stack([(w * s) @ F for s in psi] + [w @ G], axis=1), np.stack([(w * abs(s)) @ F for s in psi] + [w @ G], axis=1)
+
+
+@pytest.mark.parametrize("delta", [0.0, 2.0])
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("lo,hi", [(-2.0, 60.0), (0.0, 40.0), (3.0, 30.0), (-31.0, -1.0)])
+def test_moments_on_grids_far_from_centred(lib, lo, hi, prec, delta):
+    """Velocity grids whose middle lies many thermal speeds from the gas.  Bound:
+    FP64 sums over n terms, (16 + 2 sqrt n) ulp of the sum of magnitudes."""
+    wl = W.reduced(W.taylor_green_box(), mesh_n=(2, 1, 1), vel_n=(64, 9, 8)).replace(p=1, delta=delta)
+    wl = wl.replace(vel_lo=(lo, -3.0, lo), vel_hi=(hi, 3.0, hi))
+    u = W.velocity_nodes(wl)
+    c = np.array([min(max(0.0, lo + 1.0), hi - 1.0), 0.0, min(max(0.0, lo + 1.0), hi - 1.0)])
+    rng = np.random.default_rng(1)
+    P = wl.n_elem * wl.n_sol
+    F = np.exp(-0.5 * ((u[:, None, :] - c - 0.1 * rng.standard_normal((P, 3))) ** 2).sum(-1) / 0.4)
+    f = np.stack([F, 0.4 * F])[:wl.n_comp].reshape(wl.n_comp, wl.n_vel, wl.n_elem, wl.n_sol)
+    f = np.maximum(f, 1e-30).astype(np.float64 if prec == "fp64" else np.float32)
+    with lib.Solver(wl, lib.BGK_FP64 if prec == "fp64" else lib.BGK_MIXED) as s:
+        s.set_state(f)
+        m = s.moments()
+    ref, mag = _moments(wl, f)
+    assert np.all(np.abs(m - ref) <= (16 + 2 * wl.n_vel ** 0.5) * 2.0 ** -53 * mag)
