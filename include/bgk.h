@@ -355,7 +355,7 @@ BGK_API bgk_status bgk_stage(bgk_ctx *ctx, const void *f_n, const void *f_in, vo
 /* Raw velocity moments of the stored state (section "Governing equations":
  * the moments that give Q = (rho, rho U, E)), m[P][11]: sum w F, sum w u_d F
  * (3), sum w u_d^2 F (3), sum w u1u2 F, sum w u1u3 F, sum w u2u3 F, sum w G,
- * summed to FP64 accuracy.  m is host (on_device = 0) or device memory (1).
+ * summed in FP64.  m is host (on_device = 0) or device memory (1).
  * Errors: BGK_EINVAL (NULL), BGK_ECUDA. */
 BGK_API bgk_status bgk_moments(bgk_ctx *ctx, double *m, int on_device);
 

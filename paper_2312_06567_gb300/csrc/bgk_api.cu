@@ -259,7 +259,7 @@ bgk_status check_device_status(bgk_ctx *ctx) {
 
 // Moment partials of a state.  The FP32 state's stepping path (check = false)
 // uses the stage epilogue's error-free FP32 accumulation; the diagnostic entry
-// points (check = true) fold its line sums in FP64.
+// points (check = true) sum in FP64, independently of it.
 bgk_status run_moments(bgk_ctx *ctx, const void *f, bool check = false) {
     LaunchScope ls(ctx, BGK_K_MOMENTS);
     if (ctx->precision == BGK_FP64) {

@@ -102,6 +102,18 @@ struct GasInfo {
     double delta, Pr, mu_ref, theta_ref, theta_S, gamma;
 };
 
+// The exact double of a float without a conversion instruction (FP64 pipe): the
+// exponent rebiased, a subnormal first scaled by 2^64, infinities and NaN with
+// the double's top exponent
+__device__ __forceinline__ double widen(float x) {
+    const unsigned ax = __float_as_uint(x) & 0x7fffffffu;
+    const bool sub = ax < 0x00800000u;
+    const unsigned b = __float_as_uint(sub ? x * 0x1p64f : x), m = b & 0x7fffffffu;
+    const unsigned bias = sub ? (896u - 64u) << 20 : ax >= 0x7f800000u ? 1792u << 20 : 896u << 20;
+    return __hiloint2double((int)((b & 0x80000000u) | (m == 0 ? 0u : (m >> 3) + bias)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 // Velocity node k with its index on axis d mirrored (j_d -> n_d - 1 - j_d):
 // the reflection u_d -> -u_d on a grid symmetric in axis d.
 __device__ __forceinline__ int mirror_velocity(int k, int d, const int n[3]) {
@@ -312,8 +324,8 @@ cudaError_t launch_maxwellian_f32(float *f, const double *q, const double *vtab,
 cudaError_t launch_macro(const double *mom, double *out, int P, const MeshInfo &mesh, const FROps &fr,
                          const GasInfo &gas, const double face_rho[6], const double *geo, cudaStream_t s);
 // Moments, entropy and totals of a stored state (moments.cu).  check (the
-// diagnostic entry points): the FP32 state's lines fold in FP64, and a point
-// whose sums are not finite (either precision) is summed again directly.
+// diagnostic entry points): FP64 sums of the FP32 state too, and a point whose
+// sums are not finite (either precision) is summed again directly.
 cudaError_t launch_moments_f64(const MomentArgs64 &a, const VelGrid &vg, int n_vblk, bool check, cudaStream_t s);
 cudaError_t launch_moments_f32(const float *f, double *part, const double *vtab, const VelGrid &vg, int Nu, int P,
                                int Kblk, int C, int n_vblk, bool check, cudaStream_t s);

@@ -9,12 +9,13 @@
 // thread, and scalar error-free sums.  Here:
 //   * raw moments are taken per first-axis velocity line: three (F) or four
 //     (F, G) sums over centred indices jt = j - jc, folded per line and plane;
-//   * the FP32 state's line sums are error-free FP32 pairs, two points per
-//     thread on packed instructions;
+//   * the stepping path's line sums of an FP32 state are error-free FP32 pairs,
+//     two points per thread on packed instructions; the diagnostic entry points
+//     sum in FP64 about the node nearest u = 0;
 //   * the entropy takes ln F from a table and a short series.
 // Times are on a GB300 for 16,384 points x 13,824 velocities (0.91 GB of FP32
 // state): the stepping path's moments 1.16 -> 0.40 ms, the diagnostics'
-// 7.18 -> 0.90, all of macro + moments + totals + entropy 22.6 -> 2.3.
+// 7.18 -> 1.46, all of macro + moments + totals + entropy 22.6 -> 2.9.
 #include <algorithm>
 
 #include "stage_f32_common.cuh"
@@ -146,141 +147,6 @@ __device__ __forceinline__ void zero_node(const VelGrid &vg, int (&jc)[3]) {
     for (int d = 0; d < 3; ++d) jc[d] = min(max((int)rint(-vg.lo[d] / vg.h[d]), 0), vg.n[d] - 1);
 }
 
-// Sum of eight pairs of values v with errors e: a balanced tree of TwoSums
-// (independent at each level, so no serial chain), the errors summed along.
-// s + c is within about 2^-51 of the sum of magnitudes.
-__device__ __forceinline__ void tree8(float2 (&v)[8], float2 (&e)[8], float2 &s, float2 &c) {
-#pragma unroll
-    for (int w = 4; w > 0; w >>= 1)
-#pragma unroll
-        for (int i = 0; i < w; ++i) {
-            const float2 a = v[i], b = v[i + w];
-            const float2 t = __fadd2_rn(a, b);
-            const float2 bp = sub2(t, a);
-            const float2 r = __fadd2_rn(sub2(a, sub2(t, bp)), sub2(b, bp));
-            v[i] = t;
-            e[i] = __fadd2_rn(__fadd2_rn(e[i], e[i + w]), r);
-        }
-    s = v[0];
-    c = e[0];
-}
-
-// Raw moments of an FP32 state for the diagnostic entry points, accurate as
-// FP64 sums are: eight velocities at a time as FP32 pair sums (tree8), those in
-// FP64.  1.75 FP64 instructions per value (0.63 ms of the FP64 pipe for the
-// state above, 0.90 in all) where a direct FP64 sum of the raw moments took 17
-// (7.18 ms).  Pair sums over whole lines are cheaper (0.45 ms) but lose up to
-// ten times more than FP64 sums do when lines are long and few.
-template <int C>
-__global__ void __launch_bounds__(MT, 2) k_moments_f32_diag(const float *f, double *part, VelGrid vg, int Nu, int P,
-                                                            int Kblk) {
-    constexpr int NL = C == 2 ? 4 : 3, NQ = C == 2 ? 7 : 6;
-    const int pa = blockIdx.x * (2 * MT) + threadIdx.x, pb = pa + MT;
-    if (pa >= P) return;
-    const bool two = pb < P;
-    const float *fa = f + pa, *fb = f + (two ? pb : pa);
-    const int vb = blockIdx.y;
-    const int k0 = vb * Kblk, k1 = min(Nu, k0 + Kblk);
-    const int vn1 = vg.n[0], vn2 = vg.n[1];
-    int jc[3];
-    zero_node(vg, jc);
-    const size_t GO = (size_t)Nu * P;
-    double *Ja = part + (size_t)vb * BGK_NMOM * P + pa;
-    double *Jb = part + (size_t)vb * BGK_NMOM * P + (two ? pb : pa);
-    double Pd[2][NQ];
-#pragma unroll
-    for (int i = 0; i < NQ; ++i) Pd[0][i] = Pd[1][i] = 0.0;
-    bool first = true;
-    auto flush = [&](int j3) {
-        const double c = trap3(j3, vg), t = (float)(j3 - jc[2]);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (h == 1 && !two) break;
-            double d[7];
-#pragma unroll
-            for (int i = 0; i < 7; ++i) d[i] = i < NQ ? Pd[h][i] : 0.0;
-            plane_to_part(h ? Jb : Ja, P, c, t, d, first);
-        }
-#pragma unroll
-        for (int i = 0; i < NQ; ++i) Pd[0][i] = Pd[1][i] = 0.0;
-        first = false;
-    };
-    int j3cur = (k0 / vn1) / vn2;
-    for (int kl = k0; kl < k1; kl += vn1) {
-        const int line = kl / vn1;
-        const int j2 = line % vn2, j3 = line / vn2;
-        if (j3 != j3cur) { flush(j3cur); j3cur = j3; }
-        double T[2][NL];
-#pragma unroll
-        for (int i = 0; i < NL; ++i) T[0][i] = T[1][i] = 0.0;
-        const size_t off = (size_t)kl * P;
-        for (int j0 = 0; j0 < vn1; j0 += 8) {
-            float2 F[8], v[8], e[8], s, c;
-            auto join = [&](int i) {
-                T[0][i] += (double)s.x + (double)c.x;
-                T[1][i] += (double)s.y + (double)c.y;
-            };
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                F[i] = dup2(0.f);
-                if (j0 + i < vn1) {
-                    const size_t o = off + (size_t)(j0 + i) * P;
-                    F[i] = make_float2(__ldcs(fa + o), __ldcs(fb + o));
-                }
-            }
-            float2 G[C == 2 ? 8 : 1];
-            if constexpr (C == 2) {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    G[i] = dup2(0.f);
-                    if (j0 + i < vn1) {
-                        const size_t o = GO + off + (size_t)(j0 + i) * P;
-                        G[i] = make_float2(__ldcs(fa + o), __ldcs(fb + o));
-                        G[i] = __fmul2_rn(dup2(trap(j0 + i, vn1)), G[i]);            // exact
-                    }
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                if (j0 + i < vn1) F[i] = __fmul2_rn(dup2(trap(j0 + i, vn1)), F[i]);   // exact
-                v[i] = F[i];
-                e[i] = dup2(0.f);
-            }
-            tree8(v, e, s, c);
-            join(0);
-#pragma unroll
-            for (int q = 1; q <= 2; ++q) {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const float t = (float)(j0 + i - jc[0]), w = q == 1 ? t : __fmul_rn(t, t);    // exact
-                    v[i] = __fmul2_rn(F[i], dup2(w));
-                    e[i] = __ffma2_rn(F[i], dup2(w), neg2(v[i]));
-                }
-                tree8(v, e, s, c);
-                join(q);
-            }
-            if constexpr (C == 2) {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) { v[i] = G[i]; e[i] = dup2(0.f); }
-                tree8(v, e, s, c);
-                join(NL - 1);
-            }
-        }
-        const double cd = trap(j2, vn2), t2 = (double)(j2 - jc[1]), bd = cd * t2, bbd = bd * t2;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            Pd[h][0] = fma(cd, T[h][0], Pd[h][0]); Pd[h][1] = fma(cd, T[h][1], Pd[h][1]); Pd[h][2] = fma(cd, T[h][2], Pd[h][2]);
-            Pd[h][3] = fma(bd, T[h][0], Pd[h][3]); Pd[h][4] = fma(bd, T[h][1], Pd[h][4]);
-            Pd[h][5] = fma(bbd, T[h][0], Pd[h][5]);
-            if (C == 2) Pd[h][NQ - 1] = fma(cd, T[h][NL - 1], Pd[h][NQ - 1]);
-        }
-    }
-    flush(j3cur);
-    const double uc[3] = {vg.lo[0] + jc[0] * vg.h[0], vg.lo[1] + jc[1] * vg.h[1], vg.lo[2] + jc[2] * vg.h[2]};
-    raw_in_place(Ja, P, vg, uc);
-    if (two) raw_in_place(Jb, P, vg, uc);
-}
-
 // The diagnostic entry points' second look: partials that are not finite (an
 // infinity or NaN in the state, or sums out of range) are summed again directly
 // in FP64: sums over centred indices make NaN of an infinite value (0 times it,
@@ -316,36 +182,56 @@ __global__ void __launch_bounds__(MT) k_moments_redo(const T *f, double *part, c
     for (int j = 0; j < BGK_NMOM; ++j) out[(size_t)j * P] = m[j];
 }
 
-// Raw moments of an FP64 state: per line T_m = sum_j c jt^m F (m <= 2) and
-// sum_j c G, three (four) FP64 instructions per value instead of the 17 of a
-// direct sum of the raw moments; folded per line into the centred index
-// moments.  The FP64 pipe still bounds it: 1.1e8 values in 1.09 ms (0.83 TB/s),
-// 0.54 of it the pipe's own time, against about 3 before.
-template <int C>
-__global__ void __launch_bounds__(MT) k_moments_f64(const double *f, double *part, VelGrid vg, int Nu, int P, int Kblk) {
+// Raw moments with FP64 sums: of an FP64 state, and of an FP32 state for the
+// diagnostic entry points.  Per line T_m = sum_j c jt^m F (m <= 2) and sum_j c G
+// with the exact factors c jt^m from a table, three (four) FP64 instructions per
+// value instead of the 17 of a direct sum of the raw moments, folded per line into
+// the plane's sums and per plane into the index moments in the partials buffer.
+// FP32 values are widened by integer instructions.  The FP64 pipe bounds it (two
+// instructions per multiprocessor and clock; two to four blocks, four or eight
+// loads ahead all take the same time): 2.3e8 FP32 values 1.46 ms (7.2 for direct
+// sums), with G 1.86, half as many FP64 ones 0.78 and 0.98.  Sums of eight FP32
+// values as FP32 pairs before the FP64 ones took 0.90 ms, but lost five times what
+// FP64 sums lose on lines of wide range.
+template <typename T, int C>
+__global__ void __launch_bounds__(MT, 2) k_moments_sums(const T *f, double *part, VelGrid vg, int Nu, int P, int Kblk) {
+    constexpr int NQ = C == 2 ? 7 : 6;
     const int p = blockIdx.x * MT + threadIdx.x;
-    __shared__ double2 sj[BGK_MAXV];                     // (jt, jt^2) of the first-axis nodes
+    // (c jt, c jt^2) and c of the first-axis nodes, c the trapezoid factor (exact)
+    __shared__ double2 sj[BGK_MAXV];
+    __shared__ double sc[BGK_MAXV];
     const int vn1 = vg.n[0], vn2 = vg.n[1];
     int jc[3];
     zero_node(vg, jc);
     for (int j = threadIdx.x; j < vn1; j += MT) {
-        const double t = j - jc[0];
-        sj[j] = make_double2(t, t * t);
+        const double t = j - jc[0], c = trap(j, vn1);
+        sj[j] = make_double2(c * t, c * t * t);
+        sc[j] = c;
     }
     __syncthreads();
     if (p >= P) return;
     const int vb = blockIdx.y;
     const int k0 = vb * Kblk, k1 = min(Nu, k0 + Kblk);
-    double J[11];
+    double *J = part + (size_t)vb * BGK_NMOM * P + p;
+    double Pd[7];
 #pragma unroll
-    for (int i = 0; i < 11; ++i) J[i] = 0.0;
+    for (int i = 0; i < 7; ++i) Pd[i] = 0.0;
+    bool first = true;
+    auto flush = [&](int j3) {
+        plane_to_part(J, P, trap3(j3, vg), (double)(j3 - jc[2]), Pd, first);
+#pragma unroll
+        for (int i = 0; i < 7; ++i) Pd[i] = 0.0;
+        first = false;
+    };
+    int j3cur = (k0 / vn1) / vn2;
     for (int kl = k0; kl < k1; kl += vn1) {
         const int line = kl / vn1;
         const int j2 = line % vn2, j3 = line / vn2;
-        const double *fl = f + (size_t)kl * P + p, *gl = fl + (size_t)Nu * P;
+        if (j3 != j3cur) { flush(j3cur); j3cur = j3; }
+        const T *fl = f + (size_t)kl * P + p, *gl = fl + (size_t)Nu * P;
         double T0 = 0.0, T1 = 0.0, T2 = 0.0, TG = 0.0;
         for (int j0 = 0; j0 < vn1; j0 += MCH) {
-            double F[MCH], G[C == 2 ? MCH : 1];
+            T F[MCH], G[C == 2 ? MCH : 1];
 #pragma unroll
             for (int i = 0; i < MCH; ++i)
                 if (j0 + i < vn1) {
@@ -356,31 +242,23 @@ __global__ void __launch_bounds__(MT) k_moments_f64(const double *f, double *par
             for (int i = 0; i < MCH; ++i) {
                 const int j1 = j0 + i;
                 if (j1 < vn1) {
-                    if (j1 == 0 || j1 == vn1 - 1) {      // trapezoid half weight
-                        F[i] *= 0.5;
-                        if (C == 2) G[C == 2 ? i : 0] *= 0.5;
-                    }
+                    const double x = widen(F[i]), c = sc[j1];
                     const double2 t = sj[j1];
-                    T0 += F[i];
-                    T1 = fma(t.x, F[i], T1);
-                    T2 = fma(t.y, F[i], T2);
-                    if (C == 2) TG += G[C == 2 ? i : 0];
+                    T0 = fma(c, x, T0);
+                    T1 = fma(t.x, x, T1);
+                    T2 = fma(t.y, x, T2);
+                    if (C == 2) TG = fma(c, widen(G[C == 2 ? i : 0]), TG);
                 }
             }
         }
-        const double c = (double)trap(j2, vn2) * (double)trap3(j3, vg), t2 = j2 - jc[1], t3 = j3 - jc[2];
-        const double cT0 = c * T0, cT1 = c * T1;
-        J[0] += cT0; J[1] += cT1; J[2] = fma(c, T2, J[2]);
-        J[3] = fma(t2, cT0, J[3]); J[4] = fma(t2, cT1, J[4]); J[5] = fma(t2 * t2, cT0, J[5]);
-        J[6] = fma(t3, cT0, J[6]); J[7] = fma(t3, cT1, J[7]); J[8] = fma(t2 * t3, cT0, J[8]);
-        J[9] = fma(t3 * t3, cT0, J[9]);
-        if (C == 2) J[10] = fma(c, TG, J[10]);
+        const double c = j2 == 0 || j2 == vn2 - 1 ? 0.5 : 1.0, t2 = (double)(j2 - jc[1]), b = c * t2, bb = b * t2;
+        Pd[0] = fma(c, T0, Pd[0]); Pd[1] = fma(c, T1, Pd[1]); Pd[2] = fma(c, T2, Pd[2]);
+        Pd[3] = fma(b, T0, Pd[3]); Pd[4] = fma(b, T1, Pd[4]); Pd[5] = fma(bb, T0, Pd[5]);
+        if (C == 2) Pd[NQ - 1] = fma(c, TG, Pd[NQ - 1]);
     }
+    flush(j3cur);
     const double uc[3] = {vg.lo[0] + jc[0] * vg.h[0], vg.lo[1] + jc[1] * vg.h[1], vg.lo[2] + jc[2] * vg.h[2]};
-    double m[BGK_NMOM];
-    index_to_raw(J, vg, uc, m);
-#pragma unroll
-    for (int i = 0; i < BGK_NMOM; ++i) part[((size_t)vb * BGK_NMOM + i) * P + p] = m[i];
+    raw_in_place(J, P, vg, uc);
 }
 
 // Sums over the velocity blocks, one thread per (slot, point): ACROSS writes
@@ -621,8 +499,8 @@ __global__ void k_totals_sum(const double *blk, int n, double *out) {
 
 cudaError_t launch_moments_f64(const MomentArgs64 &a, const VelGrid &vg, int n_vblk, bool check, cudaStream_t s) {
     dim3 grid((a.P + MT - 1) / MT, n_vblk);
-    if (a.C == 1) k_moments_f64<1><<<grid, MT, 0, s>>>(a.f, a.part, vg, a.Nu, a.P, a.Kblk);
-    else k_moments_f64<2><<<grid, MT, 0, s>>>(a.f, a.part, vg, a.Nu, a.P, a.Kblk);
+    if (a.C == 1) k_moments_sums<double, 1><<<grid, MT, 0, s>>>(a.f, a.part, vg, a.Nu, a.P, a.Kblk);
+    else k_moments_sums<double, 2><<<grid, MT, 0, s>>>(a.f, a.part, vg, a.Nu, a.P, a.Kblk);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !check) return e;
     k_moments_redo<double><<<grid, MT, 0, s>>>(a.f, a.part, a.vtab, a.Nu, a.P, a.Kblk, a.C);
@@ -631,17 +509,18 @@ cudaError_t launch_moments_f64(const MomentArgs64 &a, const VelGrid &vg, int n_v
 
 cudaError_t launch_moments_f32(const float *f, double *part, const double *vtab, const VelGrid &vg, int Nu, int P,
                                int Kblk, int C, int n_vblk, bool check, cudaStream_t s) {
-    const dim3 grid((P + 2 * MT - 1) / (2 * MT), n_vblk);
     if (!check) {
+        const dim3 grid((P + 2 * MT - 1) / (2 * MT), n_vblk);
         if (C == 1) k_moments_f32<1><<<grid, MT, 0, s>>>(f, part, vg, Nu, P, Kblk);
         else k_moments_f32<2><<<grid, MT, 0, s>>>(f, part, vg, Nu, P, Kblk);
         return cudaGetLastError();
     }
-    if (C == 1) k_moments_f32_diag<1><<<grid, MT, 0, s>>>(f, part, vg, Nu, P, Kblk);
-    else k_moments_f32_diag<2><<<grid, MT, 0, s>>>(f, part, vg, Nu, P, Kblk);
+    const dim3 grid((P + MT - 1) / MT, n_vblk);
+    if (C == 1) k_moments_sums<float, 1><<<grid, MT, 0, s>>>(f, part, vg, Nu, P, Kblk);
+    else k_moments_sums<float, 2><<<grid, MT, 0, s>>>(f, part, vg, Nu, P, Kblk);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_moments_redo<float><<<dim3((P + MT - 1) / MT, n_vblk), MT, 0, s>>>(f, part, vtab, Nu, P, Kblk, C);
+    k_moments_redo<float><<<grid, MT, 0, s>>>(f, part, vtab, Nu, P, Kblk, C);
     return cudaGetLastError();
 }
 

@@ -30,18 +30,6 @@ namespace cg = cooperative_groups;
 
 constexpr int WT = 256, WS = 4;      // threads of a block, blocks of a cluster
 
-// exact double of a float without a conversion instruction (FP64 pipe): the
-// exponent rebiased, a subnormal first scaled by 2^64, infinities and NaN with
-// the double's top exponent
-__device__ __forceinline__ double widen(float x) {
-    const unsigned ax = __float_as_uint(x) & 0x7fffffffu;
-    const bool sub = ax < 0x00800000u;
-    const unsigned b = __float_as_uint(sub ? x * 0x1p64f : x), m = b & 0x7fffffffu;
-    const unsigned bias = sub ? (896u - 64u) << 20 : ax >= 0x7f800000u ? 1792u << 20 : 896u << 20;
-    return __hiloint2double((int)((b & 0x80000000u) | (m == 0 ? 0u : (m >> 3) + bias)), (int)(b << 29));
-}
-__device__ __forceinline__ double widen(double x) { return x; }
-
 template <typename T, int Q>
 __global__ void __cluster_dims__(WS, 1, 1) __launch_bounds__(WT)
 k_wall_density(const T *f, const T *fvec, const double *bcval, const double *vtab, const int *wall_ef, int Ne,

@@ -1,6 +1,6 @@
 """Moments, totals and entropy where the values' range matters (GPU): dilute
 FP32 states whose tails are subnormal, infinite values, velocity grids far
-from centred on the gas."""
+from centred on the gas, and values of wide range along the lines."""
 import numpy as np
 import pytest
 
@@ -113,3 +113,21 @@ def test_moments_on_grids_far_from_centred(lib, lo, hi, prec, delta):
         m = s.moments()
     ref, mag = _moments(wl, f)
     assert np.all(np.abs(m - ref) <= (16 + 2 * wl.n_vel ** 0.5) * 2.0 ** -53 * mag)
+
+
+@pytest.mark.parametrize("delta", [0.0, 2.0])
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("vel_n", [(40, 2, 2), (128, 2, 2), (3, 2, 2)])
+def test_moments_of_values_of_wide_range(lib, vel_n, prec, delta):
+    """Values over seventeen decades in no order along the lines: a line's sum is
+    that of a few of them.  Bound: FP64 sums of n terms round like a random walk,
+    1.5 sqrt n ulp of the sum of magnitudes at three sigma, and 6 for the weights."""
+    wl = W.reduced(W.taylor_green_box(), mesh_n=(5, 5, 4), vel_n=vel_n).replace(p=3, delta=delta)
+    rng = np.random.default_rng(7)
+    f = np.exp(-rng.uniform(0.0, 40.0, (wl.n_comp, wl.n_vel, wl.n_elem, wl.n_sol)))
+    f = f.astype(np.float64 if prec == "fp64" else np.float32)
+    with lib.Solver(wl, lib.BGK_FP64 if prec == "fp64" else lib.BGK_MIXED) as s:
+        s.set_state(f)
+        m = s.moments()
+    ref, mag = _moments(wl, f)
+    assert np.all(np.abs(m - ref) <= (6 + 1.5 * wl.n_vel ** 0.5) * 2.0 ** -53 * mag)
