@@ -97,27 +97,25 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);      // a in the low half (lower address)
     return *reinterpret_cast<const uint32_t *>(&h);
 }
-// SiLU z / (1 + e^-z) of two values.  e^-z is held below 2^60 (beyond z = -41,
-// where the result is under 1e-16 either way), so that one reciprocal serves
-// both denominators, 1/d_a = d_b / (d_a d_b); each quotient is then corrected by
-// its exact remainder (Markstein 1990), which gives the correctly rounded
-// division but for rare last bits.  The IEEE divisions this replaces were half
-// of the kernel's instructions.
+// SiLU z / (1 + e^-z) of two values: an approximate reciprocal, then each quotient
+// corrected by its exact remainder (Markstein 1990), which gives the correctly
+// rounded division but for rare last bits (zero below z = -87, where the
+// reciprocal underflows).  The IEEE divisions this replaces were half of the
+// kernel's instructions.  One reciprocal for both denominators, with e^-z held
+// below 2^60 for it, made -|z| 2^-60 of what underflows.
 __device__ __forceinline__ float rcp_approx(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 __device__ __forceinline__ float2 silu2(float2 z) {
-    const float2 e = make_float2(fminf(__expf(-z.x), 1.15292150460684698e18f), fminf(__expf(-z.y), 1.15292150460684698e18f));
-    const float2 d = __fadd2_rn(e, make_float2(1.f, 1.f));
-    const float r = rcp_approx(__fmul_rn(d.x, d.y));
-    const float2 r2 = __fmul2_rn(make_float2(r, r), make_float2(d.y, d.x));
-    const float2 q = __fmul2_rn(z, r2);
+    const float2 d = __fadd2_rn(make_float2(__expf(-z.x), __expf(-z.y)), make_float2(1.f, 1.f));
+    const float2 r = make_float2(rcp_approx(d.x), rcp_approx(d.y));
+    const float2 q = __fmul2_rn(z, r);
     const float2 rem = __ffma2_rn(make_float2(-q.x, -q.y), d, z);
-    const float2 c = __ffma2_rn(rem, r2, q);
-    // an infinite z: the remainder is not a number, the quotient is the result
-    return make_float2(fabsf(z.x) <= 3.0e38f ? c.x : q.x, fabsf(z.y) <= 3.0e38f ? c.y : q.y);
+    const float2 c = __ffma2_rn(rem, r, q);
+    // an infinite z or d: the remainder is not a number, the quotient is the result
+    return make_float2(c.x == c.x ? c.x : q.x, c.y == c.y ? c.y : q.y);
 }
 // SiLU of 32 accumulator columns plus bias, rounded to BF16, written as four
 // 16-byte chunks of this thread's row of a K = 64 operand (chunks c0 .. c0+3)

@@ -89,3 +89,26 @@ def test_training_repeats_for_a_seed(lib):
     assert np.isfinite(runs[0][0])
     assert runs[1] == runs[0] and runs[2] == runs[0]
     assert runs[3][1] != runs[0][1]
+
+
+@pytest.mark.parametrize("z", [-50.0, -300.0, -1e4, -1e10, -1e30])
+def test_inference_where_silu_underflows(lib, z):
+    """First-layer arguments far below zero, where SiLU is below 1e-19 and a second
+    layer of weights 1e12 would show anything larger."""
+    params = [np.zeros(p.shape) for p in omlp.init_params(0)]
+    params[0][0, :] = 1.0
+    params[2][:] = 1e12
+    params[3][:] = 1.0
+    params[4][:] = 1.0
+    norm = np.concatenate([np.zeros(9), np.ones(9), np.zeros(5), np.ones(5)])
+    x = np.zeros((300, 9))
+    x[:, 0] = z
+    x[::7, 0] = 2.0 ** -60                                 # (beside ordinary arguments)
+    wl = W.reduced(W.periodic_sine_box(), mesh_n=(1, 1, 1), vel_n=(4, 4, 4))
+    with lib.Solver(wl) as s:
+        s.mlp_weights(load=(params, norm))
+        d = s.mlp_infer(x)
+    with np.errstate(over="ignore"):
+        y = omlp.forward_bf16([p.astype(np.float32).astype(np.float64) for p in params],
+                              x.astype(np.float32).astype(np.float64))
+    assert np.max(np.abs(d - y)) <= 5e-3 * np.abs(y).max()
