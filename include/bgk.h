@@ -461,7 +461,7 @@ BGK_API bgk_status bgk_shard_stage(bgk_ctx *ctx, const double *m, int stage, dou
  * quantities of section "Governing equations".  totals is host memory.
  * entropy (host memory, may be NULL): the discrete entropy
  * H = sum_e sum_s W_s J_s sum_k w_k F ln F of the stored F component with the
- * same quadrature, to FP64 accuracy (section "Numerical method": the
+ * same quadrature, summed in FP64 (section "Numerical method": the
  * discrete-velocity BGK relaxation does not increase it).  It is NaN when
  * some stored F is not positive.  With delta > 0 it covers F only (the paper
  * states no entropy functional for the reduced F, G pair).

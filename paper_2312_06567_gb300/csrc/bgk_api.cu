@@ -41,6 +41,7 @@ struct bgk_ctx {
     float *geop;                      // the same in the FP32 stage kernel's thread order
     double *rho_w;                    // [Ne][6][q*q] diffuse-wall densities
     float2 *rho_w2, *bc2;             // rho_w and bcval as FP32 pairs (mixed form)
+    double *log_tab;                  // logarithm table of the FP32 state's entropy (mixed form)
     CurvOps32 cops;                   // FP32 tables of the mixed-form curvilinear stage
     int *wall_ef;                     // [n_wall][2] (element, face) pairs on diffuse faces
     int n_wall;
@@ -646,6 +647,7 @@ bgk_status create_ctx(bgk_ctx **out, const bgk_mesh_desc *mesh, const bgk_vgrid_
     ctx->curved = curved;
     ctx->geo = ctx->fvec = nullptr; ctx->geo32 = ctx->fvec32 = ctx->geop = nullptr;
     ctx->rho_w2 = ctx->bc2 = nullptr;
+    ctx->log_tab = nullptr;
     ctx->rho_w = nullptr; ctx->wall_ef = nullptr; ctx->n_wall = 0;
     std::vector<double> fvec_h;
     std::vector<int> wall_h;
@@ -765,6 +767,12 @@ bgk_status create_ctx(bgk_ctx **out, const bgk_mesh_desc *mesh, const bgk_vgrid_
     ctx->eq32 = nullptr;
     if (st == BGK_OK && precision == BGK_MIXED)
         cu(cudaMalloc(&ctx->eq32, P * BGK_NEQ32 * sizeof(float)), "cudaMalloc(eq32)");
+    if (st == BGK_OK && precision == BGK_MIXED) {
+        std::vector<double> lt;
+        entropy_log_table(lt);
+        cu(cudaMalloc(&ctx->log_tab, lt.size() * sizeof(double)), "cudaMalloc(log_tab)");
+        if (st == BGK_OK) cu(cudaMemcpy(ctx->log_tab, lt.data(), lt.size() * sizeof(double), cudaMemcpyHostToDevice), "upload log_tab");
+    }
     if (st == BGK_OK) cu(cudaMalloc(&ctx->qp, P * 5 * sizeof(double)), "cudaMalloc(qp)");
     if (st == BGK_OK) cu(cudaMalloc(&ctx->iters, P * sizeof(int)), "cudaMalloc(iters)");
     if (st == BGK_OK) cu(cudaMalloc(&ctx->vtab, ctx->vtab_h.size() * sizeof(double)), "cudaMalloc(vtab)");
@@ -973,7 +981,7 @@ bgk_status bgk_destroy(bgk_ctx *ctx) {
     if (ctx->shard) { cudaFree(ctx->vtab_q); cudaFree(ctx->vtab32_q); }
     cudaFree(ctx->stats);
     cudaFree(ctx->geo); cudaFree(ctx->fvec); cudaFree(ctx->geo32); cudaFree(ctx->fvec32); cudaFree(ctx->geop);
-    cudaFree(ctx->rho_w2); cudaFree(ctx->bc2);
+    cudaFree(ctx->rho_w2); cudaFree(ctx->bc2); cudaFree(ctx->log_tab);
     cudaFree(ctx->rho_w); cudaFree(ctx->wall_ef);
     cudaFree(ctx->mlp_w); cudaFree(ctx->mlp_w16); cudaFree(ctx->mlp_norm); cudaFree(ctx->mlp_m); cudaFree(ctx->mlp_v);
     cudaFree(ctx->mlp_grad); cudaFree(ctx->mlp_loss); cudaFree(ctx->log); cudaFree(ctx->log_count);
@@ -1580,7 +1588,7 @@ bgk_status bgk_totals(bgk_ctx *ctx, double totals[5], double *entropy) {
             e = ctx->precision == BGK_FP64
                     ? launch_entropy_f64((const double *)ctx->f[0], ctx->vg, ctx->Nu, ctx->P, ctx->Kblk, ctx->n_vblk, ent,
                                          bad, ctx->stream)
-                    : launch_entropy_f32((const float *)ctx->f[0], ctx->vg, ctx->Nu, ctx->P, ctx->Kblk, ctx->n_vblk, ent,
+                    : launch_entropy_f32((const float *)ctx->f[0], ctx->log_tab, ctx->vg, ctx->Nu, ctx->P, ctx->Kblk, ctx->n_vblk, ent,
                                          bad, ctx->stream);
     }
     if (e == cudaSuccess)

@@ -335,9 +335,10 @@ cudaError_t launch_sum_partials(const double *part, int n_vblk, int P, double *o
 cudaError_t launch_reduce_moments(const double *part, int n_vblk, int P, double *m_out,
                                   cudaStream_t s);
 // per-point entropy partials part[n_vblk][P] of the F component; *nonpos counts
-// the values that are not positive
-cudaError_t launch_entropy_f32(const float *f, const VelGrid &vg, int Nu, int P, int Kblk, int n_vblk, double *part,
-                               unsigned int *nonpos, cudaStream_t s);
+// the values that are not positive; logs: entropy_log_table's on the device
+void entropy_log_table(std::vector<double> &out);
+cudaError_t launch_entropy_f32(const float *f, const double *logs, const VelGrid &vg, int Nu, int P, int Kblk, int n_vblk,
+                               double *part, unsigned int *nonpos, cudaStream_t s);
 cudaError_t launch_entropy_f64(const double *f, const VelGrid &vg, int Nu, int P, int Kblk, int n_vblk, double *part,
                                unsigned int *nonpos, cudaStream_t s);
 // scratch[0..5] = domain totals (5) and entropy from mom[P][11] and ent[n_vblk][P]

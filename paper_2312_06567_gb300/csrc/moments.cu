@@ -12,11 +12,14 @@
 //   * the stepping path's line sums of an FP32 state are error-free FP32 pairs,
 //     two points per thread on packed instructions; the diagnostic entry points
 //     sum in FP64 about the node nearest u = 0;
-//   * the entropy takes ln F from a table and a short series.
+//   * the entropy takes ln F from a table and a short series, the part that FP32
+//     holds exactly or that lies far below the result on packed instructions.
 // Times are on a GB300 for 16,384 points x 13,824 velocities (0.91 GB of FP32
 // state): the stepping path's moments 1.16 -> 0.40 ms, the diagnostics'
-// 7.18 -> 1.46, all of macro + moments + totals + entropy 22.6 -> 2.9.
+// 7.18 -> 1.46, all of macro + moments + totals + entropy 22.6 -> 3.9.
 #include <algorithm>
+#include <cmath>
+#include <cstring>
 
 #include "stage_f32_common.cuh"
 
@@ -24,12 +27,6 @@ namespace {
 
 constexpr int MT = 256;          // threads per block
 constexpr int MCH = 8;           // velocities loaded before they are used
-// ln2 = 45426 / 2^16 + LN2_MID + LN2_LO, the first two of at most 16 bits (an
-// integer of up to 8 bits times either is exact in FP32)
-constexpr double kLn2Rest = 0.69314718055994530942 - 45426.0 / 65536.0;
-constexpr float LN2_MID = (float)((double)(long long)(kLn2Rest * 34359738368.0) / 34359738368.0);     // 2^35
-constexpr float LN2_LO = (float)(kLn2Rest - (double)LN2_MID);
-
 // one plane quantity of two points: P += c * (s + e), error-free
 __device__ __forceinline__ void plane_add2(float2 &P, float2 &Pe, float c, float2 s, float2 e) {
     const float2 c2 = dup2(c);
@@ -275,66 +272,48 @@ __global__ void __launch_bounds__(MT) k_reduce_moments(const double *part, int n
 }
 
 // ---- entropy ---------------------------------------------------------------
-// ln x of a normal FP32 x as an unevaluated pair s + c (table-driven, after
-// Tang 1990): x = 2^e m with m in [1, 2), k_i = 1/m to 9 bits for the 256
-// subintervals of m, so r = m k_i - 1 is exact in FP32 (33 bits of m k_i less
-// the 9 that cancel, |r| <= 2^-8), and
-//   ln x = e ln2 - ln k_i + r - r^2/2 + r^3 (1/3 - r/4 + r^2/5 - ...).
-// ln2 is split so that e times its two leading parts is exact; the large
-// terms are added with their rounding errors kept (TwoSum).  The pair is good
-// to about 2^-47 of max(|ln x|, 1); on two values at once.
-struct LogTab { float k, hi, lo, pad; };                 // k_i, -ln k_i = hi + lo
-__device__ __forceinline__ void two_sum2(float2 &s, float2 &c, float2 v) {
-    const float2 t = __fadd2_rn(s, v);
-    const float2 bp = sub2(t, s);
-    c = __fadd2_rn(c, __fadd2_rn(sub2(s, sub2(t, bp)), sub2(v, bp)));
-    s = t;
-}
-__device__ __forceinline__ void log_pair2(const LogTab *tab, float2 x, float2 &s, float2 &c) {
-    const unsigned ba = __float_as_uint(x.x), bb = __float_as_uint(x.y);
-    const float4 ta = *reinterpret_cast<const float4 *>(tab + ((ba >> 15) & 255u));
-    const float4 tb = *reinterpret_cast<const float4 *>(tab + ((bb >> 15) & 255u));
-    const float2 m = make_float2(__uint_as_float((ba & 0x007fffffu) | 0x3f800000u),
-                                 __uint_as_float((bb & 0x007fffffu) | 0x3f800000u));
-    // the exponent as a float: 2^23 + biased exponent, minus 2^23 + 127 (exact)
-    const float2 e = __fadd2_rn(make_float2(__uint_as_float((ba >> 23) | 0x4b000000u),
-                                            __uint_as_float((bb >> 23) | 0x4b000000u)), dup2(-8388735.f));
-    const float2 r = __ffma2_rn(m, make_float2(ta.x, tb.x), dup2(-1.f));             // exact
+// ln x of a normal FP32 x (table-driven, after Tang 1990): x = 2^e m with m in
+// [1, 2), k_i = 1/m to ten bits for the 1024 subintervals of m, so r = m k_i - 1
+// is exact in FP32 (33 bits of m k_i less the 9 that cancel, |r| < 2^-9.6), and
+//   ln x = (e ln2 - ln k_i) + (r - r^2/2) + r^3 (1/3 - r/4 + r^2/5):
+// the first term in FP64, the second as an FP32 pair, the third, below 2^-30, in
+// FP32 with the pair's low part and the rest of ln2.  Within 2^-50 of |ln x| for x
+// outside [0.875, 1.125) (2^-54 root mean square, as log() has), where ln x itself
+// is small; log() serves that interval.
+constexpr int LOG_N = 1024;
+struct LogTab { float k, pad; double l; };               // k_i, -ln k_i
+// s + c = r - r^2/2 + r^3 (...) + e (ln2 - its FP64 value), on two values at once
+__device__ __forceinline__ void log_tail2(float2 r, float2 e, float2 &s, float2 &c) {
     const float2 q = __fmul2_rn(r, r);
     const float2 qe = __ffma2_rn(r, r, neg2(q));                                     // r^2 = q + qe
-    float2 t = __ffma2_rn(r, dup2(-1.f / 6.f), dup2(0.2f));
-    t = __ffma2_rn(r, t, dup2(-0.25f));
+    float2 t = __ffma2_rn(r, dup2(0.2f), dup2(-0.25f));
     t = __ffma2_rn(r, t, dup2(1.f / 3.f));
     t = __fmul2_rn(__fmul2_rn(r, q), t);
-    s = __fmul2_rn(e, dup2(0.693145751953125f));                                     // exact
-    c = dup2(0.f);
-    two_sum2(s, c, make_float2(ta.y, tb.y));
-    two_sum2(s, c, r);
-    two_sum2(s, c, __fmul2_rn(e, dup2(LN2_MID)));                                    // exact product
-    two_sum2(s, c, __fmul2_rn(q, dup2(-0.5f)));
-    float2 w = __ffma2_rn(qe, dup2(-0.5f), t);
-    w = __fadd2_rn(w, make_float2(ta.z, tb.z));
-    w = __ffma2_rn(e, dup2(LN2_LO), w);
-    c = __fadd2_rn(c, w);
+    s = __ffma2_rn(q, dup2(-0.5f), r);
+    const float2 low = __ffma2_rn(q, dup2(-0.5f), sub2(r, s));                       // exact: |r| > q/2
+    c = __fadd2_rn(__ffma2_rn(qe, dup2(-0.5f), t), low);
+    c = __ffma2_rn(e, dup2(2.3190468138e-17f), c);
+}
+// the exact double of a normal FP32 value, halved for half = 1; of zero 2^-127,
+// nothing beside the terms it is added to
+__device__ __forceinline__ double widen_normal(float x, unsigned half = 0) {
+    const unsigned b = __float_as_uint(x);
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + ((896u - half) << 20))), (int)(b << 29));
 }
 
 // Discrete entropy of the F component, partial over velocity blocks:
 // part[vb][p] = sum_{k in block vb} w_k F ln F; a non-positive F (or NaN) has
-// no entropy and is counted in *nonpos instead.  Two points per thread, the
-// logarithm and the line sums as FP32 pairs, one FP64 update per line: the
-// FP64 log and sum of every value took 12 ms for 2.3e8 values (25 FP64
-// instructions each), this is bound by FP32 issue (about 45 per value).
-__global__ void __launch_bounds__(MT, 4) k_entropy_f32(const float *f, VelGrid vg, int Nu, int P, int Kblk, double *part,
-                                                       unsigned int *nonpos) {
-    __shared__ __align__(16) LogTab tab[256];
-    for (int i = threadIdx.x; i < 256; i += MT) {
-        const double k = rint(512.0 / (1.0 + (i + 0.5) / 256.0)) / 512.0;
-        const double l = -log(k);
-        tab[i].k = (float)k;
-        tab[i].hi = (float)l;
-        tab[i].lo = (float)(l - (double)(float)l);
-        tab[i].pad = 0.f;
-    }
+// no entropy and is counted in *nonpos instead.  The sums are FP64 ones; two
+// points per thread, so that what FP32 can do of the logarithm exactly or far
+// below the result runs packed and four FP64 instructions per value remain (a
+// library log and its sum take 25): 2.3e8 values 1.7 ms, 12 ms with log(), bound
+// by the FP64 pipe at any occupancy from two to five blocks.  With ln F and the
+// line sums as FP32 pairs 0.7 ms, but 2^-46 of F off where log() has 2^-53.
+__global__ void __launch_bounds__(MT, 4) k_entropy_f32(const float *f, const LogTab *logs, VelGrid vg, int Nu, int P,
+                                                       int Kblk, double *part, unsigned int *nonpos) {
+    __shared__ __align__(16) LogTab tab[LOG_N];
+    for (int i = threadIdx.x; i < LOG_N; i += MT)
+        reinterpret_cast<float4 *>(tab)[i] = __ldg(reinterpret_cast<const float4 *>(logs) + i);
     __syncthreads();
     const int pa = blockIdx.x * (2 * MT) + threadIdx.x, pb = pa + MT;
     if (pa >= P) return;
@@ -345,10 +324,15 @@ __global__ void __launch_bounds__(MT, 4) k_entropy_f32(const float *f, VelGrid v
     const int vn1 = vg.n[0], vn2 = vg.n[1];
     double h[2] = {0.0, 0.0};
     unsigned int bad = 0;
+    // not the table's: outside the positive normal range, or near 1
+    auto other = [](float v) {
+        const unsigned b = __float_as_uint(v);
+        return b - 0x00800000u >= 0x7f000000u || b - 0x3f600000u < 0x00300000u;
+    };
     for (int kl = k0; kl < k1; kl += vn1) {
         const int line = kl / vn1;
         const double c23 = (double)trap(line % vn2, vn2) * (double)trap3(line / vn2, vg);
-        float2 L = dup2(0.f), E = dup2(0.f);
+        double T[2] = {0.0, 0.0}, S[2] = {0.0, 0.0};
         for (int j0 = 0; j0 < vn1; j0 += MCH) {
             float2 F[MCH];
 #pragma unroll
@@ -360,31 +344,40 @@ __global__ void __launch_bounds__(MT, 4) k_entropy_f32(const float *f, VelGrid v
 #pragma unroll
             for (int i = 0; i < MCH; ++i) {
                 if (j0 + i >= vn1) continue;
-                float2 cj = dup2(trap(j0 + i, vn1));
-                // outside the positive normal range: subnormal and infinite
-                // values by the FP64 log, anything else is counted.  Their place
-                // in the pair is taken by 1 with weight zero: log_pair2(1) is
-                // -2.2e-16, not 0, which F as small as these would not hide
-                if ((__float_as_uint(F[i].x) - 0x00800000u) >= 0x7f000000u || (__float_as_uint(F[i].y) - 0x00800000u) >= 0x7f000000u) {
+                const bool end = j0 + i == 0 || j0 + i == vn1 - 1;                   // trapezoid half weight
+                double xa = widen_normal(F[i].x, end), xb = widen_normal(F[i].y, end);
+                if (other(F[i].x) || other(F[i].y)) {
+                    // positive values by log(), anything else is counted; their
+                    // weight in the sums below is zero
                     for (int q = 0; q < 2; ++q) {
                         const float v = q ? F[i].y : F[i].x;
-                        if ((__float_as_uint(v) - 0x00800000u) < 0x7f000000u) continue;
-                        if (v > 0.f) h[q] = fma(c23 * (double)(q ? cj.y : cj.x) * (double)v, log((double)v), h[q]);
+                        if (!other(v)) continue;
+                        if (v > 0.f) h[q] = fma(c23 * (end ? 0.5 : 1.0) * (double)v, log((double)v), h[q]);
                         else if (q == 0 || two) ++bad;
-                        if (q) { F[i].y = 1.f; cj.y = 0.f; }
-                        else { F[i].x = 1.f; cj.x = 0.f; }
+                        if (q) { F[i].y = 1.f; xb = 0.0; }
+                        else { F[i].x = 1.f; xa = 0.0; }
                     }
                 }
-                float2 ls, lc;
-                log_pair2(tab, F[i], ls, lc);
-                const float2 cF = __fmul2_rn(cj, F[i]);                              // exact
-                const float2 p = __fmul2_rn(cF, ls);
-                sum2x2(L, E, p);
-                E = __fadd2_rn(E, __ffma2_rn(cF, lc, __ffma2_rn(cF, ls, neg2(p))));
+                const unsigned ba = __float_as_uint(F[i].x), bb = __float_as_uint(F[i].y);
+                const LogTab ta = tab[(ba >> 13) & (LOG_N - 1)], tb = tab[(bb >> 13) & (LOG_N - 1)];
+                const float2 m = make_float2(__uint_as_float((ba & 0x007fffffu) | 0x3f800000u),
+                                             __uint_as_float((bb & 0x007fffffu) | 0x3f800000u));
+                // the exponent as a float: 2^23 + biased exponent, minus 2^23 + 127 (exact)
+                const float2 e = __fadd2_rn(make_float2(__uint_as_float((ba >> 23) | 0x4b000000u),
+                                                        __uint_as_float((bb >> 23) | 0x4b000000u)), dup2(-8388735.f));
+                const float2 r = __ffma2_rn(m, make_float2(ta.k, tb.k), dup2(-1.f));             // exact
+                float2 s, c;
+                log_tail2(r, e, s, c);
+                T[0] = fma(xa, fma(widen_normal(e.x), 0.69314718055994530942, ta.l), T[0]);
+                T[1] = fma(xb, fma(widen_normal(e.y), 0.69314718055994530942, tb.l), T[1]);
+                S[0] = fma(xa, widen_normal(s.x), S[0]);
+                S[1] = fma(xb, widen_normal(s.y), S[1]);
+                S[0] = fma(xa, widen_normal(c.x), S[0]);
+                S[1] = fma(xb, widen_normal(c.y), S[1]);
             }
         }
-        h[0] = fma(c23, (double)L.x + (double)E.x, h[0]);
-        h[1] = fma(c23, (double)L.y + (double)E.y, h[1]);
+        h[0] = fma(c23, T[0] + S[0], h[0]);
+        h[1] = fma(c23, T[1] + S[1], h[1]);
     }
     const double W = vg.h[0] * vg.h[1] * vg.h[2];
     part[(size_t)vb * P + pa] = W * h[0];
@@ -392,9 +385,9 @@ __global__ void __launch_bounds__(MT, 4) k_entropy_f32(const float *f, VelGrid v
     if (bad) atomicAdd(nonpos, bad);
 }
 
-// The same of an FP64 state.  ln F by the same table in FP64, r = m k_i - 1
-// with one rounding and the series to r^7 (2^-67 of the next term): 12 FP64
-// instructions per value in place of the library log()'s path (36 ms for
+// The same of an FP64 state.  ln F by a table of 256 subintervals in FP64, r =
+// m k_i - 1 with one rounding and the series to r^7 (2^-67 of the next term): 12
+// FP64 instructions per value in place of the library log()'s path (36 ms for
 // 1.1e8 values); the FP64 pipe bounds it.
 __global__ void __launch_bounds__(MT) k_entropy_f64(const double *f, VelGrid vg, int Nu, int P, int Kblk, double *part,
                                                     unsigned int *nonpos) {
@@ -426,7 +419,9 @@ __global__ void __launch_bounds__(MT) k_entropy_f64(const double *f, VelGrid vg,
                 const double F = Fc[i];
                 const unsigned hi = (unsigned)__double2hiint(F);
                 double l;
-                if (hi - 0x00100000u >= 0x7fe00000u) {           // not a positive normal value
+                // not a positive normal value, or in [0.875, 1.125), where ln F
+                // is small beside the table's roundings
+                if (hi - 0x00100000u >= 0x7fe00000u || hi - 0x3fec0000u < 0x00060000u) {
                     if (!(F > 0.0)) { ++bad; continue; }
                     l = log(F);
                 } else {
@@ -534,9 +529,20 @@ cudaError_t launch_reduce_moments(const double *part, int n_vblk, int P, double 
     return cudaGetLastError();
 }
 
-cudaError_t launch_entropy_f32(const float *f, const VelGrid &vg, int Nu, int P, int Kblk, int n_vblk, double *part,
-                               unsigned int *nonpos, cudaStream_t s) {
-    k_entropy_f32<<<dim3((P + 2 * MT - 1) / (2 * MT), n_vblk), MT, 0, s>>>(f, vg, Nu, P, Kblk, part, nonpos);
+void entropy_log_table(std::vector<double> &out) {
+    out.resize(2 * LOG_N);
+    for (int i = 0; i < LOG_N; ++i) {
+        LogTab t{};
+        t.k = (float)(std::rint(LOG_N / (1.0 + (i + 0.5) / LOG_N)) / LOG_N);
+        t.l = -std::log((double)t.k);
+        std::memcpy(&out[2 * i], &t, sizeof t);
+    }
+}
+
+cudaError_t launch_entropy_f32(const float *f, const double *logs, const VelGrid &vg, int Nu, int P, int Kblk, int n_vblk,
+                               double *part, unsigned int *nonpos, cudaStream_t s) {
+    k_entropy_f32<<<dim3((P + 2 * MT - 1) / (2 * MT), n_vblk), MT, 0, s>>>(f, reinterpret_cast<const LogTab *>(logs), vg, Nu, P,
+                                                                           Kblk, part, nonpos);
     return cudaGetLastError();
 }
 cudaError_t launch_entropy_f64(const double *f, const VelGrid &vg, int Nu, int P, int Kblk, int n_vblk, double *part,

@@ -1,6 +1,7 @@
 """Moments, totals and entropy where the values' range matters (GPU): dilute
 FP32 states whose tails are subnormal, infinite values, velocity grids far
-from centred on the gas, and values of wide range along the lines."""
+from centred on the gas, values of wide range along the lines, and
+values around 1, where ln F is small."""
 import numpy as np
 import pytest
 
@@ -131,3 +132,36 @@ def test_moments_of_values_of_wide_range(lib, vel_n, prec, delta):
         m = s.moments()
     ref, mag = _moments(wl, f)
     assert np.all(np.abs(m - ref) <= (6 + 1.5 * wl.n_vel ** 0.5) * 2.0 ** -53 * mag)
+
+
+CONSTANTS = [1e-30, 3e-7, 0.0635, 0.31, 0.52, 0.74, 0.86, 0.9, 0.9999, 1.0, 1.0000002, 1.06, 1.13, 1.19, 1.9, 7.3, 4e5]
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("vel_n", [(24, 3, 2), (128, 2, 2), (5, 2, 2)])
+def test_entropy_of_one_value_everywhere(lib, vel_n, prec):
+    """Every term has the same rounding, so nothing averages out.  Bound: a
+    logarithm good to 4 ulp and FP64 sums of n1 terms, (8 + n1) ulp."""
+    wl = W.reduced(W.taylor_green_box(), mesh_n=(1, 1, 1), vel_n=vel_n).replace(p=1)
+    dt = np.float64 if prec == "fp64" else np.float32
+    with lib.Solver(wl, lib.BGK_FP64 if prec == "fp64" else lib.BGK_MIXED) as s:
+        for c in CONSTANTS:
+            f = np.full((1, wl.n_vel, wl.n_elem, wl.n_sol), c, dtype=dt)
+            s.set_state(f)
+            want, mag = _entropy(wl, f)
+            assert abs(s.entropy() - want) <= (8 + vel_n[0]) * 2.0 ** -53 * mag, c
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("vel_n", [(24, 5, 4), (128, 3, 2), (3, 2, 2)])
+def test_entropy_of_values_of_wide_range(lib, vel_n, prec):
+    """Seventeen decades in no order, and a second state around 1."""
+    wl = W.reduced(W.taylor_green_box(), mesh_n=(3, 1, 1), vel_n=vel_n).replace(p=2)
+    rng = np.random.default_rng(9)
+    shape = (1, wl.n_vel, wl.n_elem, wl.n_sol)
+    with lib.Solver(wl, lib.BGK_FP64 if prec == "fp64" else lib.BGK_MIXED) as s:
+        for lo, hi in ((-40.0, 0.0), (-0.3, 0.3)):
+            f = np.exp(rng.uniform(lo, hi, shape)).astype(np.float64 if prec == "fp64" else np.float32)
+            s.set_state(f)
+            want, mag = _entropy(wl, f)
+            assert abs(s.entropy() - want) <= (8 + vel_n[0]) * 2.0 ** -53 * mag
