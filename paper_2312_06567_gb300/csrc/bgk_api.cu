@@ -1200,9 +1200,7 @@ bgk_status bgk_tune_stage(bgk_ctx *ctx, double dt, int reps, int *variant_out, i
         for (int d : {2, 3, 4, 6, 8, 12, 16})
             if (stage_f32_variant_supported(sa, ctx->C, v, d)) cands.push_back({v, d});
     // the line kernel reading directly, where that is what AUTO would run
-    int auto_depth = 0;
-    if (!ctx->curved && !stage_f32_auto_ring(sa, ctx->C, &auto_depth) && stage_f32_direct_supported(sa))
-        cands.push_back({BGK_STAGE_AUTO, ctx->stage_depth});
+    if (stage_f32_auto_direct(sa, ctx->C, ctx->n_vblk, ctx->stage_depth)) cands.push_back({BGK_STAGE_AUTO, ctx->stage_depth});
     cudaEvent_t ea = nullptr, eb = nullptr;
     CU(cudaEventCreate(&ea));
     CU(cudaEventCreate(&eb));

@@ -314,8 +314,10 @@ bool stage_f32_line_supported(const StageArgs<float> &a, int C, int kind, int de
 cudaError_t launch_stage_f32_line(const StageArgs<float> &a, int C, int n_vblk, int kind, int depth, cudaStream_t s);
 // the line kernel without the copy ring (any order, element count and box face)
 bool stage_f32_direct_supported(const StageArgs<float> &a);
-// whether BGK_STAGE_AUTO takes the ring form on this mesh, and its depth
+// whether the line kernel's form for this mesh is the ring, and its depth
 bool stage_f32_auto_ring(const StageArgs<float> &a, int C, int *depth);
+// whether BGK_STAGE_AUTO runs the line kernel without the ring
+bool stage_f32_auto_direct(const StageArgs<float> &a, int C, int n_vblk, int depth);
 cudaError_t launch_stage_f32_direct(const StageArgs<float> &a, int C, int n_vblk, cudaStream_t s);
 // any FP32 stage variant: is it available for these arguments
 bool stage_f32_variant_supported(const StageArgs<float> &a, int C, int variant, int depth);

@@ -736,6 +736,71 @@ bool stage_f32_variant_supported(const StageArgs<float> &a, int C, int variant, 
     }
 }
 
+// Blocks of the node-per-thread kernels (256 threads of whole elements; the
+// asynchronous one keeps to element rows).
+static long long node_blocks(const StageArgs<float> &a, int n_vblk, bool async) {
+    const int eb = 256 / (a.fr.q * a.fr.q * a.fr.q);
+    const long long n = async ? (long long)((a.mesh.n[0] + eb - 1) / eb) * a.mesh.n[1] * a.mesh.n[2] : (a.mesh.Ne + eb - 1) / eb;
+    return n * n_vblk;
+}
+
+static int multiprocessors() {
+    int dev = 0, sms = 0;
+    const bool ok = cudaGetDevice(&dev) == cudaSuccess &&
+                    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+    return ok ? sms : 152;
+}
+
+// Which kernel BGK_STAGE_AUTO runs on a box.  While the node-per-thread kernels
+// (asynchronous where it applies, else plain) fit the GPU in one wave of two
+// blocks per multiprocessor, every node has a thread of its own at once, and a
+// velocity costs the latency of one node; the line kernel's threads walk p + 1
+// nodes each, and its fewer warps hide less.  Beyond one wave the line kernel's
+// smaller instruction count wins.  Measured (us per stage, line kernel / the
+// other; 152 multiprocessors, up to 64 velocity blocks):
+//   p = 4, F and G, x faces Dirichlet, 24^3   8 elements 1169 / 565, 12: 1473 / 1196,
+//     18: 2.0 waves, 0.90 of the other's speed, 24: 1.06; periodic from one wave on 1.01
+//   p = 4, one component, 24^3                8 elements 630 / 533, 12: 1.47 times faster
+//   p = 3, F and G, 24^3                      8 elements 600 / 297, 12: 493 / 361, 24: 1.16
+//   p = 3, one component, periodic            8 elements 0.92, 9: 1.08; Dirichlet 16: 0.91, 24: 1.43
+//   p = 2, Dirichlet, 24^3                    8 elements 245 / 213, 36: 0.95, 64: 1.89;
+//     F and G, periodic: 36 elements 0.93, 64: 1.96; one component, periodic: 1.0 to 1.5
+//   p = 1, F and G, 33 x 28 x 26              27 elements 936 / 420, 64: 998 / 1609
+//   p = 1, one component, Dirichlet, 24^3     27 elements 180 / 154, 48: 182 / 455; periodic 0.98 to 5
+//   specular faces (the other is the plain kernel): p = 3, one component 1.2, F and G 0.8
+//     below one wave; p <= 2 above 1
+//   blocks of a line or two, p = 2, one component, periodic, 8^3: 4 elements 26.5 / 23.3
+enum { FORM_NODE, FORM_RING, FORM_DIRECT };
+static int auto_form(const StageArgs<float> &a, int C, int n_vblk, int depth, int *ring_depth) {
+    const bool ring = stage_f32_auto_ring(a, C, ring_depth);
+    if (!ring && !stage_f32_direct_supported(a)) return FORM_NODE;
+    const int sms = multiprocessors();
+    bool open = false;                                   // some face holds a Dirichlet state
+    for (int f = 0; f < 6; ++f) open |= !a.mesh.periodic[f / 2] && !a.mesh.specular[f];
+    const bool async = stage_f32_tma_supported(a, C, depth), spec = any_specular(a.mesh);
+    const double waves = (double)node_blocks(a, n_vblk, false) / (2.0 * sms);
+    const bool brief = a.Kblk <= 24;                     // a block's velocities are a line or two, whose set-up counts
+    bool node = false;
+    switch (a.fr.q) {
+        case 2: {
+            // the asynchronous kernel's rows may leave its blocks half empty
+            const long long nb = node_blocks(a, n_vblk, true), line = (long long)((a.mesh.Ne + 15) / 16) * n_vblk;
+            node = async && (C == 2 || open) &&
+                   (nb <= 2 * sms || (open && nb <= 4 * sms && line >= (C == 2 ? sms : 2 * sms)));
+            break;
+        }
+        case 3: node = waves <= (C == 2 || open ? 1.0 : brief ? 0.25 : 0.0); break;
+        case 4: node = waves <= (C == 2 || (open && !spec) ? 1.05 : !spec ? 0.5 : brief ? 0.25 : 0.0); break;
+        case 5: node = waves <= (C == 2 && (open || spec) ? 2.0 : 1.05); break;
+    }
+    return node ? FORM_NODE : ring ? FORM_RING : FORM_DIRECT;
+}
+
+bool stage_f32_auto_direct(const StageArgs<float> &a, int C, int n_vblk, int depth) {
+    int d = 0;
+    return !a.geo && auto_form(a, C, n_vblk, depth, &d) == FORM_DIRECT;
+}
+
 cudaError_t launch_stage_f32(const StageArgs<float> &a, int C, int n_vblk, int variant, int depth, cudaStream_t s) {
     if (variant >= BGK_STAGE_LINE && variant <= BGK_STAGE_HALF_WIDE)
         return launch_stage_f32_line(a, C, n_vblk, variant - BGK_STAGE_LINE, depth, s);
@@ -746,8 +811,12 @@ cudaError_t launch_stage_f32(const StageArgs<float> &a, int C, int n_vblk, int v
     }
     if (variant == BGK_STAGE_AUTO && !a.geo) {
         int d = 0;
-        if (stage_f32_auto_ring(a, C, &d)) return launch_stage_f32_line(a, C, n_vblk, 0, d, s);
-        if (stage_f32_direct_supported(a)) return launch_stage_f32_direct(a, C, n_vblk, s);
+        switch (auto_form(a, C, n_vblk, depth, &d)) {
+            case FORM_RING: return launch_stage_f32_line(a, C, n_vblk, 0, d, s);
+            case FORM_DIRECT: return launch_stage_f32_direct(a, C, n_vblk, s);
+            default:
+                if (stage_f32_tma_supported(a, C, depth)) return launch_stage_f32(a, C, n_vblk, BGK_STAGE_ASYNC, depth, s);
+        }
     }
     switch (a.fr.q) {
         case 2: return stage32_q<2>(a, C, n_vblk, s);

@@ -73,3 +73,28 @@ def test_tuner_tries_the_direct_form_where_it_is_the_default(lib):
         v, d, ms = s.tune_stage(wl.dt(), reps=1)
         assert v in ("auto", "plain") and ms > 0.0
         assert np.array_equal(s.get_state(), f)
+
+
+# meshes whose node-per-thread grid is above the waves up to which that kernel is
+# the default (below them the test above compares it with itself)
+LARGER = [(1, (5, 4, 3)), (1, (17, 3, 3)), (2, (3, 5, 5)), (2, (13, 5, 1)), (2, (16, 4, 1)), (3, (2, 4, 4)), (3, (7, 4, 1)),
+          (3, (9, 3, 1)), (4, (3, 4, 2)), (4, (5, 5, 1))]
+
+
+@pytest.mark.parametrize("faces", ["periodic", "dirichlet", "specular", "mixed"])
+@pytest.mark.parametrize("delta", [0.0, 2.0])
+@pytest.mark.parametrize("p,mesh_n", LARGER)
+def test_line_kernel_by_default_equals_plain(lib, p, mesh_n, delta, faces):
+    wl = _wl(p, mesh_n, delta, faces)
+    f = W.random_anisotropic_state(wl, seed=35).astype(np.float32)
+    out = []
+    for kernel in ("plain", "auto"):
+        with lib.Solver(wl, lib.BGK_MIXED) as s:
+            s.set_velocity_blocks(s.velocity_blocks()[2])
+            s.set_stage_kernel(kernel)
+            s.set_state(f)
+            r = s.rhs(f)
+            assert s.step(wl.dt(), 2) == lib.BGK_OK
+            out.append((r, s.get_state(), s.moments()))
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
