@@ -33,11 +33,10 @@ __device__ __forceinline__ float2 psub(float2 x, float2 y) { return __ffma2_rn(y
 // R = -div + (g' - f)/tau.  g' = exp(c0) * exp2(-log2(e)/2 c^T A c) with the
 // per-point factor exp(c0) from FP64 and the exponent in FP32.
 //
-// Curvilinear elements (CURV; p = 4 with F and G only, where the line kernel of
-// kernels_f32_curved.cu spills: 1.85 against 2.9 ms per stage on 48 warped
-// elements, 18^3 velocities): the transformed-flux form of the FP64 stage
-// kernel (kernels_f64.cu) in FP32, regrouped so that every rounding acts on
-// deviations (see CurvOps32).  a_d = u . S^d per node is staged beside f; per
+// Curvilinear elements (CURV; small meshes, and p = 4 with F and G, see
+// curved_node): the transformed-flux form of the FP64 stage kernel
+// (kernels_f64.cu) in FP32, regrouped so that every rounding acts on deviations
+// (see CurvOps32).  a_d = u . S^d per node is staged beside f; per
 // direction, with w_j = a_j (f_j - f_i),
 //   t_i = sum_{j != i} D_ij w_j - sum_j def_j w_j
 //       + g_R'_i (A_R dev_R - sum_j l_j(+1) w_j) + g_L'_i (A_L dev_L - sum_j l_j(-1) w_j),
@@ -372,6 +371,60 @@ __global__ void __launch_bounds__(256, BGK_PLAIN_MINB) k_stage_f32(StageArgs<flo
                     const float *sfc = sf[buf][c];
                     const float fi = fself[c];
                     float div = 0.f;
+                    if constexpr (CURV) {
+#pragma unroll
+                        for (int d = 0; d < 3; ++d) {
+                            const float *own = sfc + le * NS + base[d];
+                            const float *ownA = sA[buf][d] + le * NS + base[d];
+                            float dF = 0.f, E = 0.f, trL = 0.f, trR = 0.f, fmL = 0.f, fmR = 0.f;
+#pragma unroll
+                            for (int m = 1; m < Q; ++m) {
+                                const int j = (id[d] + m) % Q;
+                                const float dfj = own[j * stride[d]] - fi;
+                                const float wj = ownA[j * stride[d]] * dfj;
+                                dF = fmaf(cD[id[d]][j], wj, dF);
+                                E = fmaf(cdef[j], wj, E);
+                                trL = fmaf(cl[1][j], wj, trL);
+                                trR = fmaf(cl[0][j], wj, trR);
+                                fmL = fmaf(cl[1][j], dfj, fmL);
+                                fmR = fmaf(cl[0][j], dfj, fmR);
+                            }
+                            float X[2];
+#pragma unroll
+                            for (int side = 0; side < 2; ++side) {
+                                const int fpi = d == 0 ? id[1] + Q * id[2] : (d == 1 ? id[0] + Q * id[2] : id[0] + Q * id[1]);
+                                const float A = sAf[buf][(le * 6 + 2 * d + side) * Q * Q + fpi];
+                                const float un = side ? A : -A;           // outward
+                                const int en = en_[d][side];
+                                const int kind = a.mesh.face_kind[2 * d + side];
+                                float dev;
+                                if (en < 0 && kind == BGK_FK_CLOSED) {
+                                    dev = -fi;                            // F^I = 0
+                                } else if (un > 0.f) {
+                                    dev = side ? fmR : fmL;
+                                } else if (en >= e0 && en < e0 + EB) {
+                                    const float *nb = sfc + (en - e0) * NS + base[d];
+                                    dev = 0.f;
+#pragma unroll
+                                    for (int j = 0; j < Q; ++j) dev = fmaf(cl[side][j], nb[j * stride[d]] - fi, dev);
+                                } else if (en >= 0) {
+                                    const float *nb = fs + (size_t)en * NS + base[d];
+                                    dev = 0.f;
+#pragma unroll
+                                    for (int j = 0; j < Q; ++j) dev = fmaf(cl[side][j], __ldg(nb + j * stride[d]) - fi, dev);
+                                } else {
+                                    double fpd = __ldg(a.bcval + ((size_t)(2 * d + side) * C + c) * a.Nu + k);
+                                    if (kind == BGK_FK_DIFFUSE)
+                                        fpd *= __ldg(a.rho_w + ((size_t)e * 6 + 2 * d + side) * Q * Q + fpi);
+                                    dev = (float)fpd - fi;
+                                }
+                                X[side] = fmaf(A, dev, -(side ? trR : trL));
+                            }
+                            div += fmaf(X[1], cg[1][id[d]], fmaf(X[0], cg[0][id[d]], dF - E));
+                        }
+                        div = fmaf(fi, fmaf(u[0], sG[tid][9], fmaf(u[1], sG[tid][10], u[2] * sG[tid][11])), div);
+                        div *= sG[tid][12];
+                    } else {
 #pragma unroll
                     for (int d = 0; d < 3; ++d) {
                         const int side = u[d] > 0.f ? 0 : 1;
@@ -411,6 +464,7 @@ __global__ void __launch_bounds__(256, BGK_PLAIN_MINB) k_stage_f32(StageArgs<flo
                         }
                         t = fmaf(sdg[side][id[d]], dn, fmaf(seps[side][id[d]], fi, t));
                         div = fmaf(toh[d] * u[d], t, div);
+                    }
                     }
                     const float eqv = (c == 0) ? g32 : __fmul_rn(gfac, g32);
                     const float eqc = (c == 0) ? gc : __fmul_rn(gfac, gc);
@@ -649,33 +703,75 @@ __global__ void k_maxwellian_f32(float *f, const double *qin, const double *vtab
 
 }  // namespace
 
+// Blocks of the node-per-thread kernels (256 threads of whole elements; the
+// asynchronous one keeps to element rows).
+static long long node_blocks(const StageArgs<float> &a, int n_vblk, bool async) {
+    const int eb = 256 / (a.fr.q * a.fr.q * a.fr.q);
+    const long long n = async ? (long long)((a.mesh.n[0] + eb - 1) / eb) * a.mesh.n[1] * a.mesh.n[2] : (a.mesh.Ne + eb - 1) / eb;
+    return n * n_vblk;
+}
+
+static int multiprocessors() {
+    int dev = 0, sms = 0;
+    const bool ok = cudaGetDevice(&dev) == cudaSuccess &&
+                    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+    return ok ? sms : 152;
+}
+
+// Whether a curvilinear mesh runs on the node-per-thread kernel: while its grid
+// leaves the GPU half empty, more threads per element hide more latency than the
+// line-group kernel's fewer instructions save, and where a velocity block is a
+// line or two (Kblk), that kernel's work per line counts.  Line-group against
+// node-per-thread, us per stage, periodic warped boxes:
+//   p = 1, one component, 8^3: 8 elements 28.0 / 22.9, 64: 30.9 / 30.2; 16^3 and up the
+//     line-group kernel (24^3: 1.1 to 1.9 times faster)
+//   p = 1, F and G, 16^3: 8 elements (one warp per block) 102 / 87, 64: 1.0;
+//     O-grid 16 elements, 38 x 36 x 40: 1.3 times faster
+//   p = 2, one component, 24^3: 1 element 269 / 252, 9: 1.06 times faster; F and G: 8 elements
+//     444 / 318, 36: 676 / 608, 48: 1.7 times faster; O-grid 32 elements: 0.87
+//   p = 3, F and G, 16^3: 8 elements 153 / 129, 12: 1.0; one component 8^3: 31 / 23
+//   p = 4, one component, 16^3: 8 elements 200 / 181, 12: 1.5 times faster; with F and G,
+//     where the line-group kernel spills, 48 elements at 18^3 2900 / 1850
+static bool curved_node(const StageArgs<float> &a, int C, int n_vblk) {
+    const double waves = (double)node_blocks(a, n_vblk, false) / (2.0 * multiprocessors());
+    const bool brief = a.Kblk <= 24;                     // velocities of a block
+    switch (a.fr.q) {
+        case 2:
+            if (!a.mesh.periodic[0] || !a.mesh.periodic[1] || !a.mesh.periodic[2]) return false;
+            return C == 1 ? brief && waves <= 0.25 : (a.mesh.Ne <= 16 && waves <= 0.25) || (brief && waves <= 0.5);
+        case 3: return waves <= (C == 2 ? 0.9 : 0.25);
+        case 4: return waves <= (C == 2 || brief ? 0.45 : 0.25);
+        default: return C == 2 || waves <= 0.95;
+    }
+}
+
+template <int Q, int C>
+static cudaError_t stage32_curved_node(const StageArgs<float> &a, dim3 grid, cudaStream_t s) {
+    constexpr int NS = Q * Q * Q, EB = 256 / NS;
+    // the curvilinear instantiations' moment accumulators (dynamic shared memory)
+    const size_t dyn = (size_t)EB * NS * (11 * sizeof(double) + 14 * sizeof(float));
+    static SmemLimit lim;
+    size_t *attr = lim.slot();
+    if (!attr) return cudaErrorInvalidDevice;
+    if (dyn > *attr) {
+        const cudaError_t e = cudaFuncSetAttribute(k_stage_f32<Q, C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+        if (e != cudaSuccess) return e;
+        *attr = dyn;
+    }
+    k_stage_f32<Q, C, true><<<grid, EB * NS, dyn, s>>>(a);
+    return cudaGetLastError();
+}
+
 template <int Q>
 static cudaError_t stage32_q(const StageArgs<float> &a, int C, int n_vblk, cudaStream_t s) {
     constexpr int NS = Q * Q * Q, EB = 256 / NS;
     dim3 grid((a.mesh.Ne + EB - 1) / EB, n_vblk);
     if (a.geo) {
-        if constexpr (Q == 5) {
-            if (C == 2) {
-                // the curvilinear instantiation's moment accumulators (dynamic shared memory)
-                const size_t dyn = (size_t)EB * NS * (11 * sizeof(double) + 14 * sizeof(float));
-                static SmemLimit lim;
-                size_t *attr = lim.slot();
-                if (!attr) return cudaErrorInvalidDevice;
-                if (dyn > *attr) {
-                    const cudaError_t e =
-                        cudaFuncSetAttribute(k_stage_f32<Q, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-                    if (e != cudaSuccess) return e;
-                    *attr = dyn;
-                }
-                k_stage_f32<Q, 2, true><<<grid, EB * NS, dyn, s>>>(a);
-                return cudaGetLastError();
-            }
-        }
-        return launch_stage_f32_curved(a, C, n_vblk, s);
-    } else {
-        if (C == 1) k_stage_f32<Q, 1, false><<<grid, EB * NS, 0, s>>>(a);
-        else k_stage_f32<Q, 2, false><<<grid, EB * NS, 0, s>>>(a);
+        if (!curved_node(a, C, n_vblk)) return launch_stage_f32_curved(a, C, n_vblk, s);
+        return C == 1 ? stage32_curved_node<Q, 1>(a, grid, s) : stage32_curved_node<Q, 2>(a, grid, s);
     }
+    if (C == 1) k_stage_f32<Q, 1, false><<<grid, EB * NS, 0, s>>>(a);
+    else k_stage_f32<Q, 2, false><<<grid, EB * NS, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -734,21 +830,6 @@ bool stage_f32_variant_supported(const StageArgs<float> &a, int C, int variant, 
         case BGK_STAGE_HALF_WIDE: return stage_f32_line_supported(a, C, variant - BGK_STAGE_LINE, depth);
         default: return false;
     }
-}
-
-// Blocks of the node-per-thread kernels (256 threads of whole elements; the
-// asynchronous one keeps to element rows).
-static long long node_blocks(const StageArgs<float> &a, int n_vblk, bool async) {
-    const int eb = 256 / (a.fr.q * a.fr.q * a.fr.q);
-    const long long n = async ? (long long)((a.mesh.n[0] + eb - 1) / eb) * a.mesh.n[1] * a.mesh.n[2] : (a.mesh.Ne + eb - 1) / eb;
-    return n * n_vblk;
-}
-
-static int multiprocessors() {
-    int dev = 0, sms = 0;
-    const bool ok = cudaGetDevice(&dev) == cudaSuccess &&
-                    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
-    return ok ? sms : 152;
 }
 
 // Which kernel BGK_STAGE_AUTO runs on a box.  While the node-per-thread kernels

@@ -72,3 +72,24 @@ def test_unaligned_caller_buffers(lib, p, delta):
         s.stage(off(g), off(f), b, 0.75, 0.25, 0.25 * wl.dt())
     assert float((a - b).abs().max()) <= 8 * 2.0 ** -24 * float(f.abs().max())
     assert not torch.equal(a, f)
+
+
+def _larger_wl(p, delta, walls):
+    n = {1: (13, 5, 1), 2: (3, 13, 1), 3: (3, 3, 1), 4: (3, 4, 1)}[p]
+    wl = W.wavy_periodic_box(p=p, n=n, vel_n=(9, 8, 7), amp=0.06, Pr=0.72).replace(delta=delta)
+    if walls:
+        wl = wl.replace(periodic=(False, True, True), diffuse={(0, -1): ((0.0, 0.2, 0.0), 0.8)},
+                        dirichlet={(0, 1): (1.1, (0.1, 0.0, -0.1), 1.2)})
+    return wl
+
+
+@pytest.mark.parametrize("walls", [False, True])
+@pytest.mark.parametrize("delta", [0.0, 2.0])
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+def test_meshes_above_the_node_per_thread_range(lib, p, delta, walls, monkeypatch):
+    """The tests above on meshes that the line-group kernel runs whatever their
+    faces and components (p = 4 with F and G excepted)."""
+    monkeypatch.setitem(globals(), "_wl", _larger_wl)
+    test_curved_rhs_matches_oracle(lib, p, delta, walls)
+    if walls and p in (1, 3):
+        test_unaligned_caller_buffers(lib, p, delta)
