@@ -855,10 +855,12 @@ bgk_status create_ctx(bgk_ctx **out, const bgk_mesh_desc *mesh, const bgk_vgrid_
         if (st == BGK_OK) cu(cudaMalloc(&ctx->rho_w, (size_t)ctx->Ne * 6 * ctx->q * ctx->q * sizeof(double)), "cudaMalloc(rho_w)");
         if (st == BGK_OK && ctx->n_wall) cu(cudaMalloc(&ctx->wall_ef, wall_h.size() * sizeof(int)), "cudaMalloc(wall)");
         if (st == BGK_OK && precision == BGK_MIXED) {
-            std::vector<float> gp;
-            curved_geop(q, g32.data(), f32.data(), ctx->mesh, ctx->cops, gp);
-            cu(cudaMalloc(&ctx->geop, gp.size() * sizeof(float)), "cudaMalloc(geop)");
-            if (st == BGK_OK) cu(cudaMemcpy(ctx->geop, gp.data(), gp.size() * sizeof(float), cudaMemcpyHostToDevice), "upload geop");
+            if (q < 5 || ctx->C == 1) {                  // p = 4 with F and G has no line-group kernel
+                std::vector<float> gp;
+                curved_geop(q, g32.data(), f32.data(), ctx->mesh, ctx->cops, gp);
+                cu(cudaMalloc(&ctx->geop, gp.size() * sizeof(float)), "cudaMalloc(geop)");
+                if (st == BGK_OK) cu(cudaMemcpy(ctx->geop, gp.data(), gp.size() * sizeof(float), cudaMemcpyHostToDevice), "upload geop");
+            }
             std::vector<float2> b2(bcv.size());
             for (size_t i = 0; i < bcv.size(); ++i) b2[i] = make_float2((float)bcv[i], (float)(bcv[i] - (double)(float)bcv[i]));
             const size_t nw = (size_t)ctx->Ne * 6 * ctx->q * ctx->q * sizeof(float2);

@@ -93,3 +93,19 @@ def test_meshes_above_the_node_per_thread_range(lib, p, delta, walls, monkeypatc
     test_curved_rhs_matches_oracle(lib, p, delta, walls)
     if walls and p in (1, 3):
         test_unaligned_caller_buffers(lib, p, delta)
+
+
+def test_no_line_group_geometry_where_no_kernel_reads_it(lib):
+    """p = 4 with F and G runs on the node-per-thread kernel: its context holds the
+    second component's state beyond a one-component context, not 31 KB per element."""
+    import torch
+    used = {}
+    for delta in (0.0, 2.0):
+        wl = W.wavy_periodic_box(p=4, n=(10, 10, 10), vel_n=(2, 2, 2), amp=0.03, Pr=0.72).replace(delta=delta)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        s = lib.Solver(wl, lib.BGK_MIXED)
+        used[delta] = free - torch.cuda.mem_get_info()[0]
+        s.destroy()
+    state = 3 * 1000 * 125 * 8 * 4
+    assert used[2.0] <= used[0.0] + state - 1000 * 31000 + (8 << 20)
