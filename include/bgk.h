@@ -253,12 +253,15 @@ BGK_API bgk_status bgk_set_qprime_engine(bgk_ctx *ctx, int fp32_sums);
  *   4 line, runs twice as long;
  *   5 half: the same copy ring, one thread per half first-axis node line;
  *   6 half, runs twice as long.
- * depth: 2..16 copy-ring stages (default 6).  Variants 2-6 need p = 1 or 3
- * (element slabs of whole 16-byte units) and 16-byte aligned state buffers
- * (bgk_stage runs caller buffers that are not on the plain kernel); every
- * wait in them is bounded and a wait that gives up makes the next status
- * check return BGK_ETIMEOUT.  Errors: BGK_EINVAL (range), BGK_ENOTSUP
- * (variants 2-6 on the FP64 form or an unsupported order). */
+ * depth: 2..16 copy-ring stages (default 6) of variants 2-6, and of variant 0
+ * where it runs variant 2.  Variants 2-6 need 16-byte aligned state buffers and
+ * element slabs of whole 16-byte units: p = 1 or 3; variant 3 also takes p = 2
+ * with rows of whole 4-element groups.  Caller buffers of bgk_stage that a
+ * variant cannot take run as the default would for them.  Every wait of a copy
+ * ring (variants 2-6, and 0 where it has one) is bounded; a wait that gives up
+ * makes the next status check return BGK_ETIMEOUT.  Errors: BGK_EINVAL (range),
+ * BGK_ENOTSUP (variants 2-6 on the FP64 form, on a mesh or an order they do not
+ * take). */
 BGK_API bgk_status bgk_set_stage_kernel(bgk_ctx *ctx, int variant, int depth);
 
 /* Velocity blocking of the stage and moment kernels: the velocities are
@@ -277,7 +280,8 @@ BGK_API bgk_status bgk_set_velocity_blocks(bgk_ctx *ctx, int n);
  * Errors: BGK_EINVAL (NULL context). */
 BGK_API bgk_status bgk_get_velocity_blocks(const bgk_ctx *ctx, int *n_blocks, int *per_block, int *max_blocks);
 
-/* Test entry for the bounded waits of the copy-ring kernels (variants 2-6):
+/* Test entry for the bounded waits of the copy-ring kernels (variants 2-6, and 0
+ * where it runs one of them; without effect on the others):
  * with after > 0 every block's ring delivers only its first `after`
  * velocities and stops, so the consumers' next wait runs out, after
  * wait_seconds (0: about 2 s) instead of about 2 s; the kernel then lets its

@@ -399,7 +399,7 @@ bgk_status run_stage(bgk_ctx *ctx, const void *fn, const void *fs, void *fo, dou
                             ctx->stream));
     else {
         const StageArgs<float> sa = stage_args<float>(ctx, fn, fs, fo, a, b, c, moments);
-        // caller buffers that a chosen variant cannot take (alignment) run on the plain kernel
+        // caller buffers that a chosen variant cannot take (alignment) run on what the default is for them
         const int v = stage_f32_variant_supported(sa, ctx->C, ctx->stage_variant, ctx->stage_depth) ? ctx->stage_variant
                                                                                                    : BGK_STAGE_AUTO;
         CU(launch_stage_f32(sa, ctx->C, ctx->n_vblk, v, ctx->stage_depth, ctx->stream));
@@ -1094,7 +1094,8 @@ bgk_status bgk_set_stage_kernel(bgk_ctx *ctx, int variant, int depth) {
         const StageArgs<float> a = stage_args<float>(ctx, ctx->f[0], ctx->f[1], ctx->f[2], 0.5, 0.5, 1.0, true);
         if (!stage_f32_variant_supported(a, ctx->C, variant, depth))
             return fail(ctx, BGK_ENOTSUP, "asynchronous-copy stage kernels need the uniform box mesh (no specular, "
-                                          "diffuse or closed faces), p = 1 or 3 and fitting shared memory");
+                                          "diffuse or closed faces), p = 1 or 3 (line: also p = 2 with rows of "
+                                          "whole 4-element groups) and fitting shared memory");
     }
     ctx->stage_variant = variant;
     ctx->stage_depth = depth;

@@ -37,10 +37,12 @@
 // Stage of the sphere O-grid with 6 x 12 x 12 elements, p = 1, 40^3 velocities, F
 // and G (4.4e8 points x velocities): 17.1 -> 5.8 ms (1.6 TB/s, 24% of HBM), 195
 // instructions per node, 34% of the issue slots: eight warps per SM (registers
-// and shared memory) do not cover the instruction latencies.  Warped box, p = 2,
-// one component: 1.17 -> 0.58 ms.
-// Moments are the line kernel's: error-free line sums, plane pairs in shared
-// memory, FP64 index moments in the partials buffer.
+// and shared memory) do not cover the instruction latencies.  Warped box 6x5x6,
+// p = 2, one component, 20^3: 1.17 -> 0.58 ms.  Small meshes keep the node-per-
+// thread kernel (curved_node in kernels_f32.cu).
+// Moments are the line kernel's: error-free line sums, plane pairs in
+// thread-local memory (touched once per velocity line), FP64 index moments in the
+// partials buffer.
 // Dzanic & Martinelli, arXiv 2312.06567, section "Numerical method".
 
 #include "stage_f32_common.cuh"

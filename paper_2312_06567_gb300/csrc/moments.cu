@@ -49,7 +49,7 @@ __device__ __forceinline__ void plane_add2(float2 &P, float2 &Pe, float c, float
 template <int C>
 __global__ void __launch_bounds__(MT, 3) k_moments_f32(const float *f, double *part, VelGrid vg, int Nu, int P, int Kblk) {
     constexpr int NL = C == 2 ? 4 : 3, NQ = C == 2 ? 7 : 6;
-    constexpr int MCH = C == 2 ? 4 : 8;                  // with G, eight would spill
+    constexpr int MCH = C == 2 ? 4 : 8;                  // with G, eight spill 384 bytes, four 156
     const int pa = blockIdx.x * (2 * MT) + threadIdx.x, pb = pa + MT;
     if (pa >= P) return;
     const bool two = pb < P;
