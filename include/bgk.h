@@ -236,9 +236,9 @@ BGK_API bgk_status bgk_set_qprime_engine(bgk_ctx *ctx, int fp32_sums);
 /* Kernel of the mixed-form stage (the fused step of section "Methodology":
  * FR advection, BGK source, Runge--Kutta update and the moments of the
  * result).  All variants compute the same values bit for bit.
- *   0 (default) by the mesh.  On boxes, while a thread per node fills the GPU
- *     no more than once: variant 2 where it applies (at `depth`), else 1;
- *     beyond that the line kernel, on its copy ring (of a depth of its own)
+ *   0 (default) by the mesh.  On boxes too small to fill the GPU (by a rule on
+ *     elements, order, faces and velocities) variant 2 where it applies, at
+ *     `depth`, else 1; on others the line kernel, on its copy ring (of a depth of its own)
  *     where the element runs are whole 16-byte units and mostly full, else
  *     reading its operands directly (any order and face; 16-byte aligned
  *     buffers at p = 3, 8-byte at p = 1, else any).  On curvilinear meshes

@@ -311,7 +311,7 @@ void set_geometry<double>(bgk_ctx *ctx, StageArgs<double> &s) {
 template <>
 void set_geometry<float>(bgk_ctx *ctx, StageArgs<float> &s) {
     s.geo = ctx->geo32; s.fvec = ctx->fvec32; s.geop = ctx->geop; s.rho_w = ctx->rho_w;
-    s.rho_w2 = ctx->rho_w2; s.bc2 = ctx->bc2;
+    s.rho_w2 = ctx->rho_w2;
     s.cops = ctx->cops;
 }
 
@@ -376,6 +376,7 @@ StageArgs<T> stage_args(bgk_ctx *ctx, const void *fn, const void *fs, void *fo, 
     s.wait_ns = ctx->wait_ns;
     s.ring_limit = ctx->ring_limit;
     for (int d = 0; d < 3; ++d) s.toh32[d] = (float)ctx->mesh.two_over_h[d];
+    s.bc2 = ctx->bc2;
     if (ctx->curved) set_geometry<T>(ctx, s);
     return s;
 }
@@ -777,6 +778,12 @@ bgk_status create_ctx(bgk_ctx **out, const bgk_mesh_desc *mesh, const bgk_vgrid_
     if (st == BGK_OK) cu(cudaMalloc(&ctx->iters, P * sizeof(int)), "cudaMalloc(iters)");
     if (st == BGK_OK) cu(cudaMalloc(&ctx->vtab, ctx->vtab_h.size() * sizeof(double)), "cudaMalloc(vtab)");
     if (st == BGK_OK) cu(cudaMalloc(&ctx->bcval, bcv.size() * sizeof(double)), "cudaMalloc(bcval)");
+    if (st == BGK_OK && precision == BGK_MIXED) {
+        std::vector<float2> b2(bcv.size());
+        for (size_t i = 0; i < bcv.size(); ++i) b2[i] = make_float2((float)bcv[i], (float)(bcv[i] - (double)(float)bcv[i]));
+        cu(cudaMalloc(&ctx->bc2, b2.size() * sizeof(float2)), "cudaMalloc(bc2)");
+        if (st == BGK_OK) cu(cudaMemcpy(ctx->bc2, b2.data(), b2.size() * sizeof(float2), cudaMemcpyHostToDevice), "upload bc2");
+    }
     std::vector<float4> v32(Nu);
     for (int k = 0; k < Nu; ++k) {
         const double *v = &ctx->vtab_h[(size_t)k * BGK_VTAB];
@@ -861,12 +868,8 @@ bgk_status create_ctx(bgk_ctx **out, const bgk_mesh_desc *mesh, const bgk_vgrid_
                 cu(cudaMalloc(&ctx->geop, gp.size() * sizeof(float)), "cudaMalloc(geop)");
                 if (st == BGK_OK) cu(cudaMemcpy(ctx->geop, gp.data(), gp.size() * sizeof(float), cudaMemcpyHostToDevice), "upload geop");
             }
-            std::vector<float2> b2(bcv.size());
-            for (size_t i = 0; i < bcv.size(); ++i) b2[i] = make_float2((float)bcv[i], (float)(bcv[i] - (double)(float)bcv[i]));
             const size_t nw = (size_t)ctx->Ne * 6 * ctx->q * ctx->q * sizeof(float2);
-            if (st == BGK_OK) cu(cudaMalloc(&ctx->bc2, b2.size() * sizeof(float2)), "cudaMalloc(bc2)");
             if (st == BGK_OK) cu(cudaMalloc(&ctx->rho_w2, nw), "cudaMalloc(rho_w2)");
-            if (st == BGK_OK) cu(cudaMemcpy(ctx->bc2, b2.data(), b2.size() * sizeof(float2), cudaMemcpyHostToDevice), "upload bc2");
             if (st == BGK_OK) cu(cudaMemset(ctx->rho_w2, 0, nw), "memset rho_w2");
         }
         if (st == BGK_OK) cu(cudaMemcpy(ctx->geo, ctx->geo_h.data(), ng * sizeof(double), cudaMemcpyHostToDevice), "upload geo");

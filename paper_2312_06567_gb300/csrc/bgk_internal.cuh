@@ -122,6 +122,14 @@ __device__ __forceinline__ int mirror_velocity(int k, int d, const int n[3]) {
     return m1 + n[0] * (m2 + n[1] * m3);
 }
 
+// Multiprocessors of the current device, for the launch rules that count waves.
+inline int multiprocessors() {
+    int dev = 0, sms = 0;
+    const bool ok = cudaGetDevice(&dev) == cudaSuccess &&
+                    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+    return ok ? sms : 152;
+}
+
 // FP32 equilibrium exactly as the mixed-form stage evaluates it:
 // g32(u) = E0 * exp2(L), L = -log2(e)/2 c^T A c, c = u - V, all in FP32 with
 // every product rounded explicitly (no contraction), so the Q' kernel can

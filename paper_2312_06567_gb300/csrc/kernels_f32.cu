@@ -711,13 +711,6 @@ static long long node_blocks(const StageArgs<float> &a, int n_vblk, bool async) 
     return n * n_vblk;
 }
 
-static int multiprocessors() {
-    int dev = 0, sms = 0;
-    const bool ok = cudaGetDevice(&dev) == cudaSuccess &&
-                    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
-    return ok ? sms : 152;
-}
-
 // Whether a curvilinear mesh runs on the node-per-thread kernel: while its grid
 // leaves the GPU half empty, more threads per element hide more latency than the
 // line-group kernel's fewer instructions save, and where a velocity block is a
@@ -836,21 +829,20 @@ bool stage_f32_variant_supported(const StageArgs<float> &a, int C, int variant, 
 // (asynchronous where it applies, else plain) fit the GPU in one wave of two
 // blocks per multiprocessor, every node has a thread of its own at once, and a
 // velocity costs the latency of one node; the line kernel's threads walk p + 1
-// nodes each, and its fewer warps hide less.  Beyond one wave the line kernel's
-// smaller instruction count wins.  Measured (us per stage, line kernel / the
-// other; 152 multiprocessors, up to 64 velocity blocks):
-//   p = 4, F and G, x faces Dirichlet, 24^3   8 elements 1169 / 565, 12: 1473 / 1196,
-//     18: 2.0 waves, 0.90 of the other's speed, 24: 1.06; periodic from one wave on 1.01
-//   p = 4, one component, 24^3                8 elements 630 / 533, 12: 1.47 times faster
-//   p = 3, F and G, 24^3                      8 elements 600 / 297, 12: 493 / 361, 24: 1.16
-//   p = 3, one component, periodic            8 elements 0.92, 9: 1.08; Dirichlet 16: 0.91, 24: 1.43
-//   p = 2, Dirichlet, 24^3                    8 elements 245 / 213, 36: 0.95, 64: 1.89;
-//     F and G, periodic: 36 elements 0.93, 64: 1.96; one component, periodic: 1.0 to 1.5
-//   p = 1, F and G, 33 x 28 x 26              27 elements 936 / 420, 64: 998 / 1609
-//   p = 1, one component, Dirichlet, 24^3     27 elements 180 / 154, 48: 182 / 455; periodic 0.98 to 5
-//   specular faces (the other is the plain kernel): p = 3, one component 1.2, F and G 0.8
-//     below one wave; p <= 2 above 1
-//   blocks of a line or two, p = 2, one component, periodic, 8^3: 4 elements 26.5 / 23.3
+// nodes each, and its fewer warps hide less (the more so where it spills).
+// Beyond one wave its smaller instruction count wins.  At p = 1 it wins there too,
+// unless the state is too large for the L2 to hold input, f^n and output, whose
+// latency only the asynchronous copies cover.  Measured (us per stage, line kernel
+// / the other; 152 multiprocessors, up to 64 velocity blocks, 24^3 velocities):
+//   p = 4, F and G, x faces Dirichlet      8 elements 817 / 521, 12: 1203 / 1202, 24: 1236 / 1762
+//   p = 4, one component                   8 elements 550 / 441, 12: 713 / 1155
+//   p = 3, F and G, periodic               8 elements 421 / 286, 16: 499 / 371, 24: 537 / 619
+//   p = 3, one component, Dirichlet        16 elements 258 / 235, 24: 287 / 412
+//   p = 3, one component, periodic         8 elements 208 / 191, 9: 216 / 235; specular 1.1 to 1.3 times faster
+//   p = 2, F and G, Dirichlet              8 elements 319 / 269, 36: 534 / 499, 64: 542 / 1017
+//   p = 2, one component                   0.95 to 1.9 times the other's speed
+//   p = 2 and 3, blocks of a line or two   4 elements, 8^3: 27 / 23; 2 elements, specular: 37 / 32
+//   p = 1, F and G, 43 elements            33 x 28 x 26 (66 MB) 592 / 423, 16 x 15 x 14 76 / 81
 enum { FORM_NODE, FORM_RING, FORM_DIRECT };
 static int auto_form(const StageArgs<float> &a, int C, int n_vblk, int depth, int *ring_depth) {
     const bool ring = stage_f32_auto_ring(a, C, ring_depth);
@@ -858,21 +850,18 @@ static int auto_form(const StageArgs<float> &a, int C, int n_vblk, int depth, in
     const int sms = multiprocessors();
     bool open = false;                                   // some face holds a Dirichlet state
     for (int f = 0; f < 6; ++f) open |= !a.mesh.periodic[f / 2] && !a.mesh.specular[f];
-    const bool async = stage_f32_tma_supported(a, C, depth), spec = any_specular(a.mesh);
+    const bool spec = any_specular(a.mesh);
     const double waves = (double)node_blocks(a, n_vblk, false) / (2.0 * sms);
-    const bool brief = a.Kblk <= 24;                     // a block's velocities are a line or two, whose set-up counts
     bool node = false;
-    switch (a.fr.q) {
-        case 2: {
-            // the asynchronous kernel's rows may leave its blocks half empty
-            const long long nb = node_blocks(a, n_vblk, true), line = (long long)((a.mesh.Ne + 15) / 16) * n_vblk;
-            node = async && (C == 2 || open) &&
-                   (nb <= 2 * sms || (open && nb <= 4 * sms && line >= (C == 2 ? sms : 2 * sms)));
-            break;
-        }
-        case 3: node = waves <= (C == 2 || open ? 1.0 : brief ? 0.25 : 0.0); break;
-        case 4: node = waves <= (C == 2 || (open && !spec) ? 1.05 : !spec ? 0.5 : brief ? 0.25 : 0.0); break;
-        case 5: node = waves <= (C == 2 && (open || spec) ? 2.0 : 1.05); break;
+    if (a.fr.q == 2) {
+        node = 4.0 * C * a.Nu * a.P > 30.0e6 && stage_f32_tma_supported(a, C, depth) && node_blocks(a, n_vblk, true) <= 2 * sms;
+    } else {
+        double most = 1.05;                              // waves up to which the node-per-thread kernels run
+        if (a.fr.q == 3) most = C == 1 || spec ? 0.0 : open ? 1.05 : 0.3;
+        if (a.fr.q == 4 && C == 1) most = spec ? 0.0 : open ? 1.05 : 0.5;
+        if (a.fr.q == 5 && C == 2 && open) most = 1.7;   // (spills most: 15 elements 1100 / 1043)
+        if (a.Kblk <= 24 && most < 0.5) most = 0.5;      // a block's velocities are a line or two, whose set-up counts
+        node = waves <= most;
     }
     return node ? FORM_NODE : ring ? FORM_RING : FORM_DIRECT;
 }

@@ -263,8 +263,10 @@ __device__ __forceinline__ void add_pair(LineAcc<C> &A, LineAcc<C> &B, float cj1
 // 10,560 velocities).  A reflecting face is no case of its own there: its upwind
 // operand is the element itself at the mirrored velocity, so the threads of a
 // warp differ in an address and a row of weights, not in a branch (1107 us with
-// a branch per direction).  On the ring the pointers would cost 1.6% (p = 2, F
-// and G), so it keeps offsets.
+// a branch per direction).  At a Dirichlet face the sum is formed all the same and
+// replaced: loads inside a branch wait for the branch before them (octant, p = 2:
+// 829 -> 636 us; p = 1, see `exterior`).  On the ring the pointers would cost 1.6%
+// (p = 2, F and G), so it keeps offsets.
 template <int Q, int C, int EB, int NPT, bool BC, bool RING = true>
 __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, EB, NPT>::MINB) k_stage_f32_line(StageArgs<float> a, int S) {
     using SG = StageGeom<Q, C, EB>;
@@ -357,11 +359,24 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
         const int ec[3] = {el % n1, (el / n1) % n2, el / (n1 * n2)}, es[3] = {1, n1, n1 * n2}, nn[3] = {n1, n2, n3};
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            nbo[2 * d] = ec[d] > 0 ? -es[d] : (nn[d] - 1) * es[d];
-            nbo[2 * d + 1] = ec[d] < nn[d] - 1 ? es[d] : -(nn[d] - 1) * es[d];
+            // (at a boundary face the element itself: its values are in cache, and not used)
+            const bool per = !BC || a.mesh.periodic[d];
+            nbo[2 * d] = ec[d] > 0 ? -es[d] : per ? (nn[d] - 1) * es[d] : 0;
+            nbo[2 * d + 1] = ec[d] < nn[d] - 1 ? es[d] : per ? -(nn[d] - 1) * es[d] : 0;
             if (BC && !a.mesh.periodic[d]) bcm |= (ec[d] == 0 ? 1 << 2 * d : 0) | (ec[d] == nn[d] - 1 ? 2 << 2 * d : 0);
         }
     }
+    // Value of the Dirichlet state on face f, component c, at velocity k, in FP32.
+    // Without the ring, at p = 1 and 3, every thread reads one (any, where it has no
+    // such face) and selects afterwards: a branch per direction and component keeps
+    // the next direction's loads behind it (p = 1, F and G, 200 elements, 24^3, x faces
+    // Dirichlet: 580 -> 385 us; p = 3, F and G, specular: 1.19 times faster).  At odd Q
+    // the values' registers cost more (p = 2, F and G: 0.88 of the speed).
+    constexpr bool SEL = BC && !RING && Q % 2 == 0;
+    auto exterior = [&](bool ext, int f, int c, int k) {
+        const size_t i = ((size_t)f * C + c) * a.Nu + k;
+        return RING ? (float)__ldg(a.bcval + i) : __ldg(&a.bc2[ext || !SEL ? i : 0].x);
+    };
     const int own_off = (l + SG::PAD) * NS;              // own element within a component's stage region
     const int ln = Q * r;                                // own line within an element
     const bool mom = a.part != nullptr;
@@ -478,9 +493,9 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                 const float u1 = su1c[j1].x;
                 const int sx = u1 > 0.f ? 0 : 1;
                 const int o_own = RING ? own_off : 0;
-                const int o_x = RING ? own_off + (sx ? NS : -NS) : nbo[RING ? 0 : sx] * NS;
-                const int o_y = RING ? (SLOTS + l) * NS : nbo[RING ? 0 : 2 + sy] * NS;
-                const int o_z = RING ? (SLOTS + EB + l) * NS : nbo[RING ? 0 : 4 + sz] * NS;
+                const int o_x = RING ? own_off + (sx ? NS : -NS) : (sx ? nbo[RING ? 0 : 1] : nbo[0]) * NS;
+                const int o_y = RING ? (SLOTS + l) * NS : (sy ? nbo[RING ? 0 : 3] : nbo[RING ? 0 : 2]) * NS;
+                const int o_z = RING ? (SLOTS + EB + l) * NS : (sz ? nbo[RING ? 0 : 5] : nbo[RING ? 0 : 4]) * NS;
                 const float *fnb = RING ? st + (SLOTS + 2 * EB + l) * NS : a.f_n + (size_t)k * slab + (size_t)el * NS;
                 // upwind operand of each direction: the neighbour, or at a specular
                 // face the element itself at the mirrored velocity, with the weights
@@ -539,7 +554,8 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                             }
                         }
                         float2 dn[NPT];
-                        if (!BC || !((dirichlet >> sx) & 1)) {
+                        const bool ext = BC && ((dirichlet >> sx) & 1);
+                        if (!RING || !ext) {
                             float2 NB[Q];
                             if constexpr (RING) ld2(o_x + ln, Q, NB);
                             else
@@ -553,9 +569,9 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
 #pragma unroll
                                 for (int i = 0; i < NPT; ++i)
                                     dn[i] = __ffma2_rn(dup2(Lr[j]), sub2(NB[j], F2[i]), dn[i]);
-                        } else {
-                            const float2 bv = make_float2((float)__ldg(a.bcval + ((size_t)(0 + sx) * C + 0) * a.Nu + k),
-                                                          (float)__ldg(a.bcval + ((size_t)(0 + sx) * C + 1) * a.Nu + k));
+                        }
+                        if (SEL || ext) {
+                            const float2 bv = make_float2(exterior(ext, sx, 0, k), exterior(ext, sx, 1, k));
 #pragma unroll
                             for (int i = 0; i < NPT; ++i) dn[i] = sub2(bv, F2[i]);
                         }
@@ -587,7 +603,8 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
 #pragma unroll
                             for (int i = 0; i < NPT; ++i) t[i] = __ffma2_rn(dup2(Dr[m]), sub2(Gv[i], F2[i]), t[i]);
                         }
-                        if (!BC || !((dirichlet >> (2 * dd + sd)) & 1)) {
+                        const bool ext = BC && ((dirichlet >> (2 * dd + sd)) & 1);
+                        if (!RING || !ext) {
                             float Lr[Q];
                             ld_vec<Q>(&slam[dd == 1 ? wy : wz][0], Lr);
 #pragma unroll
@@ -604,9 +621,9 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
 #pragma unroll
                                 for (int i = 0; i < NPT; ++i) dn[i] = __ffma2_rn(dup2(Lr[jq]), sub2(H[i], F2[i]), dn[i]);
                             }
-                        } else {
-                            const float2 bv = make_float2((float)__ldg(a.bcval + ((size_t)(2 * dd + sd) * C + 0) * a.Nu + k),
-                                                          (float)__ldg(a.bcval + ((size_t)(2 * dd + sd) * C + 1) * a.Nu + k));
+                        }
+                        if (SEL || ext) {
+                            const float2 bv = make_float2(exterior(ext, 2 * dd + sd, 0, k), exterior(ext, 2 * dd + sd, 1, k));
 #pragma unroll
                             for (int i = 0; i < NPT; ++i) dn[i] = sub2(bv, F2[i]);
                         }
@@ -689,7 +706,8 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                             }
                         }
                         float dn[NPT];
-                        if (!BC || !((dirichlet >> sx) & 1)) {
+                        const bool ext = BC && ((dirichlet >> sx) & 1);
+                        if (!RING || !ext) {
                             float NB[Q];
                             ld_vec<Q>(px + c * cstr + ln, NB);
                             float Lr[Q];
@@ -702,10 +720,11 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                                 for (int i = 0; i < NPT; ++i) NBj[i] = NB[j];
                                 acc_dev<NPT>(dn, Lr[j], NBj, Fi);
                             }
-                        } else {
-                            const float bv = (float)__ldg(a.bcval + ((size_t)(0 + sx) * C + c) * a.Nu + k);
+                        }
+                        if (SEL || ext) {
+                            const float bv = exterior(ext, sx, c, k);
 #pragma unroll
-                            for (int i = 0; i < NPT; ++i) dn[i] = bv - Fi[i];
+                            for (int i = 0; i < NPT; ++i) dn[i] = ext ? bv - Fi[i] : dn[i];
                         }
                         float Gr[NPT], Er[NPT];
                         ld_vec<NPT>(&sdg[sx][i0], Gr);
@@ -727,7 +746,8 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                             ld_vec<NPT>(sc + o_own + Q * (jp + Q * kz) + i0, Gv);
                             acc_dev<NPT>(t, Dr[m], Gv, Fi);
                         }
-                        if (!BC || !((dirichlet >> (2 + sy)) & 1)) {
+                        const bool ext = BC && ((dirichlet >> (2 + sy)) & 1);
+                        if (!RING || !ext) {
                             float Lr[Q];
                             ld_vec<Q>(&slam[wy][0], Lr);
                             scale_vec<NPT>(dn, RING ? cf.x : sdlam[wy], Fi);
@@ -737,10 +757,11 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                                 ld_vec<NPT>(py + c * cstr + Q * (jp + Q * kz) + i0, H);
                                 acc_dev<NPT>(dn, Lr[jp], H, Fi);
                             }
-                        } else {
-                            const float bv = (float)__ldg(a.bcval + ((size_t)(2 + sy) * C + c) * a.Nu + k);
+                        }
+                        if (SEL || ext) {
+                            const float bv = exterior(ext, 2 + sy, c, k);
 #pragma unroll
-                            for (int i = 0; i < NPT; ++i) dn[i] = bv - Fi[i];
+                            for (int i = 0; i < NPT; ++i) dn[i] = ext ? bv - Fi[i] : dn[i];
                         }
                         float dgv[NPT], epv[NPT];
 #pragma unroll
@@ -762,7 +783,8 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                             ld_vec<NPT>(sc + o_own + Q * (jy + Q * kp) + i0, Gv);
                             acc_dev<NPT>(t, Dr[m], Gv, Fi);
                         }
-                        if (!BC || !((dirichlet >> (4 + sz)) & 1)) {
+                        const bool ext = BC && ((dirichlet >> (4 + sz)) & 1);
+                        if (!RING || !ext) {
                             float Lr[Q];
                             ld_vec<Q>(&slam[wz][0], Lr);
                             scale_vec<NPT>(dn, RING ? cf.x : sdlam[wz], Fi);
@@ -772,10 +794,11 @@ __global__ void __launch_bounds__(LineGeom<Q, C, EB, NPT>::NTHR, LineGeom<Q, C, 
                                 ld_vec<NPT>(pz + c * cstr + Q * (jy + Q * kp) + i0, H);
                                 acc_dev<NPT>(dn, Lr[kp], H, Fi);
                             }
-                        } else {
-                            const float bv = (float)__ldg(a.bcval + ((size_t)(4 + sz) * C + c) * a.Nu + k);
+                        }
+                        if (SEL || ext) {
+                            const float bv = exterior(ext, 4 + sz, c, k);
 #pragma unroll
-                            for (int i = 0; i < NPT; ++i) dn[i] = bv - Fi[i];
+                            for (int i = 0; i < NPT; ++i) dn[i] = ext ? bv - Fi[i] : dn[i];
                         }
                         float dgv[NPT], epv[NPT];
 #pragma unroll
