@@ -41,7 +41,10 @@ constexpr double kTwoPi = 6.283185307179586476925286766559;
 // The register bound of the box forms: one block per multiprocessor asked for
 // (150 to 196 registers, nothing spilled) is faster up to p = 2 and at p = 3 with
 // F and G (p = 2: 1.44 against 1.65 ms), the compiler's own choice (127, 128)
-// at p = 3 (2.66 against 3.00) and p = 4 (5.70 against 6.43).
+// at p = 3 (2.66 against 3.00) and p = 4 (5.70 against 6.43).  At p = 1 there is a
+// form of each (159 and 189 registers, 128 with at most 48 B of spills): one block
+// per multiprocessor takes 0.83 of the time of a block of the other form on its
+// own, two at a time take 1.65, so the launch counts the waves of both (stage_p1).
 //
 // Curvilinear elements (CURV): the transformed flux Ft_d = a_d f with
 // a_d = u . S^d at each node (S^d = J grad xi_d), per direction and line
@@ -53,8 +56,8 @@ constexpr double kTwoPi = 6.283185307179586476925286766559;
 // not A times the trace of f).  The element's own flux values are staged in
 // shared memory beside f.  Boundary faces: Dirichlet (prescribed exterior
 // Maxwellian), diffuse wall (rho_w times the wall Maxwellian), closed (no flux).
-template <int Q, int C, bool CURV>
-__global__ void __launch_bounds__(256, !CURV && (Q <= 3 || (Q == 4 && C == 2)) ? 1 : 0) k_stage_f64(StageArgs<double> a) {
+template <int Q, int C, bool CURV, int MINB>
+__global__ void __launch_bounds__(256, MINB) k_stage_f64(StageArgs<double> a) {
     constexpr int NS = Q * Q * Q;
     constexpr int EB = 256 / NS;
     constexpr int NT = EB * NS;
@@ -359,16 +362,33 @@ __global__ void k_maxwellian_f64(double *f, const double *qin, const double *vta
 
 }  // namespace
 
+// p = 1 boxes, in units of a block that has a multiprocessor to itself in the form
+// of one block each: a wave of that form takes 1, a wave of the form of two 1.65,
+// its last one 1.2 where it is half empty.  Both forms round alike.  24^3 velocities,
+// us per stage, one / two per multiprocessor: 12 elements, F and G 599 / 719; 120:
+// 2465 / 2116; 200: 3769 / 3863; one component, 384 elements 4494 / 3729.
+template <int C>
+static cudaError_t stage_p1(const StageArgs<double> &a, dim3 grid, cudaStream_t s) {
+    const long long n = (long long)grid.x * grid.y, sms = multiprocessors(), rest = n % (2 * sms);
+    const double one = (double)((n + sms - 1) / sms);
+    const double two = 1.65 * (double)(n / (2 * sms)) + (rest == 0 ? 0.0 : rest <= sms ? 1.2 : 1.65);
+    if (two < 0.97 * one) k_stage_f64<2, C, false, 2><<<grid, 256, 0, s>>>(a);
+    else k_stage_f64<2, C, false, 1><<<grid, 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 template <int Q>
 static cudaError_t stage_q(const StageArgs<double> &a, int C, int n_vblk, cudaStream_t s) {
     constexpr int NS = Q * Q * Q, EB = 256 / NS;
     dim3 grid((a.mesh.Ne + EB - 1) / EB, n_vblk);
     if (a.geo) {
-        if (C == 1) k_stage_f64<Q, 1, true><<<grid, EB * NS, 0, s>>>(a);
-        else k_stage_f64<Q, 2, true><<<grid, EB * NS, 0, s>>>(a);
+        if (C == 1) k_stage_f64<Q, 1, true, 0><<<grid, EB * NS, 0, s>>>(a);
+        else k_stage_f64<Q, 2, true, 0><<<grid, EB * NS, 0, s>>>(a);
+    } else if constexpr (Q == 2) {
+        return C == 1 ? stage_p1<1>(a, grid, s) : stage_p1<2>(a, grid, s);
     } else {
-        if (C == 1) k_stage_f64<Q, 1, false><<<grid, EB * NS, 0, s>>>(a);
-        else k_stage_f64<Q, 2, false><<<grid, EB * NS, 0, s>>>(a);
+        if (C == 1) k_stage_f64<Q, 1, false, Q == 3><<<grid, EB * NS, 0, s>>>(a);
+        else k_stage_f64<Q, 2, false, Q <= 4><<<grid, EB * NS, 0, s>>>(a);
     }
     return cudaGetLastError();
 }
