@@ -1497,13 +1497,15 @@ static cudaError_t qprime_launch(const QPrimeArgs &a, cudaStream_t s) {
 // two blocks per multiprocessor cost least, a block of QB points costing its QB
 // passes and about six passes' worth of algebra.  512 points, 8^3 velocities:
 // 0.211 ms with 32, 0.109 ms with 8; 6912 points, 40^3: 2.31 ms with 32 (216
-// blocks on 304 places), 1.80 with 24; 13,824 points, 32^3: 1.79 and 1.53.
+// blocks on 304 places), 1.80 with 24; 13,824 points, 32^3: 1.79 and 1.53.  A
+// smaller batch has to cost less by a twentieth: the estimate is no better than
+// that (22,500 points: 110 with 16 against 114, but 0.86 ms against 0.81).
 static int qprime_batch(int P, int sms) {
     int best = 32;
     long long cost = -1;
     for (int qb = 32; qb >= 8; qb -= 8) {
         const long long blocks = (P + qb - 1) / qb, waves = (blocks + 2 * sms - 1) / (2 * sms);
-        if (cost < 0 || waves * (qb + 6) < cost) {
+        if (cost < 0 || 20 * waves * (qb + 6) < 19 * cost) {
             cost = waves * (qb + 6);
             best = qb;
         }
