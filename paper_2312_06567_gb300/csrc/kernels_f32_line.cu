@@ -259,7 +259,7 @@ __device__ __forceinline__ void add_pair(LineAcc<C> &A, LineAcc<C> &B, float cj1
 // runs are not whole 16-byte units (p = 4, p = 2 with odd rows) or short, and
 // those that reflect specularly (the mirrored velocity's trace is not staged).
 // Bit-identical too.  Against the plain kernel: p = 4, 588 for 1399 us per stage
-// (7500 points, 4608 velocities); specular p = 2, 829 for 1987 us (5670 points,
+// (7500 points, 4608 velocities); specular p = 2, 636 for 1987 us (5670 points,
 // 10,560 velocities).  A reflecting face is no case of its own there: its upwind
 // operand is the element itself at the mirrored velocity, so the threads of a
 // warp differ in an address and a row of weights, not in a branch (1107 us with

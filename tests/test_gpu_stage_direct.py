@@ -98,3 +98,22 @@ def test_line_kernel_by_default_equals_plain(lib, p, mesh_n, delta, faces):
             out.append((r, s.get_state(), s.moments()))
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("faces", ["periodic", "dirichlet", "specular"])
+def test_state_beyond_the_cache_at_p1_equals_plain(lib, faces):
+    """One wave of the asynchronous kernel's blocks on a state of 49 MB, which that
+    kernel runs by default (specular faces excepted)."""
+    wl = _wl(1, (32, 1, 1), 2.0, faces).replace(vel_n=(33, 28, 26))
+    x = W.node_positions(wl).reshape(-1, 3)
+    q = np.stack([1 + 0.1 * np.sin(x[:, 0]), 0.1 * np.cos(x[:, 1]), 0.1 * np.sin(x[:, 2]), 0 * x[:, 0], 1 + 0.05 * np.cos(x[:, 0])], 1)
+    out = []
+    for kernel in ("plain", "auto"):
+        with lib.Solver(wl, lib.BGK_MIXED) as s:
+            s.set_stage_kernel(kernel)
+            s.set_maxwellian(q)
+            assert s.step(wl.dt(), 2) == lib.BGK_OK
+            out.append((s.get_state(), s.moments()))
+    assert out[0][0].nbytes > 30e6
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
